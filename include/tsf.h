@@ -120,16 +120,16 @@ typedef struct {
   int64_t assign_rounds;      /* auction rounds of the last assignment (0 when exact) */
   int64_t assign_phases;      /* ... its eps phases */
   int64_t assign_checks;      /* ... its passes releasing rows off eps-complementary slackness */
-  int64_t d1_reduce_rounds;   /* rounds of the saddle-saddle column reduction */
-  int64_t d1_reduce_merged;   /* entries written by its column additions */
-  int64_t d1_reduce_longest;  /* longest column an addition produced */
-  int64_t d1_reduce_big_rounds; /* its rounds with at least 4096 active columns */
+  int64_t d1_reduce_rounds;   /* whole-GPU rounds of the saddle-saddle column reduction (large diagrams) */
+  int64_t d1_reduce_merged;   /* entries written or flipped by its column additions */
+  int64_t d1_reduce_longest;  /* longest column it handled */
+  int64_t d1_reduce_big_rounds; /* the same as d1_reduce_rounds */
   int64_t d1_reduce_big_cycles; /* SM clock cycles spent in those rounds */
   int64_t d1_reduce_cycles;     /* SM clock cycles of the whole reduction */
-  int64_t d1_chain_adds;        /* additions chained in its short rounds (at most 64 active columns) */
-  int64_t d1_chain_longest;     /* ... by one column in one round, at most */
-  int64_t d1_chain_rounds;      /* its short rounds */
-  int64_t d1_chain_cycles;      /* SM clock cycles spent in those rounds */
+  int64_t d1_chain_adds;        /* additions outside the whole-GPU rounds (one warp or block per column) */
+  int64_t d1_chain_longest;     /* ... by one column between two claims of a low, at most */
+  int64_t d1_chain_rounds;      /* rounds of the columns that a block reduced */
+  int64_t d1_chain_cycles;      /* SM clock cycles of the longest-running such block */
 } tsf_stats;
 
 /* Creates a field from lx*ly*lz values (host or device memory, copied),
@@ -297,9 +297,9 @@ int64_t tsf_kernel_launches(void);
  *   4: polls a block waits at a grid barrier of the whole-GPU rounds (union-
  *      find and D1 reduction) before it gives up (default 2^24; giving up
  *      makes the call fail with TSF_ETIMEOUT);
- *   5: D1 columns from which the reduction rounds run over the whole GPU
- *      (default 65536);
- *   6: active D1 columns below which one block finishes them (default 4096);
+ *   5: critical triangles from which the D1 reduction starts with rounds
+ *      over the whole GPU (default 262144);
+ *   6: active D1 columns below which they go on on warps (default 131072);
  *   7: schedule of the D1 Morse boundaries' first phase: 0 the default
  *      (half a warp per column, registers capped for 32 warps per SM; 64 +
  *      128 frontier and stage entries for diagrams of at least 2^19
@@ -311,19 +311,18 @@ int64_t tsf_kernel_launches(void);
  *      phase);
  *   8: register budget of the lower-star gradient kernels, as blocks of
  *      128 threads per SM: 0 the default (6), 1 no cap, 2 five;
- *   9: entries of a column that the D1 reduction's short rounds (at most 64
- *      active columns) keep in shared memory while they chain additions,
- *      with one warp per column (default and maximum 512; the larger groups
- *      of the last columns scale it with their size; longer sums, or all
- *      with 0, are added in the column pool);
+ *   9: entries of a column that a warp of the D1 reduction keeps in shared
+ *      memory (at most 256; a longer column goes to a block);
  *  10: lower-star visits a thread of the D1 Morse boundaries chains in one
  *      round along updates with a single target star (0: the default, 1
  *      for diagrams of at least 2^19 critical triangles, else 2; at most 8);
  *  11: rounds of the D1 Morse boundaries' first phase before a column
  *      moves to a block of the second (0: the default, 128 for diagrams of
  *      at least 2^19 critical triangles, else 16);
- *  12: active columns up to which a round of the D1 reduction chains
- *      additions in shared memory (0: the default, 64; at most 1024).
+ *  12: additions a D1 column makes on a warp before it goes to a block (0:
+ *      the default, 24);
+ *  13: groups of 1024 rows that such a block keeps in shared memory (0: all
+ *      that fit; the rest in global memory).
  * Returns the previous value, or -1 for an unknown knob.  Set them only
  * while no call of this library is running. */
 int64_t tsf_debug_set(int what, int64_t value);

@@ -88,6 +88,7 @@ struct tsf_field {
   D1Work W{};
   int cap_cols = 0;
   uint32_t pool_cap = 0;
+  size_t cap_hbits = 0;
   // solver
   SolverBufs B{};
   int cap_pts = 0, cap_t = 0, cap_idx = 0, cap_idxcd = 0;
@@ -177,7 +178,7 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
     dev_free(F->PO.d2_max);
     dev_free(F->PO.d1_edge);
     dev_free(F->W.cols);
-    dev_free(F->W.low);
+    dev_free(F->W.heavy);
     dev_free(F->W.hoff);
     dev_free(F->W.hcap);
     dev_free(F->W.hsize);
@@ -194,7 +195,7 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
     ck(dev_alloc(&F->PO.d2_max, c2));
     ck(dev_alloc(&F->PO.d1_edge, c2));
     ck(dev_alloc(&F->W.cols, c2));
-    ck(dev_alloc(&F->W.low, c2));
+    ck(dev_alloc(&F->W.heavy, c2));
     ck(dev_alloc(&F->W.hoff, c2));
     ck(dev_alloc(&F->W.hcap, c2));
     ck(dev_alloc(&F->W.hsize, c2));
@@ -491,6 +492,12 @@ int compute_diagram(tsf_field* F, bool incremental) {
       F->pool_cap = want;
     }
     F->W.pool_cap = F->pool_cap;
+    if (const size_t words = d1_long_words(F->n1); words > F->cap_hbits) {
+      dev_free(F->W.hbits);
+      F->cap_hbits = 0;
+      ck(dev_alloc(&F->W.hbits, words));
+      F->cap_hbits = words;
+    }
     if (!F->W.pool_head) ck(dev_alloc(&F->W.pool_head, 1));
     if (!F->W.flags) ck(dev_alloc(&F->W.flags, 4));
     if (!F->W.stats) ck(dev_alloc(&F->W.stats, kD1Stats));
@@ -769,7 +776,8 @@ int tsf_destroy_field(tsf_field* F) {
   dev_free(F->PO.d2_max);
   dev_free(F->PO.d1_edge);
   dev_free(F->W.cols);
-  dev_free(F->W.low);
+  dev_free(F->W.heavy);
+  dev_free(F->W.hbits);
   dev_free(F->W.hoff);
   dev_free(F->W.hcap);
   dev_free(F->W.hsize);

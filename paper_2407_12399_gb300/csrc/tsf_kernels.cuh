@@ -118,27 +118,31 @@ struct D1Ctl {
   int n[2];         // lengths of the two column lists
   int which;        // list holding the active columns
   int rounds;       // rounds done
-  int pad[10];
+  int next;         // columns that warps have taken
+  int nheavy;       // columns moved to blocks (D1Work::heavy)
+  int next_heavy;   // ... taken by blocks
+  int pad[7];
 };
 
 // Counters of the D1 stages (D1Work::stats): [0] lower stars visited, [1]
 // by the largest column, [2] rounds over all columns, [3] of the longest,
-// [4] target-star updates, [5] reduction rounds, [6] entries merged, [7]
-// longest sum, [8] whole-GPU rounds, [9] their cycles, [10] all cycles of
-// the reduction, [11] chained additions of the short rounds, [12] the
-// longest chain of one column in one round, [13] short rounds, [14] their
-// cycles.
+// [4] target-star updates; of the reduction: [5] and [8] whole-GPU rounds,
+// [6] entries merged, [7] longest column, [9] cycles of the whole-GPU rounds,
+// [10] all its cycles, [11] additions on warps and blocks, [12] most by one
+// column between two claims, [13] rounds of the blocks, [14] cycles of the
+// longest-running block, [15] of the longest-running warp.
 constexpr int kD1Stats = 16;
 
 struct D1Work {
   int32_t* cols;          // candidate triangle index per column
-  unsigned long long* low;  // current low per column (0 = to be recomputed)
   uint32_t* hoff;         // heap offset in the pool
   uint32_t* hcap;         // heap capacity
   uint32_t* hsize;        // heap size
-  int32_t* lowc;          // critical edge index of the low
+  int32_t* lowc;          // list of active columns (whole-GPU reduction rounds)
+  int32_t* heavy;         // columns that a block reduces
+  uint32_t* hbits;        // their bit sets where they exceed shared memory (d1_long_words)
   int32_t* owner;         // per critical edge: smallest column holding it as low
-  uint4* orec;            // ... and that column's {index, pool offset, length} while it owns it
+  uint4* orec;            // ... as {column, pool offset, length, 0}
   unsigned long long* pool;
   uint32_t pool_cap;
   uint32_t* pool_head;
@@ -156,6 +160,8 @@ void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st);
 void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1, int n2, const uint32_t* rank,
                      const uint32_t* order, const float* f, const Rec* rec, const D1Tab* tab, const uint32_t* c1base,
                      D1Work& W, PairOut& P, uint32_t* status, cudaStream_t st);
+// Words of D1Work::hbits that a reduction over n1 rows uses.
+size_t d1_long_words(int n1);
 void launch_d1_reduce(int n1, int n2, D1Work& W, PairOut& P, uint32_t* status, D1Ctl* ctl, cudaStream_t st);
 
 }  // namespace tsf
