@@ -12,23 +12,15 @@
 //
 // Convolution (forward, and the data gradient as a convolution with the
 // flipped, transposed kernel) is an implicit GEMM on the tcgen05 tensor
-// cores: M = 128 output voxels (a run along x, or several short rows), N =
-// output channels, K = 27 taps x input channels.  Per tap, TMA loads the
-// 128 shifted input rows of every input plane straight from the chunk planes
-// (out-of-grid rows arrive as zeros: the convolution's zero padding), which
-// is exactly the no-swizzle K-major operand layout: 8-row x 16-byte core
-// matrices, 128 B apart along M and 2 KiB apart along K.  The weights of a
-// stage come in by one bulk copy, pre-packed in the same layout.  One thread
-// issues the MMAs into a TMEM accumulator; all four warps read it back with
-// tcgen05.ld for the epilogue (bias + ReLU or the ReLU mask of the data
-// gradient, rounding to bf16).
-//
+// cores; k_conv_tc says how.
+
 // Weight gradients, pooling, upsampling, the 1x1 head, the loss and Adam are
 // bandwidth-bound and run on the CUDA cores.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "tsf_unet.cuh"
@@ -73,12 +65,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4,
+// The same for a whole warp that goes on in step: the branch is warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  for (uint32_t it = 0; it < (1u << 22); ++it) {
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    if (it > 64) __nanosleep(32);
+  }
+  return false;
+}
+
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-      "%6}], [%7];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(bar))
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -111,29 +112,39 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
          (static_cast<uint32_t>(m >> 4) << 24);
 }
 
+// Issued by one elected lane; the whole warp calls them, with values that are
+// the same in every lane, so that descriptors stay in uniform registers (from
+// one lane of a diverged warp an MMA took about 150 cycles to issue).
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(smem_u32(bar))
+      : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -155,162 +166,339 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
                     pack_bf16x2(v[6], v[7]));
 }
 
+// q to two adjacent 16-byte rows, as one 32-byte store (p is 32-byte aligned).
+__device__ __forceinline__ void store_twice(uint4* p, const uint4& q) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %1, %2, %3, %4};" ::"l"(p), "r"(q.x), "r"(q.y), "r"(q.z),
+               "r"(q.w)
+               : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Convolution as an implicit GEMM on tcgen05
 // ---------------------------------------------------------------------------
-// Shared memory per CTA: kStages x (A stage | B stage), then the barriers.
-// A stage holds taps_per_stage x chunks K-chunks of 128 rows x 16 B; a B
-// stage the same K-chunks of cout rows x 16 B.
-__global__ void __launch_bounds__(128) k_conv_tc(const __grid_constant__ CUtensorMap in_map, ConvArgs a) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t a_bytes = static_cast<uint32_t>(a.kchunks) * 2048u;
-  const uint32_t b_bytes = static_cast<uint32_t>(a.kchunks) * static_cast<uint32_t>(a.cout) * 16u;
-  const uint32_t stage_bytes = a_bytes + b_bytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kConvStages * stage_bytes);
-  uint64_t* empty = full + kConvStages;
-  uint64_t* done = empty + kConvStages;
-  uint32_t* s_taddr = reinterpret_cast<uint32_t*>(done + 1);
-  int* s_abort = reinterpret_cast<int*>(s_taddr + 1);
+// A block computes tx x ty x tz output voxels.  For each pair of input planes
+// (16 channels, one K step) it walks the tz + 2 input z-planes; TMA brings a
+// plane's (ty + 2) x (tx + 2) voxels (zero outside the grid: the padding) as
+// 16-byte rows, one after the other.  In the no-swizzle K-major operand layout
+// 128 consecutive rows are an A tile, so a tile of 128 outputs (flattened with
+// pitch tx + 2; the two halo columns of a row give outputs that nobody keeps)
+// reads its (dy, dx) neighbours by a shift of the operand's start address: one
+// load serves nine taps.  The three dz taps of an input plane go to three
+// output planes, whose accumulators lie next to each other in TMEM, so the
+// three weight matrices form one B operand of 3 x cout columns and one MMA
+// does all three.
+// A block per SM walks over tiles: one warp issues the loads (they run ahead
+// into the next tile), two the MMAs (half of a tile's operand tiles each),
+// eight turn accumulators into outputs
+// while the other half of TMEM (256 columns) takes the next tile's MMAs.
+// Weights that fit stay in shared memory for the whole launch.
+// Bound: the A operand.  An MMA reads 4 KB of A (32 cycles of shared-memory
+// bandwidth) and 96 x cout bytes of B, 32 + 3 x cout / 4 cycles in all, for
+// 3 x cout / 2 cycles of math, so 16 output channels reach about half of the
+// tensor rate.
+// A single input plane (8 channels) takes two dx neighbours as its K step:
+// the second K half is the first one shifted by one row.
+constexpr int kConvEpiWarps = 8;
+constexpr int kConvMmaWarps = 2;
+constexpr int kConvThreads = (kConvEpiWarps + 1 + kConvMmaWarps) * 32;
 
-  // tile of 128 rows: bx voxels along x times by rows along y, at one z
-  const int tiles_x = (a.lx + a.bx - 1) / a.bx, tiles_y = (a.ly + a.by - 1) / a.by;
-  int t = blockIdx.x;
-  const int x0 = (t % tiles_x) * a.bx;
-  t /= tiles_x;
-  const int y0 = (t % tiles_y) * a.by;
-  const int z0 = t / tiles_y;
+struct ConvBars {
+  uint64_t full_a[kConvStagesMax], empty_a[kConvStagesMax], full_b[kConvBSlotsMax], empty_b[kConvBSlotsMax];
+  uint64_t tfull[2], tempty[2], done;
+  uint32_t taddr;
+  int gave_up, issued_a, issued_b;
+  float bias[96], head[17];
+};
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// The MMAs of one input plane: every (dy, dx) tap on kM operand tiles.
+struct PlaneMmas {
+  uint64_t a, b;         // operand descriptors of the first tile and tap
+  uint32_t t0, tcols;    // accumulators of d = 0 and the distance of two tiles'
+  uint32_t cout, pitch;
+  int dlo, dhi;          // dz taps that stay in the tile
+  bool first;            // first K step: output plane d = 2 starts its sums here
+};
+
+// dz taps d .. d + n - 1 of one (dy, dx) tap.
+template <int kM>
+__device__ __forceinline__ void issue_tap(const PlaneMmas& f, uint64_t ad, uint64_t bd, int d, int n, uint32_t acc) {
+  const uint32_t idesc = instr_desc(128, n * static_cast<int>(f.cout));
+  bd += static_cast<uint32_t>(d) * f.cout;
+  const uint32_t td = f.t0 + static_cast<uint32_t>(d) * f.cout;
+#pragma unroll
+  for (int m = 0; m < kM; ++m) mma_bf16(td + m * f.tcols, ad + m * 128u, bd, idesc, acc);
+}
+
+// Unrolled: an MMA of 48 columns takes 44 cycles, and the loop has to issue
+// one in as many.  256^3 voxels, 16 to 16 channels: rolled over taps and tiles
+// 1046 us, over tiles only 645, unrolled 437 (66 cycles per MMA: about 72 per
+// tap and 49 per tile); two warps that share the tiles take the whole layer
+// from 479 to 403 us.
+template <bool kSingle, int kM>
+__device__ __forceinline__ void issue_plane(const PlaneMmas& f) {
+  constexpr int kDx = kSingle ? 2 : 3;
+  const int n = f.dhi - f.dlo + 1;
+  const bool upper = f.dhi == 2 && f.dlo < 2;                       // d = 2 next to others
+  const bool wide = upper && n * static_cast<int>(f.cout) > 256;  // N <= 256
+  const bool split = wide || (f.first && upper);
+  issue_tap<kM>(f, f.a, f.b, f.dlo, split ? 2 - f.dlo : n, f.first && f.dlo == 2 ? 0u : 1u);
+  if (split) issue_tap<kM>(f, f.a, f.b, 2, 1, f.first ? 0u : 1u);
+  if (!wide) {
+#pragma unroll
+    for (int t = 1; t < 3 * kDx; ++t)
+      issue_tap<kM>(f, f.a + static_cast<uint32_t>(t / kDx) * f.pitch + t % kDx,
+                    f.b + static_cast<uint32_t>(t) * (6u * f.cout), f.dlo, n, 1u);
+  } else {
+#pragma unroll 1
+    for (int t = 1; t < 3 * kDx; ++t) {
+      const uint64_t ad = f.a + static_cast<uint32_t>(t / kDx) * f.pitch + t % kDx;
+      const uint64_t bd = f.b + static_cast<uint32_t>(t) * (6u * f.cout);
+      issue_tap<kM>(f, ad, bd, f.dlo, 2 - f.dlo, 1u);
+      issue_tap<kM>(f, ad, bd, 2, 1, 1u);
+    }
+  }
+}
+
+template <bool kSingle>
+__global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_constant__ CUtensorMap in_map, ConvArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ ConvBars sh;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const ConvPlan& p = a.plan;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t* sb0 = smem + p.stages * p.a_bytes;
+  volatile int* gave_up = &sh.gave_up;
+  const int tiles = p.tiles_x * p.tiles_y * p.tiles_z;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kConvStages; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&sh.full_a[s], 1);
+      mbar_init(&sh.empty_a[s], kConvMmaWarps);
     }
-    mbar_init(done, 1);
-    s_abort[0] = 0;
-    s_abort[2] = 0;
+    for (int s = 0; s < p.b_slots; ++s) {
+      mbar_init(&sh.full_b[s], 1);
+      mbar_init(&sh.empty_b[s], kConvMmaWarps);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&sh.tfull[s], kConvMmaWarps);
+      mbar_init(&sh.tempty[s], kConvEpiWarps);
+    }
+    mbar_init(&sh.done, kConvMmaWarps);
+    sh.gave_up = 0;
+    sh.issued_a = 0;
+    sh.issued_b = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (a.mode != kConvDgrad && threadIdx.x < a.cout) sh.bias[threadIdx.x] = a.bias[threadIdx.x];
+  if (a.mode == kConvHead && threadIdx.x < 17) sh.head[threadIdx.x] = a.head[threadIdx.x];
   __syncwarp();
-  if (warp == 0) {  // TMEM accumulator: a.tmem_cols fp32 columns x 128 lanes
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_taddr)),
-                 "r"(static_cast<uint32_t>(a.tmem_cols))
+  if (warp == 0) {  // TMEM accumulators: two halves of p.tmem_cols / 2 fp32 columns x 128 lanes
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.taddr)),
+                 "r"(static_cast<uint32_t>(p.tmem_cols))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t taddr = *s_taddr;
-  const int nst = a.nstages;
+  const uint32_t taddr = __shfl_sync(0xFFFFFFFFu, sh.taddr, 0);
+  const int role = __shfl_sync(0xFFFFFFFFu, warp, 0);  // the same value, known to be warp-uniform
+  const uint32_t thalf = static_cast<uint32_t>(p.tmem_cols / 2);
 
-  if (warp == 0 && lane == 0) {
-    // producer: per stage, the shifted input rows of its taps and its weights
-    for (int s = 0; s < nst; ++s) {
-      const int slot = s % kConvStages;
-      if (s >= kConvStages) {
-        if (!mbar_wait(&empty[slot], ((s / kConvStages) - 1) & 1)) {
-          atomicOr(a.status, kUnetErrSpin);
-          *reinterpret_cast<volatile int*>(s_abort) = 1;
-          break;
+  if (role == kConvEpiWarps && lane == 0) {
+    // producer: per tile and K step the weights (once, if all stay resident),
+    // then the input planes
+    int it = 0, bt = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+      const int x0 = (tile % p.tiles_x) * p.tx, y0 = ((tile / p.tiles_x) % p.tiles_y) * p.ty,
+                z0 = tile / (p.tiles_x * p.tiles_y) * p.tz;
+      for (int kk = 0; kk < p.ksteps && ok; ++kk) {
+        if (!p.b_resident || bt < p.ksteps) {
+          const int bs = bt % p.b_slots;
+          if (bt >= p.b_slots && !mbar_wait(&sh.empty_b[bs], ((bt / p.b_slots) - 1) & 1)) ok = false;
+          if (!ok || *gave_up) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&sh.full_b[bs], p.b_bytes);
+          bulk_load(sb0 + bs * p.b_bytes, a.wpack + static_cast<size_t>(kk) * (p.b_bytes / 2), p.b_bytes,
+                    &sh.full_b[bs]);
+          sh.issued_b = ++bt;
+        }
+        for (int zi = 0; zi < p.tz + 2; ++zi, ++it) {
+          const int slot = it % p.stages;
+          if (it >= p.stages && !mbar_wait(&sh.empty_a[slot], ((it / p.stages) - 1) & 1)) ok = false;
+          if (!ok || *gave_up) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&sh.full_a[slot], p.a_tx);
+          tma_load_4d(smem + slot * p.a_bytes, &in_map, 2 * (x0 - 1), y0 - 1, z0 - 1 + zi, kk * p.kchunks,
+                      &sh.full_a[slot]);
+          sh.issued_a = it + 1;
         }
       }
-      if (*reinterpret_cast<volatile int*>(s_abort)) break;
-      uint8_t* sa = smem + slot * stage_bytes;
-      mbar_expect_tx(&full[slot], stage_bytes);
-      for (int q = 0; q < a.taps_per_stage; ++q) {
-        const int tap = min(s * a.taps_per_stage + q, 26);  // a padding tap repeats tap 26 with zero weights
-        const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-        tma_load_5d(sa + q * a.chunks * 2048, &in_map, 0, x0 + dx - 1, y0 + dy - 1, z0 + dz - 1, 0, &full[slot]);
-      }
-      bulk_load(sa + a_bytes, a.wpack + static_cast<size_t>(s) * (b_bytes / 2), b_bytes, &full[slot]);
-      s_abort[2] = s + 1;  // stages issued
     }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer: K16 steps over the stage's K-chunks
-    const uint32_t idesc = instr_desc(128, a.cout);
-    for (int s = 0; s < nst; ++s) {
-      const int slot = s % kConvStages;
-      if (!mbar_wait(&full[slot], (s / kConvStages) & 1)) {
-        atomicOr(a.status, kUnetErrSpin);
-        *reinterpret_cast<volatile int*>(s_abort) = 1;
+    if (!ok) {
+      if (!*gave_up) atomicOr(a.status, kUnetErrSpin);
+      *gave_up = 1;
+    }
+  } else if (role > kConvEpiWarps) {
+    // MMA issuers: descriptors are built once per plane and advanced by adds to
+    // their address fields (in units of 16 bytes)
+    const int m0 = role == kConvEpiWarps + 1 ? 0 : (p.mtiles + 1) / 2;
+    const int nm = role == kConvEpiWarps + 1 ? (p.mtiles + 1) / 2 : p.mtiles / 2;
+    const uint32_t a_lbo = kSingle ? 16u : static_cast<uint32_t>((p.ty + 2) * p.pitch) * 16u;
+    const uint32_t b_lbo = static_cast<uint32_t>(3 * a.cout) * 16u;
+    const uint32_t tcols = static_cast<uint32_t>(p.tz * a.cout), cout = static_cast<uint32_t>(a.cout);
+    int it = 0, bt = 0, nt = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++nt) {
+      const int half = nt & 1;
+      if (nt >= 2 && !mbar_wait_warp(&sh.tempty[half], ((nt >> 1) - 1) & 1)) {
+        ok = false;
         break;
       }
-      if (*reinterpret_cast<volatile int*>(s_abort)) break;
       tc_fence_after();
-      const uint32_t sa = smem_u32(smem + slot * stage_bytes);
-      const uint32_t sb = sa + a_bytes;
-      for (int k = 0; k < a.kchunks / 2; ++k) {
-        const uint64_t ad = smem_desc(sa + k * 4096u, 2048u, 128u);
-        const uint64_t bd = smem_desc(sb + k * 2u * a.cout * 16u, a.cout * 16u, 128u);
-        mma_bf16(taddr, ad, bd, idesc, (s > 0 || k > 0) ? 1u : 0u);
+      for (int kk = 0; kk < p.ksteps && ok; ++kk, ++bt) {
+        const int bs = bt % p.b_slots;
+        if ((!p.b_resident || nt == 0) &&
+            !mbar_wait_warp(&sh.full_b[bs], p.b_resident ? 0 : (bt / p.b_slots) & 1)) {
+          ok = false;
+          break;
+        }
+        const uint64_t bbase = smem_desc(smem_u32(sb0 + bs * p.b_bytes), b_lbo, 128u);
+        for (int zi = 0; zi < p.tz + 2; ++zi, ++it) {
+          const int slot = it % p.stages;
+          if (!mbar_wait_warp(&sh.full_a[slot], (it / p.stages) & 1) || __any_sync(0xFFFFFFFFu, *gave_up)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          // input plane zi feeds output planes zi - 2 + d (dz tap 2 - d)
+          const int dlo = max(0, 2 - zi), dhi = min(2, p.tz + 1 - zi);
+          const uint64_t abase = smem_desc(smem_u32(smem + slot * p.a_bytes), a_lbo, 128u);
+          const PlaneMmas f{abase + static_cast<uint32_t>(m0) * 128u, bbase,
+                            taddr + (half ? thalf : 0u) + static_cast<uint32_t>(m0) * tcols +
+                                static_cast<uint32_t>((zi - 2) * a.cout),
+                            tcols, cout, static_cast<uint32_t>(p.pitch), dlo, dhi, kk == 0};
+          if (nm == 1) issue_plane<kSingle, 1>(f);
+          else if (nm == 2) issue_plane<kSingle, 2>(f);
+          mma_commit(&sh.empty_a[slot]);  // the slot is free once these MMAs have read it
+        }
+        if (ok && !p.b_resident) mma_commit(&sh.empty_b[bs]);
       }
-      mma_commit(&empty[slot]);  // the slot is free once these MMAs have read it
+      if (ok) mma_commit(&sh.tfull[half]);
     }
-    mma_commit(done);  // arrives when every MMA issued above has completed
-  }
-  __syncwarp();
-
-  // epilogue: one thread waits for the accumulator, then every row m = this
-  // thread's TMEM lane
-  if (threadIdx.x == 64) {
-    bool ok = mbar_wait(done, 0);
-    if (!ok) atomicOr(a.status, kUnetErrSpin);
-    if (*reinterpret_cast<volatile int*>(s_abort)) ok = false;
-    s_abort[1] = ok ? 1 : 0;
+    if (!ok && lane == 0) {
+      if (!*gave_up) atomicOr(a.status, kUnetErrSpin);
+      *gave_up = 1;
+    }
+    __syncwarp();
+    mma_commit(&sh.done);  // every MMA issued above is complete before TMEM is freed
+    mbar_wait(&sh.done, 0);
+  } else if (role < kConvEpiWarps) {
+    // epilogue: warp w reads TMEM lanes 32 * (w % 4) ..; the two warps of a
+    // lane quarter take every other output row of the tile
+    const size_t nv = static_cast<size_t>(a.lx) * a.ly * a.lz;
+    const uint32_t tlane = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    int nt = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++nt) {
+      const int x0 = (tile % p.tiles_x) * p.tx, y0 = ((tile / p.tiles_x) % p.tiles_y) * p.ty,
+                z0 = tile / (p.tiles_x * p.tiles_y) * p.tz;
+      const int half = nt & 1;
+      const bool ready = mbar_wait(&sh.tfull[half], (nt >> 1) & 1);
+      if (__any_sync(0xFFFFFFFFu, !ready || *gave_up)) {
+        if (lane == 0) {
+          if (!*gave_up) atomicOr(a.status, kUnetErrSpin);
+          *gave_up = 1;
+        }
+        break;
+      }
+      tc_fence_after();
+      const uint32_t tbase = taddr + (half ? thalf : 0u) + tlane;
+      int turn = warp >> 2;
+      for (int m = 0; m < p.mtiles; ++m) {
+        const int q = m * 128 + (warp & 3) * 32 + lane;  // flattened position in the tile's planes
+        const int yy = q / p.pitch, xx = q - yy * p.pitch;
+        const int x = x0 + xx, y = y0 + yy;
+        const bool in_xy = xx < p.tx && yy < p.ty && x < a.lx && y < a.ly;
+        for (int zo = 0; zo < p.tz; ++zo, turn ^= 1) {
+          const int z = z0 + zo;
+          if (turn || z >= a.lz) continue;
+          const size_t vox = (static_cast<size_t>(z) * a.ly + y) * a.lx + x;
+          const uint32_t tcol = tbase + static_cast<uint32_t>((m * p.tz + zo) * a.cout);
+          float head = 0.0f;
+          for (int c16 = 0; c16 < a.cout / 16; ++c16) {
+            float v[16];
+            __syncwarp();
+            tmem_ld16(tcol + static_cast<uint32_t>(c16 * 16), v);  // warp-wide
+            if (!in_xy) continue;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int c8 = 2 * c16 + h;
+              float* w = v + 8 * h;
+              if (a.mode == kConvDgrad) {  // masked by the ReLU of the activation it flows into
+                if (a.mask) {
+                  float mk[8];
+                  unpack8(reinterpret_cast<const uint4*>(a.mask)[(a.mask_plane0 + c8) * nv + vox], mk);
+#pragma unroll
+                  for (int i = 0; i < 8; ++i) w[i] = mk[i] > 0.0f ? w[i] : 0.0f;
+                }
+                reinterpret_cast<uint4*>(a.out)[(a.out_plane0 + c8) * nv + vox] = pack8(w);
+                continue;
+              }
+#pragma unroll
+              for (int i = 0; i < 8; ++i) w[i] = fmaxf(w[i] + sh.bias[c8 * 8 + i], 0.0f);
+              const uint4 o = pack8(w);
+              if (a.mode == kConvHead) {  // the 1x1 head on the stored (bf16) values
+                float u[8];
+                unpack8(o, u);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) head = fmaf(u[i], sh.head[c8 * 8 + i], head);
+              } else if (a.up) {  // nearest x2 upsampling: the voxel's 2x2x2 block of the fine grid
+                const int fx = a.lx * 2, fy = a.ly * 2;
+                const size_t fnv = nv * 8;
+                uint4* base = reinterpret_cast<uint4*>(a.out) + (a.out_plane0 + c8) * fnv;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)  // two voxels along x per store
+                  store_twice(base + (static_cast<size_t>(2 * z + (k >> 1)) * fy + (2 * y + (k & 1))) * fx + 2 * x, o);
+              } else {
+                reinterpret_cast<uint4*>(a.out)[(a.out_plane0 + c8) * nv + vox] = o;
+              }
+            }
+          }
+          if (a.mode == kConvHead && in_xy) {
+            const float r = __bfloat162float(__float2bfloat16_rn(head + sh.head[16]));
+            a.g0[vox] = a.f[vox] + r;
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.tempty[half]);
+    }
   }
   __syncthreads();
-  const bool ok = s_abort[1] != 0;
-  tc_fence_after();
-  const int m = threadIdx.x;  // 0..127 = 32 * warp + lane
-  const int x = x0 + m % a.bx, y = y0 + m / a.bx, z = z0;
-  const bool inside = ok && x < a.lx && y < a.ly && z < a.lz;
-  const size_t nv = static_cast<size_t>(a.lx) * a.ly * a.lz;
-  const size_t vox = (static_cast<size_t>(z) * a.ly + y) * a.lx + x;
-  for (int c8 = 0; c8 < a.cout / 8; ++c8) {
-    float v[8];
-    __syncwarp();
-    tmem_ld8(taddr + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(c8 * 8), v);  // warp-wide
-    if (!inside) continue;
-    if (a.mode == kConvForward) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i] + a.bias[c8 * 8 + i], 0.0f);
-      const uint4 q = pack8(v);
-      if (a.up) {  // nearest x2 upsampling: the voxel's 2x2x2 block of the fine grid
-        const int fx = a.lx * 2, fy = a.ly * 2;
-        const size_t fnv = nv * 8;
-        uint4* base = reinterpret_cast<uint4*>(a.out) + (a.out_plane0 + c8) * fnv;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const size_t fv = (static_cast<size_t>(2 * z + (k >> 2)) * fy + (2 * y + ((k >> 1) & 1))) * fx + 2 * x + (k & 1);
-          base[fv] = q;
-        }
-      } else {
-        reinterpret_cast<uint4*>(a.out)[(a.out_plane0 + c8) * nv + vox] = q;
-      }
-    } else {  // data gradient, masked by the ReLU of the activation it flows into
-      if (a.mask) {
-        float mk[8];
-        unpack8(reinterpret_cast<const uint4*>(a.mask)[(a.mask_plane0 + c8) * nv + vox], mk);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = mk[i] > 0.0f ? v[i] : 0.0f;
-      }
-      reinterpret_cast<uint4*>(a.out)[(a.out_plane0 + c8) * nv + vox] = pack8(v);
-    }
-  }
-  // after an abort, wait (bounded) for the copies still in flight before the
+  // after giving up, wait (bounded) for the copies still in flight before the
   // shared memory they target is released
-  if (threadIdx.x == 0 && !ok) {
-    for (int s = max(0, s_abort[2] - kConvStages); s < s_abort[2]; ++s)
-      mbar_wait(&full[s % kConvStages], (s / kConvStages) & 1);
+  if (threadIdx.x == 0 && *gave_up) {
+    for (int s = max(0, sh.issued_a - p.stages); s < sh.issued_a; ++s)
+      mbar_wait(&sh.full_a[s % p.stages], (s / p.stages) & 1);
+    for (int s = max(0, sh.issued_b - p.b_slots); s < sh.issued_b; ++s)
+      mbar_wait(&sh.full_b[s % p.b_slots], (s / p.b_slots) & 1);
   }
   tc_fence_before();
   __syncthreads();
-  __syncwarp();
+  tc_fence_after();
   if (warp == 0) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr),
-                 "r"(static_cast<uint32_t>(a.tmem_cols))
+                 "r"(static_cast<uint32_t>(p.tmem_cols))
                  : "memory");
   }
 }
@@ -401,25 +589,6 @@ __global__ void k_skip_back(const uint4* __restrict__ gs, int gs_plane0, const u
 #pragma unroll
   for (int c = 0; c < 8; ++c) a[c] = m[c] > 0.0f ? a[c] + b[c] * 0.125f : 0.0f;
   out[p * fnv + v] = pack8(a);
-}
-
-// Head, forward: g0 = f + bf16(sum_c u1[c] w[c] + b) (two planes of u1);
-// hw holds the 16 weights and then the bias.
-__global__ void k_head_forward(const uint4* __restrict__ u1, const float* __restrict__ hw, int64_t nv,
-                               const float* __restrict__ f, float* __restrict__ g0) {
-  const int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (v >= nv) return;
-  const float hb = hw[16];
-  float a[8], b[8];
-  unpack8(u1[v], a);
-  unpack8(u1[nv + v], b);
-  float r = 0.0f;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) r = fmaf(a[c], hw[c], r);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) r = fmaf(b[c], hw[8 + c], r);
-  r = __bfloat162float(__float2bfloat16_rn(r + hb));
-  g0[v] = f[v] + r;
 }
 
 // Head, backward for the loss mean((g0 - g)^2): per voxel gg = 2 (g0 - g) / nv;
@@ -622,27 +791,31 @@ __global__ void k_bias_reduce(const float* __restrict__ partial, int nblk, int c
 }
 
 // Weights of one layer from the fp32 master copy (reference layout
-// (cout, cin_real, 3, 3, 3)) into the stage-packed bf16 B operand:
-// pack[stage][kchunk][o][8], kchunk over (tap in stage, input chunk).  The
-// data-gradient packing transposes and flips: B[o'][c'][tap] =
-// w[c'][o'][26 - tap] (o' over the forward inputs, c' over its outputs).
-__global__ void k_pack_weights(const float* __restrict__ w, int cout_f, int cin_real, int cin_pad, int taps_per_stage,
-                               int nstages, int transpose, __nv_bfloat16* __restrict__ pack) {
+// (cout, cin_real, 3, 3, 3)) into the bf16 B operand of k_conv_tc:
+// pack[K step][tap][K half][d * n_out + o][8], d = 0..2 for the dz tap 2 - d.
+// Two input planes make a K step of nine (dy, dx) taps; a single one makes a
+// K step of three dy times the dx pairs (0, 1) and (-, 2).  The data-gradient
+// packing transposes and flips: B[o'][c'][tap] = w[c'][o'][26 - tap] (o' over
+// the forward inputs, c' over its outputs).
+__global__ void k_pack_weights(const float* __restrict__ w, int cout_f, int cin_real, int cin_pad, int transpose,
+                               int64_t total, __nv_bfloat16* __restrict__ pack) {
   const int n_out = transpose ? cin_pad : cout_f;   // N of the GEMM
   const int n_in = transpose ? cout_f : cin_pad;    // input channels of the GEMM
-  const int chunks = n_in / 8;
-  const int kchunks = taps_per_stage * chunks;
-  const int64_t total = static_cast<int64_t>(nstages) * kchunks * n_out * 8;
+  const bool single = n_in == 8;
+  const int taps = single ? 6 : 9;
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= total) return;
   const int e = static_cast<int>(i % 8);
-  const int o = static_cast<int>((i / 8) % n_out);
-  const int kc = static_cast<int>((i / (8 * n_out)) % kchunks);
-  const int s = static_cast<int>(i / (static_cast<int64_t>(8) * n_out * kchunks));
-  const int tap = s * taps_per_stage + kc / chunks;
-  const int ci = (kc % chunks) * 8 + e;
+  const int n = static_cast<int>((i / 8) % (3 * n_out));
+  const int half = static_cast<int>((i / (24 * n_out)) % 2);
+  const int t = static_cast<int>((i / (48 * n_out)) % taps);
+  const int kk = static_cast<int>(i / (static_cast<int64_t>(48) * n_out * taps));
+  const int o = n % n_out, dz = 2 - n / n_out;
+  const int dy = single ? t >> 1 : t / 3, dx = single ? (t & 1) + half : t % 3;
+  const int ci = single ? e : (kk * 2 + half) * 8 + e;
+  const int tap = (dz * 3 + dy) * 3 + dx;
   float val = 0.0f;
-  if (tap < 27) {
+  if (!(single && (t & 1) && half == 0)) {  // dx = 1 is in the first pair
     if (!transpose) {
       if (ci < cin_real) val = w[(static_cast<int64_t>(o) * cin_real + ci) * 27 + tap];
     } else {  // GEMM output o = forward input channel, GEMM input ci = forward output channel
@@ -699,7 +872,13 @@ EncodeTiledFn g_encode = nullptr;
 bool g_attr_set[64] = {};
 }  // namespace
 
-int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz, int chunks, int bx, int by) {
+// Planes as (2 * lx, ly, lz, chunks) 8-byte elements, two per voxel, so that a
+// row of voxels is one run of a box's innermost dimension (at most 256
+// elements): TMA takes three to five cycles per innermost run, and with
+// 16-byte runs it, not the tensor cores, set the time.  x coordinates are
+// multiples of two elements, 16 bytes.
+int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz, int chunks, int bx, int by,
+                      int bchunks) {
   if (!g_encode) {
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
@@ -709,57 +888,100 @@ int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
   const uint64_t nv = static_cast<uint64_t>(lx) * ly * lz;
-  cuuint64_t dims[5] = {8, static_cast<cuuint64_t>(lx), static_cast<cuuint64_t>(ly), static_cast<cuuint64_t>(lz),
+  cuuint64_t dims[4] = {2 * static_cast<cuuint64_t>(lx), static_cast<cuuint64_t>(ly), static_cast<cuuint64_t>(lz),
                         static_cast<cuuint64_t>(chunks)};
-  cuuint64_t strides[4] = {16, 16ull * lx, 16ull * lx * ly, 16ull * nv};
-  cuuint32_t box[5] = {8, static_cast<cuuint32_t>(bx), static_cast<cuuint32_t>(by), 1,
-                       static_cast<cuuint32_t>(chunks)};
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es,
+  cuuint64_t strides[3] = {16ull * lx, 16ull * lx * ly, 16ull * nv};
+  cuuint32_t box[4] = {2 * static_cast<cuuint32_t>(bx), static_cast<cuuint32_t>(by), 1,
+                       static_cast<cuuint32_t>(bchunks)};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(base), dims, strides, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
 }
 
-void tile_shape(int lx, int& bx, int& by) {
-  if (lx >= 128 || 128 % lx != 0) {
-    bx = 128;
-    by = 1;
-  } else {
-    bx = lx;
-    by = 128 / lx;
+// Tile of a convolution: the shape of least estimated time, in cycles.  An MMA
+// of n dz taps takes 32 + n x cout / 4 (its operands' shared-memory reads); a
+// tile's tz + 2 planes feed one, two or three output planes each; loads and
+// epilogue run beside the MMAs.  Small grids take smaller tiles so that every
+// SM has one.
+ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
+  ConvPlan best{};
+  double best_time = 0.0;
+  const int kchunks = chunks == 1 ? 1 : 2;
+  const int ksteps = (chunks + 1) / 2, taps = chunks == 1 ? 6 : 9;
+  const int b_bytes = taps * 2 * 3 * cout * 16;
+  const int room = static_cast<int>(kConvSmem) - kConvSmemFixed;
+  const int min_x = (lx + kConvTx - 1) / kConvTx;
+  for (int tiles_x = min_x; tiles_x <= min_x + 3; ++tiles_x) {
+    const int tx = (lx + tiles_x - 1) / tiles_x, pitch = tx + 2;
+    for (int tz = 1; tz <= 16; ++tz) {
+      for (int mt = 1; mt <= 4 && mt * tz * cout <= 256; ++mt) {
+        if (mt * 128 < tx) continue;
+        int ty = std::min((mt * 128 - tx) / pitch + 1, ly);
+        const int tiles_y = (ly + ty - 1) / ty;
+        ty = (ly + tiles_y - 1) / tiles_y;
+        if (ty + 2 > 256) continue;
+        ConvPlan p{};
+        p.tx = tx;
+        p.ty = ty;
+        p.tz = tz;
+        p.pitch = pitch;
+        p.mtiles = ((ty - 1) * pitch + tx + 127) / 128;
+        p.tiles_x = tiles_x;
+        p.tiles_y = tiles_y;
+        p.tiles_z = (lz + tz - 1) / tz;
+        p.kchunks = kchunks;
+        p.ksteps = ksteps;
+        p.taps = taps;
+        p.a_tx = (ty + 2) * pitch * 16 * kchunks;
+        p.a_bytes = (p.a_tx + 127) / 128 * 128;
+        p.b_bytes = b_bytes;
+        p.b_resident = ksteps <= kConvBSlotsMax && room - ksteps * b_bytes >= 4 * p.a_bytes;
+        p.b_slots = p.b_resident ? ksteps : room - 2 * b_bytes >= 4 * p.a_bytes ? 2 : 1;
+        p.stages = std::min((room - p.b_slots * b_bytes) / p.a_bytes, kConvStagesMax);
+        if (p.stages < 2) continue;
+        const int cols = 2 * p.mtiles * tz * cout;
+        p.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
+        double mma = 0.0;
+        for (int zi = 0; zi < tz + 2; ++zi)
+          mma += 32.0 + (std::min(2, tz + 1 - zi) - std::max(0, 2 - zi) + 1) * cout / 4.0;
+        // ... or what its issue takes: about 72 cycles per tap, 49 per tile
+        mma = std::max(mma * p.mtiles, (tz + 2) * (72.0 + 49.0 * ((p.mtiles + 1) / 2))) * ksteps * taps;
+        const double loads = ksteps * (tz + 2) * p.a_tx / 30.0 + (p.b_resident ? 0.0 : ksteps * b_bytes / 30.0);
+        const double epilogue = 120.0 * p.mtiles * tz * (cout / 16);
+        const int64_t tiles = static_cast<int64_t>(tiles_x) * tiles_y * p.tiles_z;
+        const double time = static_cast<double>((tiles + kConvSms - 1) / kConvSms) *
+                                std::max(std::max(mma, loads), epilogue) + std::min(mma, loads) / 2 + epilogue;
+        if (best.tx == 0 || time < best_time) {
+          best = p;
+          best_time = time;
+        }
+      }
+    }
   }
-}
-
-// Stages, barriers and alignment slack, plus a guard region that keeps every
-// address an operand descriptor of a stage can span (up to 32 KiB past the
-// start of its A or B tile) inside the allocation.
-size_t conv_smem_bytes(int kchunks, int cout) {
-  const size_t stage = static_cast<size_t>(kchunks) * 2048 + static_cast<size_t>(kchunks) * cout * 16;
-  return 1024 + kConvStages * stage + (2 * kConvStages + 1) * 8 + 32 + 40 * 1024;
+  return best;
 }
 
 int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaStream_t st) {
   ConvArgs a = a0;
-  a.chunks = in_chunks;
-  a.taps_per_stage = in_chunks == 1 ? 2 : 1;
-  a.kchunks = a.taps_per_stage * in_chunks;
-  a.nstages = (27 + a.taps_per_stage - 1) / a.taps_per_stage;
-  a.tmem_cols = a.cout <= 32 ? 32 : (a.cout <= 64 ? 64 : 128);
-  if (a.cout % 16 != 0 || a.cout > 128 || in_chunks > 12) return -1;
-  tile_shape(a.lx, a.bx, a.by);
+  if (a.cout % 16 != 0 || a.cout > 96 || (in_chunks != 1 && in_chunks % 2 != 0)) return -1;
+  a.plan = plan_conv(a.lx, a.ly, a.lz, in_chunks, a.cout);
+  const ConvPlan& p = a.plan;
+  if (p.tx == 0) return -3;
   CUtensorMap map;
-  if (encode_planes_map(&map, in_planes, a.lx, a.ly, a.lz, in_chunks, a.bx, a.by) != 0) return -2;
-  const size_t smem = conv_smem_bytes(a.kchunks, a.cout);
+  if (encode_planes_map(&map, in_planes, a.lx, a.ly, a.lz, in_chunks, p.pitch, p.ty + 2, p.kchunks) != 0) return -2;
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !g_attr_set[dev]) {
-    cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvMaxSmem));
+    cudaFuncSetAttribute(k_conv_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
+    cudaFuncSetAttribute(k_conv_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
     g_attr_set[dev] = true;
   }
-  if (smem > kConvMaxSmem) return -3;
-  const int tiles = ((a.lx + a.bx - 1) / a.bx) * ((a.ly + a.by - 1) / a.by) * a.lz;
-  k_conv_tc<<<tiles, 128, smem, st>>>(map, a);
+  const size_t smem = static_cast<size_t>(kConvSmemFixed) + static_cast<size_t>(p.stages) * p.a_bytes +
+                      static_cast<size_t>(p.b_slots) * p.b_bytes;
+  const auto kernel = in_chunks == 1 ? k_conv_tc<true> : k_conv_tc<false>;
+  kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, kConvSms), kConvThreads, smem, st>>>(map, a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
 
@@ -787,11 +1009,6 @@ void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void*
   k_skip_back<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(
       static_cast<const uint4*>(gs), gs_plane0, static_cast<const uint4*>(gp), static_cast<const uint4*>(s), s_plane0,
       planes, lx, ly, lz, static_cast<uint4*>(out));
-}
-
-void launch_head_forward(const void* u1, const float* hw, int64_t nv, const float* f, float* g0, cudaStream_t st) {
-  k_head_forward<<<static_cast<unsigned>((nv + 255) / 256), 256, 0, st>>>(static_cast<const uint4*>(u1), hw, nv, f,
-                                                                         g0);
 }
 
 int head_blocks(int64_t nv) { return static_cast<int>((nv + 255) / 256); }
@@ -833,23 +1050,15 @@ void launch_wgrad(const void* x, int x_plane0, int cin, int cin_real, const void
 
 void launch_pack_weights(const float* w, int cout_f, int cin_real, int cin_pad, int transpose, void* pack,
                          cudaStream_t st) {
-  const int n_in = transpose ? cout_f : cin_pad;
-  const int chunks = n_in / 8;
-  const int tps = chunks == 1 ? 2 : 1;
-  const int nstages = (27 + tps - 1) / tps;
-  const int n_out = transpose ? cin_pad : cout_f;
-  const int64_t total = static_cast<int64_t>(nstages) * tps * chunks * n_out * 8;
+  const int64_t total = pack_elems(cout_f, cin_pad, transpose);
   k_pack_weights<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(
-      w, cout_f, cin_real, cin_pad, tps, nstages, transpose, static_cast<__nv_bfloat16*>(pack));
+      w, cout_f, cin_real, cin_pad, transpose, total, static_cast<__nv_bfloat16*>(pack));
 }
 
 int64_t pack_elems(int cout_f, int cin_pad, int transpose) {
   const int n_in = transpose ? cout_f : cin_pad;
-  const int chunks = n_in / 8;
-  const int tps = chunks == 1 ? 2 : 1;
-  const int nstages = (27 + tps - 1) / tps;
   const int n_out = transpose ? cin_pad : cout_f;
-  return static_cast<int64_t>(nstages) * tps * chunks * n_out * 8;
+  return static_cast<int64_t>(n_in == 8 ? 1 : n_in / 16) * (n_in == 8 ? 6 : 9) * 2 * 3 * n_out * 8;
 }
 
 void launch_round_bf16(const float* in, int64_t n, float* out, cudaStream_t st) {

@@ -190,7 +190,10 @@ int conv(tsf_unet* U, int layer, int mode, const uint4* in, int in_chunks, int l
   a.mask = mask;
   a.mask_plane0 = mask_plane0;
   a.status = U->status;
-  if (mode == kConvForward) {
+  a.head = U->rounded + kNet.head_w;
+  a.f = U->fbuf;
+  a.g0 = U->g0;
+  if (mode != kConvDgrad) {
     a.cout = l.cout;
     a.bias = U->rounded + l.b_off;
     a.wpack = U->pack_f[layer];
@@ -203,9 +206,11 @@ int conv(tsf_unet* U, int layer, int mode, const uint4* in, int in_chunks, int l
   return launch_conv(a, in, in_chunks, U->st) == 0 ? TSF_OK : TSF_ECUDA;
 }
 
-// Forward pass from U->fbuf; `keep` also stores e3b and d2b without
-// upsampling (their separate copies are read by the debug output only).
-int forward(tsf_unet* U, float tau, bool keep) {
+// Forward pass from U->fbuf.  `head`: the last convolution applies the head
+// and leaves only g0 (U->g0); otherwise it stores its activation.  `keep` also
+// stores e3b and d2b without upsampling (their separate copies are read by the
+// debug output only).
+int forward(tsf_unet* U, float tau, bool head, bool keep) {
   const int lx = U->lx, ly = U->ly, lz = U->lz;
   const int64_t n1 = (int64_t)lx * ly * lz;
   const int x2 = lx / 2, y2 = ly / 2, z2 = lz / 2, x3 = lx / 4, y3 = ly / 4, z3 = lz / 4;
@@ -225,7 +230,8 @@ int forward(tsf_unet* U, float tau, bool keep) {
   if (!r) r = conv(U, D2B, kConvForward, U->a2d, 4, x2, y2, z2, U->cat1, 0, 1, nullptr, 0);
   if (!r && keep) r = conv(U, D2B, kConvForward, U->a2d, 4, x2, y2, z2, U->a2b, 0, 0, nullptr, 0);
   if (!r) r = conv(U, D1A, kConvForward, U->cat1, 6, lx, ly, lz, U->a1d, 0, 0, nullptr, 0);
-  if (!r) r = conv(U, D1B, kConvForward, U->a1d, 2, lx, ly, lz, U->u1, 0, 0, nullptr, 0);
+  if (!r && (keep || !head)) r = conv(U, D1B, kConvForward, U->a1d, 2, lx, ly, lz, U->u1, 0, 0, nullptr, 0);
+  if (!r && head) r = conv(U, D1B, kConvHead, U->a1d, 2, lx, ly, lz, nullptr, 0, 0, nullptr, 0);
   return r;
 }
 
@@ -390,9 +396,8 @@ int tsf_unet_forward(tsf_unet* U, int lx, int ly, int lz, const float* f, float 
   int r = ensure_grid(U, lx, ly, lz, false);
   if (r) return r;
   if ((r = load_inputs(U, f, nullptr, on_device))) return r;
-  if ((r = forward(U, tau, false))) return r;
+  if ((r = forward(U, tau, true, false))) return r;
   const int64_t n1 = (int64_t)lx * ly * lz;
-  launch_head_forward(U->u1, U->rounded + kNet.head_w, n1, U->fbuf, U->g0, U->st);
   if (cudaMemcpyAsync(g0, U->g0, sizeof(float) * (size_t)n1, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                       U->st) != cudaSuccess)
     return TSF_ECUDA;
@@ -406,7 +411,7 @@ int tsf_unet_gradients(tsf_unet* U, int lx, int ly, int lz, const float* f, cons
   int r = ensure_grid(U, lx, ly, lz, true);
   if (r) return r;
   if ((r = load_inputs(U, f, g, on_device))) return r;
-  if ((r = forward(U, tau, false))) return r;
+  if ((r = forward(U, tau, false, false))) return r;
   if ((r = backward(U, nullptr))) return r;
   if (grad && cudaMemcpyAsync(grad, U->grad, sizeof(float) * kNet.nparams, cudaMemcpyDeviceToHost, U->st) != cudaSuccess)
     return TSF_ECUDA;
@@ -422,7 +427,7 @@ int tsf_unet_train_step(tsf_unet* U, int lx, int ly, int lz, const float* f, con
   int r = ensure_grid(U, lx, ly, lz, true);
   if (r) return r;
   if ((r = load_inputs(U, f, g, on_device))) return r;
-  if ((r = forward(U, tau, false))) return r;
+  if ((r = forward(U, tau, false, false))) return r;
   if ((r = backward(U, nullptr))) return r;
   U->adam_t += 1;
   const double b1 = 0.9, b2 = 0.999;
@@ -453,8 +458,7 @@ int tsf_unet_debug(tsf_unet* U, int lx, int ly, int lz, const float* f, const fl
                          16 * n1;
   if (acts_cap < need || (train && (!gz || gz_cap < need_g))) return TSF_ECAPACITY;
   if ((r = load_inputs(U, f, g, 0))) return r;
-  if ((r = forward(U, tau, true))) return r;
-  launch_head_forward(U->u1, U->rounded + kNet.head_w, n1, U->fbuf, U->g0, U->st);
+  if ((r = forward(U, tau, true, true))) return r;
   float* tmp = nullptr;
   if (dalloc(&tmp, std::max(need, train ? need_g : 0)) != cudaSuccess) return TSF_ENOMEM;
   int64_t o = 0;

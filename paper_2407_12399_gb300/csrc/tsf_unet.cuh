@@ -11,33 +11,50 @@
 namespace tsf {
 namespace unet {
 
-constexpr int kConvStages = 4;                 // TMA/MMA pipeline depth of the convolution
-constexpr size_t kConvMaxSmem = 200 * 1024;    // dynamic shared memory limit set for it
+constexpr int kConvStagesMax = 12;             // input planes in flight in a convolution block
+constexpr int kConvBSlotsMax = 6;              // K steps' weights in shared memory
+constexpr size_t kConvSmem = 220 * 1024;       // dynamic shared memory, one block per SM
+constexpr int kConvSmemFixed = 1024;           // ... of which alignment
+constexpr int kConvTx = 126;                   // voxels of a tile along x: a row with its halo is one TMA run
+constexpr int kConvSms = 152;
 constexpr uint32_t kUnetErrSpin = 1u << 5;     // a bounded wait gave up (same bit as the solver's)
 
-enum ConvMode { kConvForward = 0, kConvDgrad = 1 };
+enum ConvMode { kConvForward = 0, kConvDgrad = 1, kConvHead = 2 };
 
-// One 3x3x3 'same' convolution as an implicit GEMM (k_conv_tc).  The caller
-// fills the first group; launch_conv derives the rest.
+// Tile, pipeline and grid of one convolution launch (plan_conv).
+struct ConvPlan {
+  int tx, ty, tz;                   // output voxels of a block
+  int pitch, mtiles;                // row pitch tx + 2; operand tiles of 128 flattened positions
+  int tiles_x, tiles_y, tiles_z;
+  int kchunks, ksteps, taps;        // input planes per K step, K steps, MMA taps per K step and z-plane
+  int stages, b_slots, b_resident;  // input planes and K steps' weights in flight; all weights stay
+  int a_tx, a_bytes, b_bytes;       // bytes of a stage (loaded, reserved) and of a K step's weights
+  int tmem_cols;
+};
+
+// One 3x3x3 'same' convolution as an implicit GEMM (k_conv_tc).  launch_conv
+// fills the plan.
 struct ConvArgs {
   int lx, ly, lz;     // grid of input and output (the output of an `up` launch is 2x)
-  int cout;           // output channels (multiple of 16, <= 128)
-  int mode;           // kConvForward: relu(acc + bias); kConvDgrad: acc masked by mask > 0
+  int cout;           // output channels (multiple of 16, <= 96)
+  int mode;           // kConvForward: relu(acc + bias); kConvDgrad: acc masked by mask > 0;
+                      // kConvHead: forward, then g0 = f + the 1x1 head, nothing else stored
   int up;             // forward only: store every voxel to its 2x2x2 block of a 2x grid
   void* out;          // output planes (bf16)
   int64_t out_plane0; // first output plane
   const void* mask;   // dgrad: activation whose ReLU masks the output (may be null)
   int64_t mask_plane0;
   const float* bias;  // forward: cout biases (bf16 values)
-  const __nv_bfloat16* wpack;  // stage-packed weights (k_pack_weights)
+  const __nv_bfloat16* wpack;  // packed weights (k_pack_weights)
+  const float* head;  // kConvHead: 16 weights, then the bias (bf16 values)
+  const float* f;
+  float* g0;
   uint32_t* status;   // device status word (kUnetErrSpin)
-  // derived
-  int chunks, taps_per_stage, kchunks, nstages, tmem_cols, bx, by;
+  ConvPlan plan;
 };
 
+ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout);
 int launch_conv(const ConvArgs& a, const void* in_planes, int in_chunks, cudaStream_t st);
-size_t conv_smem_bytes(int kchunks, int cout);
-void tile_shape(int lx, int& bx, int& by);
 
 void launch_pack_input(const float* f, float tau, int64_t nv, void* x, cudaStream_t st);
 void launch_avgpool(const void* in, int in_plane0, int planes, int lx, int ly, int lz, void* out, cudaStream_t st);
@@ -45,7 +62,6 @@ void launch_upsample_back(const void* g, int g_plane0, int planes, int lx, int l
                           int act_plane0, void* out, cudaStream_t st);
 void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void* s, int s_plane0, int planes, int lx,
                       int ly, int lz, void* out, cudaStream_t st);
-void launch_head_forward(const void* u1, const float* hw, int64_t nv, const float* f, float* g0, cudaStream_t st);
 int head_blocks(int64_t nv);
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
                           double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st);
