@@ -12,10 +12,9 @@
 //
 // Convolution (forward, and the data gradient as a convolution with the
 // flipped, transposed kernel) is an implicit GEMM on the tcgen05 tensor
-// cores; k_conv_tc says how.
-
-// Weight gradients, pooling, upsampling, the 1x1 head, the loss and Adam are
-// bandwidth-bound and run on the CUDA cores.
+// cores; k_conv_tc says how.  The weight gradients are GEMMs over the voxels
+// (k_wgrad_tc).  Pooling, upsampling, the head's backward pass, the loss and
+// Adam are bandwidth-bound and run on the CUDA cores.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -106,9 +105,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both
-// K-major, M x N.
-__host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
+// K-major (or both MN-major), M x N.
+__host__ __device__ constexpr uint32_t instr_desc(int m, int n, bool mn_major = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? 3u << 15 : 0u) | (static_cast<uint32_t>(n >> 3) << 17) |
          (static_cast<uint32_t>(m >> 4) << 24);
 }
 
@@ -147,6 +146,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);  // .x = a (low half), .y = b
   return *reinterpret_cast<const uint32_t*>(&h);
@@ -176,28 +185,28 @@ __device__ __forceinline__ void store_twice(uint4* p, const uint4& q) {
 // ---------------------------------------------------------------------------
 // Convolution as an implicit GEMM on tcgen05
 // ---------------------------------------------------------------------------
-// A block computes tx x ty x tz output voxels.  For each pair of input planes
-// (16 channels, one K step) it walks the tz + 2 input z-planes; TMA brings a
-// plane's (ty + 2) x (tx + 2) voxels (zero outside the grid: the padding) as
-// 16-byte rows, one after the other.  In the no-swizzle K-major operand layout
-// 128 consecutive rows are an A tile, so a tile of 128 outputs (flattened with
-// pitch tx + 2; the two halo columns of a row give outputs that nobody keeps)
-// reads its (dy, dx) neighbours by a shift of the operand's start address: one
-// load serves nine taps.  The three dz taps of an input plane go to three
-// output planes, whose accumulators lie next to each other in TMEM, so the
-// three weight matrices form one B operand of 3 x cout columns and one MMA
-// does all three.
+// A block computes tx x ty x tz output voxels, walking the tz + 2 input
+// z-planes.  TMA brings a plane's (ty + 2) x (tx + 2) voxels of every input
+// channel (zero outside the grid: the padding) as 16-byte rows, one after the
+// other.  In the no-swizzle K-major operand layout 128 consecutive rows are an
+// A tile, so a tile of 128 outputs (flattened with pitch tx + 2; the two halo
+// columns of a row give outputs that nobody keeps) reads its (dy, dx)
+// neighbours by a shift of the operand's start address: one load serves nine
+// taps.  The three dz taps of an input plane go to three output planes, whose
+// accumulators lie next to each other in TMEM, so the three weight matrices
+// form one B operand of 3 x cout columns and one MMA does all three.  Every
+// output still sums its taps in (dz, dy, dx) order, 16 channels at a time.
 // A block per SM walks over tiles: one warp issues the loads (they run ahead
 // into the next tile), two the MMAs (half of a tile's operand tiles each),
-// eight turn accumulators into outputs
-// while the other half of TMEM (256 columns) takes the next tile's MMAs.
-// Weights that fit stay in shared memory for the whole launch.
+// eight turn accumulators into outputs while the other half of TMEM (256
+// columns) takes the next tile's MMAs.  Weights that fit stay in shared memory
+// for the whole launch, others come again for every plane.
 // Bound: the A operand.  An MMA reads 4 KB of A (32 cycles of shared-memory
 // bandwidth) and 96 x cout bytes of B, 32 + 3 x cout / 4 cycles in all, for
 // 3 x cout / 2 cycles of math, so 16 output channels reach about half of the
 // tensor rate.
-// A single input plane (8 channels) takes two dx neighbours as its K step:
-// the second K half is the first one shifted by one row.
+// A single input plane (8 channels, kSteps = 0) makes K steps of two taps: the
+// second half of K is the next tap's rows, at their distance from the first's.
 constexpr int kConvEpiWarps = 8;
 constexpr int kConvMmaWarps = 2;
 constexpr int kConvThreads = (kConvEpiWarps + 1 + kConvMmaWarps) * 32;
@@ -214,13 +223,13 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// The MMAs of one input plane: every (dy, dx) tap on kM operand tiles.
+// The MMAs of one input plane on kM operand tiles.
 struct PlaneMmas {
-  uint64_t a, b;         // operand descriptors of the first tile and tap
+  uint64_t a;            // operand descriptor of the first tile, tap and K step
+  uint32_t kstep;        // ... distance of two K steps (16-byte units)
   uint32_t t0, tcols;    // accumulators of d = 0 and the distance of two tiles'
   uint32_t cout, pitch;
   int dlo, dhi;          // dz taps that stay in the tile
-  bool first;            // first K step: output plane d = 2 starts its sums here
 };
 
 // dz taps d .. d + n - 1 of one (dy, dx) tap.
@@ -233,37 +242,63 @@ __device__ __forceinline__ void issue_tap(const PlaneMmas& f, uint64_t ad, uint6
   for (int m = 0; m < kM; ++m) mma_bf16(td + m * f.tcols, ad + m * 128u, bd, idesc, acc);
 }
 
-// Unrolled: an MMA of 48 columns takes 44 cycles, and the loop has to issue
-// one in as many.  256^3 voxels, 16 to 16 channels: rolled over taps and tiles
-// 1046 us, over tiles only 645, unrolled 437 (66 cycles per MMA: about 72 per
-// tap and 49 per tile); two warps that share the tiles take the whole layer
-// from 479 to 403 us.
-template <bool kSingle, int kM>
-__device__ __forceinline__ void issue_plane(const PlaneMmas& f) {
-  constexpr int kDx = kSingle ? 2 : 3;
+// One (dy, dx) tap on every K step; at, bt its operand rows and weights.
+// `first` (tap 0): input plane zi is the first to reach output plane zi
+// (d = 2), which starts its sums here.  kWide: three dz taps are more than 256
+// columns, so d = 2 always has an MMA of its own.
+template <int kSteps, int kM, bool kWide>
+__device__ __forceinline__ void issue_tap_steps(const PlaneMmas& f, uint64_t at, uint64_t bt, bool first) {
   const int n = f.dhi - f.dlo + 1;
-  const bool upper = f.dhi == 2 && f.dlo < 2;                       // d = 2 next to others
-  const bool wide = upper && n * static_cast<int>(f.cout) > 256;  // N <= 256
-  const bool split = wide || (f.first && upper);
-  issue_tap<kM>(f, f.a, f.b, f.dlo, split ? 2 - f.dlo : n, f.first && f.dlo == 2 ? 0u : 1u);
-  if (split) issue_tap<kM>(f, f.a, f.b, 2, 1, f.first ? 0u : 1u);
-  if (!wide) {
+  const bool upper = f.dhi == 2 && f.dlo < 2;  // d = 2 next to others
 #pragma unroll
-    for (int t = 1; t < 3 * kDx; ++t)
-      issue_tap<kM>(f, f.a + static_cast<uint32_t>(t / kDx) * f.pitch + t % kDx,
-                    f.b + static_cast<uint32_t>(t) * (6u * f.cout), f.dlo, n, 1u);
-  } else {
-#pragma unroll 1
-    for (int t = 1; t < 3 * kDx; ++t) {
-      const uint64_t ad = f.a + static_cast<uint32_t>(t / kDx) * f.pitch + t % kDx;
-      const uint64_t bd = f.b + static_cast<uint32_t>(t) * (6u * f.cout);
+  for (int kk = 0; kk < kSteps; ++kk) {
+    const uint64_t ad = at + static_cast<uint32_t>(kk) * f.kstep, bd = bt + static_cast<uint32_t>(kk) * (6u * f.cout);
+    const bool start = kk == 0 && first;
+    if ((kWide || start) && upper) {
       issue_tap<kM>(f, ad, bd, f.dlo, 2 - f.dlo, 1u);
-      issue_tap<kM>(f, ad, bd, 2, 1, 1u);
+      issue_tap<kM>(f, ad, bd, 2, 1, start ? 0u : 1u);
+    } else {
+      issue_tap<kM>(f, ad, bd, f.dlo, n, start && f.dlo == 2 ? 0u : 1u);
     }
   }
 }
 
-template <bool kSingle>
+// Every tap of one input plane (resident weights at b, btap apart).  An MMA of
+// 48 columns takes 44 cycles, and the loop has to issue one in as many.
+// 256^3 voxels, 16 to 16 channels: rolled over taps and tiles 1046 us, over
+// tiles only 645, unrolled 437 (66 cycles per MMA: about 72 per tap and 49 per
+// tile); two warps that share the tiles take the whole layer from 479 to 403
+// us.  With two or more K steps the tap loop stays rolled: a small grid's one
+// pass through a long unrolled body waits for its instructions (32^3, 32 to
+// 32 channels: 22 us unrolled, 14 rolled).
+template <int kSteps, int kM, bool kWide>
+__device__ __forceinline__ void issue_plane(const PlaneMmas& f, uint64_t b, uint32_t btap) {
+  issue_tap_steps<kSteps, kM, kWide>(f, f.a, b, true);
+#pragma unroll(kSteps == 1 ? 8 : 1)
+  for (int tap = 1; tap < 9; ++tap)
+    issue_tap_steps<kSteps, kM, kWide>(f, f.a + static_cast<uint32_t>(tap / 3) * f.pitch + static_cast<uint32_t>(tap % 3),
+                                       b + static_cast<uint32_t>(tap) * btap, false);
+}
+
+// A single input plane of 8 channels: the 14 K steps (27 taps in pairs; the
+// last tap's partner has zero weights) of one output plane, from the input
+// planes at a, a + dplane, a + 2 dplane.
+template <int kM>
+__device__ __forceinline__ void issue_single(const PlaneMmas& f, uint32_t dplane, uint64_t bt) {
+  const uint32_t idesc = instr_desc(128, static_cast<int>(f.cout));
+#pragma unroll
+  for (int t = 0; t < 14; ++t) {
+    const int t0 = 2 * t, t1 = t == 13 ? 26 : 2 * t + 1;
+    const uint32_t o0 = static_cast<uint32_t>(t0 / 9) * dplane + static_cast<uint32_t>(t0 / 3 % 3) * f.pitch + t0 % 3;
+    const uint32_t o1 = static_cast<uint32_t>(t1 / 9) * dplane + static_cast<uint32_t>(t1 / 3 % 3) * f.pitch + t1 % 3;
+    const uint64_t ad = f.a + o0 + (static_cast<uint64_t>(o1 - o0) << 16);  // the distance of the K halves
+    const uint64_t bd = bt + static_cast<uint32_t>(t) * (2u * f.cout);
+#pragma unroll
+    for (int m = 0; m < kM; ++m) mma_bf16(f.t0 + m * f.tcols, ad + m * 128u, bd, idesc, t > 0 ? 1u : 0u);
+  }
+}
+
+template <int kSteps, bool kWide = false>
 __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_constant__ CUtensorMap in_map, ConvArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ ConvBars sh;
@@ -279,7 +314,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_consta
       mbar_init(&sh.full_a[s], 1);
       mbar_init(&sh.empty_a[s], kConvMmaWarps);
     }
-    for (int s = 0; s < p.b_slots; ++s) {
+    for (int s = 0; s < kConvBSlotsMax; ++s) {
       mbar_init(&sh.full_b[s], 1);
       mbar_init(&sh.empty_b[s], kConvMmaWarps);
     }
@@ -310,15 +345,24 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_consta
   const uint32_t thalf = static_cast<uint32_t>(p.tmem_cols / 2);
 
   if (role == kConvEpiWarps && lane == 0) {
-    // producer: per tile and K step the weights (once, if all stay resident),
-    // then the input planes
+    // producer: each plane, then its taps' weights (once, if all stay, after
+    // the first plane; else again as the ring frees up)
     int it = 0, bt = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
       const int x0 = (tile % p.tiles_x) * p.tx, y0 = ((tile / p.tiles_x) % p.tiles_y) * p.ty,
                 z0 = tile / (p.tiles_x * p.tiles_y) * p.tz;
-      for (int kk = 0; kk < p.ksteps && ok; ++kk) {
-        if (!p.b_resident || bt < p.ksteps) {
+      for (int zi = 0; zi < p.tz + 2 && ok; ++zi, ++it) {
+        const int slot = it % p.stages;
+        if (it >= p.stages && !mbar_wait(&sh.empty_a[slot], ((it / p.stages) - 1) & 1)) ok = false;
+        if (!ok || *gave_up) {
+          ok = false;
+          break;
+        }
+        mbar_expect_tx(&sh.full_a[slot], p.a_tx);
+        tma_load_4d(smem + slot * p.a_bytes, &in_map, 2 * (x0 - 1), y0 - 1, z0 - 1 + zi, 0, &sh.full_a[slot]);
+        sh.issued_a = it + 1;
+        for (int tap = 0; (!p.b_resident || it == 0) && tap < p.taps; ++tap, ++bt) {
           const int bs = bt % p.b_slots;
           if (bt >= p.b_slots && !mbar_wait(&sh.empty_b[bs], ((bt / p.b_slots) - 1) & 1)) ok = false;
           if (!ok || *gave_up) {
@@ -326,21 +370,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_consta
             break;
           }
           mbar_expect_tx(&sh.full_b[bs], p.b_bytes);
-          bulk_load(sb0 + bs * p.b_bytes, a.wpack + static_cast<size_t>(kk) * (p.b_bytes / 2), p.b_bytes,
+          bulk_load(sb0 + bs * p.b_bytes, a.wpack + static_cast<size_t>(tap) * (p.b_bytes / 2), p.b_bytes,
                     &sh.full_b[bs]);
-          sh.issued_b = ++bt;
-        }
-        for (int zi = 0; zi < p.tz + 2; ++zi, ++it) {
-          const int slot = it % p.stages;
-          if (it >= p.stages && !mbar_wait(&sh.empty_a[slot], ((it / p.stages) - 1) & 1)) ok = false;
-          if (!ok || *gave_up) {
-            ok = false;
-            break;
-          }
-          mbar_expect_tx(&sh.full_a[slot], p.a_tx);
-          tma_load_4d(smem + slot * p.a_bytes, &in_map, 2 * (x0 - 1), y0 - 1, z0 - 1 + zi, kk * p.kchunks,
-                      &sh.full_a[slot]);
-          sh.issued_a = it + 1;
+          sh.issued_b = bt + 1;
         }
       }
     }
@@ -353,9 +385,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_consta
     // their address fields (in units of 16 bytes)
     const int m0 = role == kConvEpiWarps + 1 ? 0 : (p.mtiles + 1) / 2;
     const int nm = role == kConvEpiWarps + 1 ? (p.mtiles + 1) / 2 : p.mtiles / 2;
-    const uint32_t a_lbo = kSingle ? 16u : static_cast<uint32_t>((p.ty + 2) * p.pitch) * 16u;
-    const uint32_t b_lbo = static_cast<uint32_t>(3 * a.cout) * 16u;
-    const uint32_t tcols = static_cast<uint32_t>(p.tz * a.cout), cout = static_cast<uint32_t>(a.cout);
+    const uint32_t a_lbo = kSteps == 0 ? 0u : static_cast<uint32_t>((p.ty + 2) * p.pitch) * 16u;
+    const uint32_t b_lbo = static_cast<uint32_t>((kSteps == 0 ? 1 : 3) * a.cout) * 16u;
+    const uint32_t tcols = static_cast<uint32_t>(p.tz * a.cout);
     int it = 0, bt = 0, nt = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++nt) {
@@ -365,33 +397,59 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __grid_consta
         break;
       }
       tc_fence_after();
-      for (int kk = 0; kk < p.ksteps && ok; ++kk, ++bt) {
-        const int bs = bt % p.b_slots;
-        if ((!p.b_resident || nt == 0) &&
-            !mbar_wait_warp(&sh.full_b[bs], p.b_resident ? 0 : (bt / p.b_slots) & 1)) {
+      const uint32_t tmine = taddr + (half ? thalf : 0u) + static_cast<uint32_t>(m0) * tcols;
+      for (int zi = 0; zi < p.tz + 2 && ok; ++zi, ++it) {
+        const int slot = it % p.stages;
+        if (!mbar_wait_warp(&sh.full_a[slot], (it / p.stages) & 1) || __any_sync(0xFFFFFFFFu, *gave_up)) {
           ok = false;
           break;
         }
-        const uint64_t bbase = smem_desc(smem_u32(sb0 + bs * p.b_bytes), b_lbo, 128u);
-        for (int zi = 0; zi < p.tz + 2; ++zi, ++it) {
-          const int slot = it % p.stages;
-          if (!mbar_wait_warp(&sh.full_a[slot], (it / p.stages) & 1) || __any_sync(0xFFFFFFFFu, *gave_up)) {
-            ok = false;
-            break;
+        tc_fence_after();
+        if (kSteps == 0) {
+          // planes zi - 2 .. zi make output plane zi - 2 (a tile's planes lie
+          // one after the other: stages is a multiple of tz + 2)
+          for (int tap = 0; it == 0 && tap < p.taps && ok; ++tap) ok = mbar_wait_warp(&sh.full_b[tap], 0);
+          if (zi < 2) continue;
+          const uint64_t abase = smem_desc(smem_u32(smem + (slot - 2) * p.a_bytes), a_lbo, 128u);
+          const PlaneMmas f{abase + static_cast<uint32_t>(m0) * 128u, 0u, tmine + static_cast<uint32_t>((zi - 2) * a.cout),
+                            tcols, static_cast<uint32_t>(a.cout), static_cast<uint32_t>(p.pitch), 0, 0};
+          const uint64_t bd = smem_desc(smem_u32(sb0), b_lbo, 128u);
+          if (nm == 1) issue_single<1>(f, static_cast<uint32_t>(p.a_bytes / 16), bd);
+          else if (nm == 2) issue_single<2>(f, static_cast<uint32_t>(p.a_bytes / 16), bd);
+          mma_commit(&sh.empty_a[slot - 2]);  // the slot is free once these MMAs have read it
+          if (zi == p.tz + 1) {
+            mma_commit(&sh.empty_a[slot - 1]);
+            mma_commit(&sh.empty_a[slot]);
           }
-          tc_fence_after();
-          // input plane zi feeds output planes zi - 2 + d (dz tap 2 - d)
-          const int dlo = max(0, 2 - zi), dhi = min(2, p.tz + 1 - zi);
-          const uint64_t abase = smem_desc(smem_u32(smem + slot * p.a_bytes), a_lbo, 128u);
-          const PlaneMmas f{abase + static_cast<uint32_t>(m0) * 128u, bbase,
-                            taddr + (half ? thalf : 0u) + static_cast<uint32_t>(m0) * tcols +
-                                static_cast<uint32_t>((zi - 2) * a.cout),
-                            tcols, cout, static_cast<uint32_t>(p.pitch), dlo, dhi, kk == 0};
-          if (nm == 1) issue_plane<kSingle, 1>(f);
-          else if (nm == 2) issue_plane<kSingle, 2>(f);
-          mma_commit(&sh.empty_a[slot]);  // the slot is free once these MMAs have read it
+          continue;
         }
-        if (ok && !p.b_resident) mma_commit(&sh.empty_b[bs]);
+        // input plane zi feeds output planes zi - 2 + d (dz tap 2 - d)
+        const uint64_t abase = smem_desc(smem_u32(smem + slot * p.a_bytes), a_lbo, 128u);
+        const PlaneMmas f{abase + static_cast<uint32_t>(m0) * 128u, 2u * (a_lbo >> 4),
+                          tmine + static_cast<uint32_t>((zi - 2) * a.cout), tcols, static_cast<uint32_t>(a.cout),
+                          static_cast<uint32_t>(p.pitch), max(0, 2 - zi), min(2, p.tz + 1 - zi)};
+        constexpr int kS = kSteps > 0 ? kSteps : 1;
+        if (p.b_resident && it > 0) {
+          const uint64_t bbase = smem_desc(smem_u32(sb0), b_lbo, 128u);
+          const uint32_t btap = static_cast<uint32_t>(p.b_bytes) >> 4;
+          if (nm == 1) issue_plane<kS, 1, kWide>(f, bbase, btap);
+          else if (nm == 2) issue_plane<kS, 2, kWide>(f, bbase, btap);
+        } else {  // weights arrive tap by tap
+          for (int tap = 0; tap < 9; ++tap, ++bt) {
+            const int bs = bt % p.b_slots;
+            if (!mbar_wait_warp(&sh.full_b[bs], (bt / p.b_slots) & 1)) {
+              ok = false;
+              break;
+            }
+            const uint64_t bd = smem_desc(smem_u32(sb0 + bs * p.b_bytes), b_lbo, 128u);
+            const uint64_t at = f.a + static_cast<uint32_t>(tap / 3) * f.pitch + static_cast<uint32_t>(tap % 3);
+            if (nm == 1) issue_tap_steps<kS, 1, kWide>(f, at, bd, tap == 0);
+            else if (nm == 2) issue_tap_steps<kS, 2, kWide>(f, at, bd, tap == 0);
+            if (!p.b_resident) mma_commit(&sh.empty_b[bs]);
+          }
+          if (!ok) break;
+        }
+        mma_commit(&sh.empty_a[slot]);
       }
       if (ok) mma_commit(&sh.tfull[half]);
     }
@@ -594,17 +652,20 @@ __global__ void k_skip_back(const uint4* __restrict__ gs, int gs_plane0, const u
 // Head, backward for the loss mean((g0 - g)^2): per voxel gg = 2 (g0 - g) / nv;
 // the u1 gradient gg * w masked by u1's ReLU; block partial sums (fp64) of
 // the loss, of gg and of gg * u1[c] (the head's bias and weight gradients).
+// Bound: fp64 arithmetic (two operations per clock on an SM), most of all the
+// warp sums, so a block per SM loops over the voxels and sums across a warp
+// once: 64^3 voxels 71 us with a block per 256 voxels, 32 us now.
 __global__ void __launch_bounds__(256) k_head_backward(const uint4* __restrict__ u1, const float* __restrict__ hw,
                                                        int64_t nv, const float* __restrict__ f,
                                                        const float* __restrict__ g, uint4* __restrict__ gz,
                                                        double* __restrict__ partial) {
   __shared__ double red[18][8];
   const float hb = hw[16];
-  const int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   double acc[18];
 #pragma unroll
   for (int k = 0; k < 18; ++k) acc[k] = 0.0;
-  if (v < nv) {
+  for (int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; v < nv;
+       v += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     float a[16];
     unpack8(u1[v], a);
     unpack8(u1[nv + v], a + 8);
@@ -614,12 +675,12 @@ __global__ void __launch_bounds__(256) k_head_backward(const uint4* __restrict__
     r = __bfloat162float(__float2bfloat16_rn(r + hb));
     const float d = (f[v] + r) - g[v];
     const float gg = 2.0f * d / static_cast<float>(nv);
-    acc[0] = static_cast<double>(d) * d;
-    acc[1] = gg;
+    acc[0] += static_cast<double>(d) * d;
+    acc[1] += gg;
     float o[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-      acc[2 + c] = static_cast<double>(gg) * a[c];
+      acc[2 + c] += static_cast<double>(gg) * a[c];
       o[c] = a[c] > 0.0f ? gg * hw[c] : 0.0f;
     }
     gz[v] = pack8(o);
@@ -640,182 +701,295 @@ __global__ void __launch_bounds__(256) k_head_backward(const uint4* __restrict__
   }
 }
 
-// Sums the head's block partials in block order: out[0] = loss (mean),
-// grad[hw_off + c] = sum gg u1[c], grad[hb_off] = sum gg.
-__global__ void k_head_reduce(const double* __restrict__ partial, int nblocks, int64_t nv, double* __restrict__ loss,
-                              float* __restrict__ grad, int64_t hw_off, int64_t hb_off) {
-  const int k = threadIdx.x;
-  if (k >= 18) return;
+// Sums the head's block partials, one warp per value, in a fixed order: out[0]
+// = loss (mean), grad[hw_off + c] = sum gg u1[c], grad[hb_off] = sum gg.
+__global__ void __launch_bounds__(18 * 32) k_head_reduce(const double* __restrict__ partial, int nblocks, int64_t nv,
+                                                         double* __restrict__ loss, float* __restrict__ grad,
+                                                         int64_t hw_off, int64_t hb_off) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += partial[static_cast<int64_t>(b) * 18 + k];
+  for (int b = lane; b < nblocks; b += 32) s += partial[static_cast<int64_t>(b) * 18 + k];
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if (lane != 0) return;
   if (k == 0) *loss = s / static_cast<double>(nv);
   else if (k == 1) grad[hb_off] = static_cast<float>(s);
   else grad[hw_off + (k - 2)] = static_cast<float>(s);
 }
 
 // Weight gradient of one convolution: gw[o][c][tap] = sum over voxels p of
-// gz[o][p] x[c][p + tap - 1] (zero outside the grid), gb[o] = sum gz[o][p].
-// Block (tap, chunk of kWgV voxels in linear order); each thread owns a
-// 4 (o) x 4 (c) register tile and a share of the voxels; partial sums per
-// block, reduced in block order by k_wgrad_reduce (deterministic).
-constexpr int kWgV = 64;     // voxels staged in shared memory at a time
-constexpr int kWgChunk = 1024;  // voxels per block
+// gz[o][p] x[c][p + tap - 1] (zero outside the grid), gb[o] = sum gz[o][p],
+// as a GEMM over the voxels on the tensor cores.  The chunk planes are
+// MN-major operands as they lie: 8 channels of a voxel are one 16-byte row, 8
+// consecutive voxels a core matrix, so 16 voxels along x are a K step.
+//   M: the cout channels of gz, three times: shifted by the dy taps (copies
+//      that TMA loads; with 64 channels one copy, and a third of the blocks
+//      per dy).
+//   N: a block of input channels at the planes z - 1, z, z + 1 (dz taps).
+//   The three dx taps are shifts of the N operand's start address by one row,
+//   each with its own accumulator, issued by its own warp.
+// gz is zero outside the grid and tx is a multiple of 16, so every pair of a
+// voxel and a tap counts once.  A step is one z-plane of a tx x ty tile; a
+// block takes a range of steps, keeps its sums in TMEM, and writes one partial
+// per launch; k_wgrad_reduce adds the partials in a fixed order.
+// Bound: loads (gz and x three times each, from L2).  64^3 voxels, 48 to 16
+// channels: 2264 us on the CUDA cores with operands converted to fp32 in
+// shared memory, 23 us here.
+constexpr int kWgThreads = 256;  // warps 0-3 bias and epilogue, 4 loads, 5-7 MMAs of one dx tap each
+constexpr int kWgStagesMax = 4;
 
-__global__ void __launch_bounds__(256) k_wgrad(const uint4* __restrict__ x, int x_plane0, int cin,
-                                               const uint4* __restrict__ gz, int cout, int lx, int ly, int lz,
-                                               float* __restrict__ partial) {
-  extern __shared__ float wsm[];
-  float* sg = wsm;                    // [cout][kWgV]
-  float* sx = wsm + cout * kWgV;      // [cin][kWgV]
-  float* sred = sx + cin * kWgV;      // reduction across voxel groups
-  const int tap = blockIdx.y;
-  const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-  const int64_t nv = static_cast<int64_t>(lx) * ly * lz;
-  const int64_t v0 = static_cast<int64_t>(blockIdx.x) * kWgChunk;
-  const int to = cout / 4, tc = cin / 4, ntile = to * tc;
-  const int groups = max(1, 256 / ntile);  // voxel groups sharing the tiles
-  const int tid = threadIdx.x;
-  const int tile = tid % ntile, grp = tid / ntile;
-  const bool active = tid < ntile * groups;
-  const int o0 = (tile / tc) * 4, c0 = (tile % tc) * 4;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-  for (int64_t vb = v0; vb < v0 + kWgChunk && vb < nv; vb += kWgV) {
-    __syncthreads();
-    // stage gz (cout planes) and the tap-shifted x (cin planes) as fp32
-    for (int i = tid; i < (cout / 8) * kWgV; i += 256) {
-      const int p = i / kWgV, k = i % kWgV;
-      const int64_t v = vb + k;
-      float t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      if (v < nv) unpack8(gz[p * nv + v], t);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) sg[(p * 8 + c) * kWgV + k] = t[c];
+struct WgBars {
+  uint64_t full[kWgStagesMax], empty[kWgStagesMax], done;
+  uint32_t taddr;
+  int gave_up, issued;
+  float bias[128 * 8];
+};
+
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ CUtensorMap x_map,
+                                                            const __grid_constant__ CUtensorMap g_map, WgradPlan p,
+                                                            float* __restrict__ partial, float* __restrict__ bpartial,
+                                                            uint32_t* status) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ WgBars sh;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* gave_up = &sh.gave_up;
+  const int cb = blockIdx.y % p.cin_blocks, dyi = blockIdx.y / p.cin_blocks;  // input channel block, dy tap (one copy)
+  const int s0 = static_cast<int>(static_cast<int64_t>(p.steps) * blockIdx.x / gridDim.x);
+  const int s1 = static_cast<int>(static_cast<int64_t>(p.steps) * (blockIdx.x + 1) / gridDim.x);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&sh.full[s], 1);
+      mbar_init(&sh.empty[s], 3 + 4);
     }
-    for (int i = tid; i < (cin / 8) * kWgV; i += 256) {
-      const int p = i / kWgV, k = i % kWgV;
-      const int64_t v = vb + k;
-      float t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      if (v < nv) {
-        const int vx = static_cast<int>(v % lx) + dx, vy = static_cast<int>((v / lx) % ly) + dy,
-                  vz = static_cast<int>(v / (static_cast<int64_t>(lx) * ly)) + dz;
-        if (vx >= 0 && vx < lx && vy >= 0 && vy < ly && vz >= 0 && vz < lz)
-          unpack8(x[(x_plane0 + p) * nv + (static_cast<int64_t>(vz) * ly + vy) * lx + vx], t);
-      }
-#pragma unroll
-      for (int c = 0; c < 8; ++c) sx[(p * 8 + c) * kWgV + k] = t[c];
-    }
-    __syncthreads();
-    if (active) {
-      for (int k = grp; k < kWgV; k += groups) {
-        float go[4], xc[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) go[i] = sg[(o0 + i) * kWgV + k];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xc[j] = sx[(c0 + j) * kWgV + k];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(go[i], xc[j], acc[i][j]);
-      }
-    }
+    mbar_init(&sh.done, 3);
+    sh.gave_up = 0;
+    sh.issued = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // combine the voxel groups (fixed order), then write the block's partial
+  __syncwarp();
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.taddr)),
+                 "r"(static_cast<uint32_t>(p.tmem_cols))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
   __syncthreads();
-  float* out = partial + (static_cast<int64_t>(tap) * gridDim.x + blockIdx.x) * cout * cin;
-  for (int g = 0; g < groups; ++g) {
-    if (active && grp == g) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float* p = &sred[(o0 + i) * cin + c0 + j];
-          *p = (g == 0 ? 0.0f : *p) + acc[i][j];
+  tc_fence_after();
+  const uint32_t taddr = __shfl_sync(0xFFFFFFFFu, sh.taddr, 0);
+  const int role = __shfl_sync(0xFFFFFFFFu, warp, 0);
+  const int n = 24 * p.cin_chunks;  // N: dz taps x 8 channels per plane
+
+  if (role == 4 && lane == 0) {
+    bool ok = true;
+    for (int s = s0, it = 0; s < s1; ++s, ++it) {
+      const int slot = it % p.stages;
+      if (it >= p.stages && !mbar_wait(&sh.empty[slot], ((it / p.stages) - 1) & 1)) ok = false;
+      if (!ok || *gave_up) {
+        ok = false;
+        break;
+      }
+      const int z = s % p.lz, t = s / p.lz;
+      const int x0 = (t % p.tiles_x) * p.tx, y0 = (t / p.tiles_x) * p.ty;
+      uint8_t* sg = smem + slot * p.stage_bytes;
+      mbar_expect_tx(&sh.full[slot], p.tx_bytes);
+      for (int c = 0; c < p.copies; ++c) {  // row y of copy c holds gz at y - dy, dy = c - 1
+        const int dy = p.copies == 3 ? c : dyi;
+        tma_load_4d(sg + c * p.copy_bytes, &g_map, 2 * x0, y0 + 1 - dy, z, 0, &sh.full[slot]);
+      }
+      tma_load_4d(sg + p.copies * p.copy_bytes, &x_map, 2 * (x0 - 1), y0, z - 1, cb * p.cin_chunks, &sh.full[slot]);
+      sh.issued = it + 1;
+    }
+    if (!ok) {
+      if (!*gave_up) atomicOr(status, kUnetErrSpin);
+      *gave_up = 1;
+    }
+  } else if (role > 4) {
+    const int dx = role - 5;
+    const uint32_t idesc = instr_desc(p.m, n, true);
+    const uint32_t td = taddr + static_cast<uint32_t>(dx * n);
+    const uint32_t g_sbo = static_cast<uint32_t>(p.tx * p.ty) * 16u, x_sbo = static_cast<uint32_t>(p.pitch * p.ty) * 16u;
+    const int kx = p.tx / 16;
+    uint32_t acc = 0u;
+    bool ok = true;
+    for (int s = s0, it = 0; s < s1; ++s, ++it) {
+      const int slot = it % p.stages;
+      if (!mbar_wait_warp(&sh.full[slot], (it / p.stages) & 1) || __any_sync(0xFFFFFFFFu, *gave_up)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t sg = smem_u32(smem + slot * p.stage_bytes);
+      uint64_t ad = smem_desc(sg, 128u, g_sbo);
+      uint64_t brow = smem_desc(sg + static_cast<uint32_t>(p.copies * p.copy_bytes), 128u, x_sbo) + dx;
+      for (int y = 0; y < p.ty; ++y) {
+        uint64_t bd = brow;
+#pragma unroll 4
+        for (int k = 0; k < kx; ++k) {
+          mma_bf16(td, ad, bd, idesc, acc);
+          acc = 1u;
+          ad += 16u;
+          bd += 16u;
         }
+        brow += static_cast<uint32_t>(p.pitch);
+      }
+      mma_commit(&sh.empty[slot]);
     }
-    __syncthreads();
-  }
-  for (int i = tid; i < cout * cin; i += 256) out[i] = sred[i];
-}
-
-// gw in the reference layout (cout, cin_real, 3, 3, 3) = sum over blocks of
-// the partials, in block order.
-__global__ void k_wgrad_reduce(const float* __restrict__ partial, int nblk, int cout, int cin, int cin_real,
-                               float* __restrict__ gw) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // over 27 * cout * cin_real
-  if (i >= 27 * cout * cin_real) return;
-  const int tap = i % 27, c = (i / 27) % cin_real, o = i / (27 * cin_real);
-  const float* p = partial + static_cast<int64_t>(tap) * nblk * cout * cin + o * cin + c;
-  float s = 0.0f;
-  for (int b = 0; b < nblk; ++b) s += p[static_cast<int64_t>(b) * cout * cin];
-  gw[i] = s;
-}
-
-// gb[o] = sum over voxels of gz[o]: block partials, then an ordered sum.
-__global__ void __launch_bounds__(256) k_bias_partial(const uint4* __restrict__ gz, int cout, int64_t nv,
-                                                      float* __restrict__ partial) {
-  __shared__ float red[8][96];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t v0 = static_cast<int64_t>(blockIdx.x) * 2048;
-  for (int p = 0; p < cout / 8; ++p) {
+    if (!ok && lane == 0) {
+      if (!*gave_up) atomicOr(status, kUnetErrSpin);
+      *gave_up = 1;
+    }
+    __syncwarp();
+    mma_commit(&sh.done);
+    mbar_wait_warp(&sh.done, 0);
+  } else if (role < 4) {
+    // bias: thread t sums channels of plane t / per over the rows t % per,
+    // t % per + per, ... of the unshifted copy
+    const bool bias = cb == 0 && (p.copies == 3 || dyi == 1);
+    const int per = 128 / p.cout_chunks, plane = threadIdx.x / per, rows = p.tx * p.ty;
+    const int copy = p.copies == 3 ? 1 : 0;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t v = v0 + threadIdx.x; v < v0 + 2048 && v < nv; v += 256) {
-      float t[8];
-      unpack8(gz[p * nv + v], t);
+    bool ok = true;
+    for (int s = s0, it = 0; s < s1; ++s, ++it) {
+      const int slot = it % p.stages;
+      if (!mbar_wait_warp(&sh.full[slot], (it / p.stages) & 1) || __any_sync(0xFFFFFFFFu, *gave_up)) {
+        ok = false;
+        break;
+      }
+      if (bias) {
+        const uint4* g = reinterpret_cast<const uint4*>(smem + slot * p.stage_bytes + copy * p.copy_bytes) +
+                         static_cast<size_t>(plane) * rows;
+        for (int r = threadIdx.x % per; r < rows; r += per) {
+          float t[8];
+          unpack8(g[r], t);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) acc[c] += t[c];
+          for (int c = 0; c < 8; ++c) acc[c] += t[c];
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.empty[slot]);
     }
+    if (ok && !mbar_wait_warp(&sh.done, 0)) ok = false;
+    if (__any_sync(0xFFFFFFFFu, !ok || *gave_up)) {
+      if (lane == 0) {
+        if (!*gave_up) atomicOr(status, kUnetErrSpin);
+        *gave_up = 1;
+      }
+    } else {
+      tc_fence_after();
+      // M = 64: row 16 w + l in lane l < 16 of warp w; M = 128: row 32 w + l
+      const int row = p.m == 64 ? (lane < 16 ? warp * 16 + lane : p.m) : warp * 32 + lane;
+      const int mrows = p.copies * p.cout_chunks * 8;
+      float* out = partial + (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * (3 * mrows * n);
+      for (int dx = 0; dx < 3; ++dx)
+        for (int c = 0; c < n; c += 8) {
+          float v[8];
+          __syncwarp();
+          tmem_ld8(taddr + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(dx * n + c), v);
+          if (s0 >= s1) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      float x = acc[c];
-      for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-      if (lane == 0) red[w][p * 8 + c] = x;
+            for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+          }
+          if (row < mrows) {
+            float4* o = reinterpret_cast<float4*>(out + (static_cast<size_t>(dx) * mrows + row) * n + c);
+            o[0] = make_float4(v[0], v[1], v[2], v[3]);
+            o[1] = make_float4(v[4], v[5], v[6], v[7]);
+          }
+        }
+      tc_fence_before();
+    }
+    if (bias) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) sh.bias[threadIdx.x * 8 + c] = acc[c];
     }
   }
   __syncthreads();
-  if (threadIdx.x < cout) {
-    float s = 0.0f;
-    for (int i = 0; i < 8; ++i) s += red[i][threadIdx.x];
-    partial[static_cast<int64_t>(blockIdx.x) * cout + threadIdx.x] = s;
+  if (cb == 0 && (p.copies == 3 || dyi == 1) && threadIdx.x < p.cout_chunks * 8) {
+    const int per = 128 / p.cout_chunks, plane = threadIdx.x / 8, c = threadIdx.x % 8;
+    float sum = 0.0f;
+    for (int t = 0; t < per; ++t) sum += sh.bias[(plane * per + t) * 8 + c];
+    bpartial[static_cast<size_t>(blockIdx.x) * p.cout_chunks * 8 + threadIdx.x] = sum;
+  }
+  // after giving up, wait (bounded) for the copies still in flight before the
+  // shared memory they target is released
+  if (threadIdx.x == 0 && *gave_up) {
+    for (int s = max(0, sh.issued - p.stages); s < sh.issued; ++s)
+      mbar_wait(&sh.full[s % p.stages], (s / p.stages) & 1);
+  }
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr),
+                 "r"(static_cast<uint32_t>(p.tmem_cols))
+                 : "memory");
   }
 }
 
-__global__ void k_bias_reduce(const float* __restrict__ partial, int nblk, int cout, float* __restrict__ gb) {
-  const int o = threadIdx.x;
-  if (o >= cout) return;
+// gw in the reference layout (cout, cin_real, 3, 3, 3) and gb: the partials
+// summed as eight interleaved shares of the blocks, then the shares, in fixed
+// order.  Thread (i, share): element i of a partial's order, so that reads are
+// coalesced.
+__global__ void __launch_bounds__(256) k_wgrad_reduce(WgradPlan p, const float* __restrict__ partial,
+                                                      const float* __restrict__ bpartial, int cin_real,
+                                                      float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float red[8][32];
+  const int lane = threadIdx.x & 31, share = threadIdx.x >> 5;
+  const int n = 24 * p.cin_chunks, cout = p.cout_chunks * 8, mrows = p.copies * cout;
+  const int per = 3 * mrows * n, total = p.groups * per;
+  const int i = blockIdx.x * 32 + lane;
+  const bool weight = i < total, bias = !weight && i < total + cout;
+  const float* src = weight ? partial + static_cast<size_t>(i / per) * p.blocks * per + i % per : bpartial + (i - total);
+  const size_t step = weight ? per : cout;
   float s = 0.0f;
-  for (int b = 0; b < nblk; ++b) s += partial[static_cast<int64_t>(b) * cout + o];
-  gb[o] = s;
+  if (weight || bias) {
+#pragma unroll 8
+    for (int b = share; b < p.blocks; b += 8) s += src[static_cast<size_t>(b) * step];
+  }
+  red[share][lane] = s;
+  __syncthreads();
+  if (share != 0) return;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) s += red[k][lane];
+  if (bias) gb[i - total] = s;
+  if (!weight) return;
+  const int grp = i / per, cb = grp % p.cin_blocks, dyg = grp / p.cin_blocks;
+  const int col = i % n, row = (i % per) / n % mrows, dx = (i % per) / n / mrows;
+  const int e = col % 8, dz = col / 8 % 3, c = (cb * p.cin_chunks + col / 24) * 8 + e;
+  const int o = row % cout, dy = p.copies == 3 ? row / cout : dyg;
+  if (c < cin_real) gw[(static_cast<int64_t>(o) * cin_real + c) * 27 + (dz * 3 + dy) * 3 + dx] = s;
 }
 
 // Weights of one layer from the fp32 master copy (reference layout
 // (cout, cin_real, 3, 3, 3)) into the bf16 B operand of k_conv_tc:
-// pack[K step][tap][K half][d * n_out + o][8], d = 0..2 for the dz tap 2 - d.
-// Two input planes make a K step of nine (dy, dx) taps; a single one makes a
-// K step of three dy times the dx pairs (0, 1) and (-, 2).  The data-gradient
-// packing transposes and flips: B[o'][c'][tap] = w[c'][o'][26 - tap] (o' over
-// the forward inputs, c' over its outputs).
+// pack[(dy, dx) tap][K step][K half][d * n_out + o][8], d = 0..2 for the dz
+// tap 2 - d; for a single input plane pack[pair of taps][K half][o][8].  The
+// data-gradient packing transposes and flips: B[o'][c'][tap] =
+// w[c'][o'][26 - tap] (o' over the forward inputs, c' over its outputs).
 __global__ void k_pack_weights(const float* __restrict__ w, int cout_f, int cin_real, int cin_pad, int transpose,
                                int64_t total, __nv_bfloat16* __restrict__ pack) {
   const int n_out = transpose ? cin_pad : cout_f;   // N of the GEMM
   const int n_in = transpose ? cout_f : cin_pad;    // input channels of the GEMM
-  const bool single = n_in == 8;
-  const int taps = single ? 6 : 9;
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= total) return;
   const int e = static_cast<int>(i % 8);
-  const int n = static_cast<int>((i / 8) % (3 * n_out));
-  const int half = static_cast<int>((i / (24 * n_out)) % 2);
-  const int t = static_cast<int>((i / (48 * n_out)) % taps);
-  const int kk = static_cast<int>(i / (static_cast<int64_t>(48) * n_out * taps));
-  const int o = n % n_out, dz = 2 - n / n_out;
-  const int dy = single ? t >> 1 : t / 3, dx = single ? (t & 1) + half : t % 3;
-  const int ci = single ? e : (kk * 2 + half) * 8 + e;
-  const int tap = (dz * 3 + dy) * 3 + dx;
+  int o, ci, tap;
+  if (n_in == 8) {
+    o = static_cast<int>((i / 8) % n_out);
+    tap = static_cast<int>(i / (8 * n_out));  // pair and half
+    ci = e;
+  } else {
+    const int ksteps = n_in / 16;
+    const int n = static_cast<int>((i / 8) % (3 * n_out));
+    const int half = static_cast<int>((i / (24 * n_out)) % 2);
+    const int kk = static_cast<int>((i / (48 * n_out)) % ksteps);
+    const int t = static_cast<int>(i / (static_cast<int64_t>(48) * n_out * ksteps));
+    o = n % n_out;
+    ci = (kk * 2 + half) * 8 + e;
+    tap = (2 - n / n_out) * 9 + t;
+  }
   float val = 0.0f;
-  if (!(single && (t & 1) && half == 0)) {  // dx = 1 is in the first pair
+  if (tap < 27) {
     if (!transpose) {
       if (ci < cin_real) val = w[(static_cast<int64_t>(o) * cin_real + ci) * 27 + tap];
     } else {  // GEMM output o = forward input channel, GEMM input ci = forward output channel
@@ -877,7 +1051,7 @@ bool g_attr_set[64] = {};
 // elements): TMA takes three to five cycles per innermost run, and with
 // 16-byte runs it, not the tensor cores, set the time.  x coordinates are
 // multiples of two elements, 16 bytes.
-int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz, int chunks, int bx, int by,
+int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz, int chunks, int bx, int by, int bz,
                       int bchunks) {
   if (!g_encode) {
     cudaDriverEntryPointQueryResult q;
@@ -891,7 +1065,7 @@ int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz
   cuuint64_t dims[4] = {2 * static_cast<cuuint64_t>(lx), static_cast<cuuint64_t>(ly), static_cast<cuuint64_t>(lz),
                         static_cast<cuuint64_t>(chunks)};
   cuuint64_t strides[3] = {16ull * lx, 16ull * lx * ly, 16ull * nv};
-  cuuint32_t box[4] = {2 * static_cast<cuuint32_t>(bx), static_cast<cuuint32_t>(by), 1,
+  cuuint32_t box[4] = {2 * static_cast<cuuint32_t>(bx), static_cast<cuuint32_t>(by), static_cast<cuuint32_t>(bz),
                        static_cast<cuuint32_t>(bchunks)};
   cuuint32_t es[4] = {1, 1, 1, 1};
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(base), dims, strides, box, es,
@@ -903,14 +1077,14 @@ int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz
 // Tile of a convolution: the shape of least estimated time, in cycles.  An MMA
 // of n dz taps takes 32 + n x cout / 4 (its operands' shared-memory reads); a
 // tile's tz + 2 planes feed one, two or three output planes each; loads and
-// epilogue run beside the MMAs.  Small grids take smaller tiles so that every
-// SM has one.
+// epilogue run beside the MMAs, and a change of tiles costs about 1200.  Small
+// grids take smaller tiles so that every SM has one.
 ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
   ConvPlan best{};
   double best_time = 0.0;
-  const int kchunks = chunks == 1 ? 1 : 2;
-  const int ksteps = (chunks + 1) / 2, taps = chunks == 1 ? 6 : 9;
-  const int b_bytes = taps * 2 * 3 * cout * 16;
+  const bool single = chunks == 1;
+  const int ksteps = chunks / 2, taps = single ? 14 : 9;
+  const int b_bytes = single ? 2 * cout * 16 : ksteps * 2 * 3 * cout * 16;  // weights of a tap (of a pair of taps)
   const int room = static_cast<int>(kConvSmem) - kConvSmemFixed;
   const int min_x = (lx + kConvTx - 1) / kConvTx;
   for (int tiles_x = min_x; tiles_x <= min_x + 3; ++tiles_x) {
@@ -931,28 +1105,35 @@ ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
         p.tiles_x = tiles_x;
         p.tiles_y = tiles_y;
         p.tiles_z = (lz + tz - 1) / tz;
-        p.kchunks = kchunks;
-        p.ksteps = ksteps;
+        p.chunks = chunks;
         p.taps = taps;
-        p.a_tx = (ty + 2) * pitch * 16 * kchunks;
+        p.a_tx = (ty + 2) * pitch * 16 * chunks;
         p.a_bytes = (p.a_tx + 127) / 128 * 128;
         p.b_bytes = b_bytes;
-        p.b_resident = ksteps <= kConvBSlotsMax && room - ksteps * b_bytes >= 4 * p.a_bytes;
-        p.b_slots = p.b_resident ? ksteps : room - 2 * b_bytes >= 4 * p.a_bytes ? 2 : 1;
-        p.stages = std::min((room - p.b_slots * b_bytes) / p.a_bytes, kConvStagesMax);
-        if (p.stages < 2) continue;
+        p.b_resident = room - taps * b_bytes >= 3 * p.a_bytes;
+        p.b_slots = taps;
+        if (p.b_resident) {
+          p.stages = std::min((room - taps * b_bytes) / p.a_bytes, kConvStagesMax);
+        } else {  // up to three planes, the rest of the room for weights
+          p.stages = std::min((room - 3 * b_bytes) / p.a_bytes, 3);
+          p.b_slots = std::min((room - p.stages * p.a_bytes) / b_bytes, taps);
+        }
+        if (single) p.stages = p.stages / (tz + 2) * (tz + 2);
+        if (single ? !p.b_resident || p.stages < tz + 2 : p.stages < 2) continue;
         const int cols = 2 * p.mtiles * tz * cout;
         p.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
+        const int groups = single ? tz * taps : (tz + 2) * taps * ksteps;  // operand pairs issued per tile
         double mma = 0.0;
         for (int zi = 0; zi < tz + 2; ++zi)
           mma += 32.0 + (std::min(2, tz + 1 - zi) - std::max(0, 2 - zi) + 1) * cout / 4.0;
+        mma = single ? tz * 14 * 40.0 : mma * taps * ksteps;
         // ... or what its issue takes: about 72 cycles per tap, 49 per tile
-        mma = std::max(mma * p.mtiles, (tz + 2) * (72.0 + 49.0 * ((p.mtiles + 1) / 2))) * ksteps * taps;
-        const double loads = ksteps * (tz + 2) * p.a_tx / 30.0 + (p.b_resident ? 0.0 : ksteps * b_bytes / 30.0);
+        mma = std::max(mma * p.mtiles, groups * (72.0 + 49.0 * ((p.mtiles + 1) / 2)));
+        const double loads = (tz + 2) * (p.a_tx + (p.b_resident ? 0.0 : static_cast<double>(taps) * b_bytes)) / 30.0;
         const double epilogue = 120.0 * p.mtiles * tz * (cout / 16);
         const int64_t tiles = static_cast<int64_t>(tiles_x) * tiles_y * p.tiles_z;
         const double time = static_cast<double>((tiles + kConvSms - 1) / kConvSms) *
-                                std::max(std::max(mma, loads), epilogue) + std::min(mma, loads) / 2 + epilogue;
+                                std::max(std::max(mma + 1200.0, loads), epilogue) + std::min(mma, loads) / 2 + epilogue;
         if (best.tx == 0 || time < best_time) {
           best = p;
           best_time = time;
@@ -965,22 +1146,31 @@ ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
 
 int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaStream_t st) {
   ConvArgs a = a0;
-  if (a.cout % 16 != 0 || a.cout > 96 || (in_chunks != 1 && in_chunks % 2 != 0)) return -1;
+  using Kernel = void (*)(const CUtensorMap, ConvArgs);
+  // the network's layers; more than 85 output channels: from 32 inputs only
+  const Kernel kernel = in_chunks == 1    ? k_conv_tc<0>
+                        : in_chunks == 2  ? k_conv_tc<1>
+                        : in_chunks == 4  ? (a.cout > 85 ? k_conv_tc<2, true> : k_conv_tc<2>)
+                        : in_chunks == 6  ? k_conv_tc<3>
+                        : in_chunks == 8  ? k_conv_tc<4>
+                        : in_chunks == 12 ? k_conv_tc<6>
+                                          : nullptr;
+  if (!kernel || a.cout % 16 != 0 || a.cout > 96 || (a.cout > 85 && in_chunks != 4)) return -1;
   a.plan = plan_conv(a.lx, a.ly, a.lz, in_chunks, a.cout);
   const ConvPlan& p = a.plan;
   if (p.tx == 0) return -3;
   CUtensorMap map;
-  if (encode_planes_map(&map, in_planes, a.lx, a.ly, a.lz, in_chunks, p.pitch, p.ty + 2, p.kchunks) != 0) return -2;
+  if (encode_planes_map(&map, in_planes, a.lx, a.ly, a.lz, in_chunks, p.pitch, p.ty + 2, 1, in_chunks) != 0) return -2;
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !g_attr_set[dev]) {
-    cudaFuncSetAttribute(k_conv_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
-    cudaFuncSetAttribute(k_conv_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
+    for (const Kernel k : {k_conv_tc<0>, k_conv_tc<1>, k_conv_tc<2>, k_conv_tc<2, true>, k_conv_tc<3>, k_conv_tc<4>,
+                           k_conv_tc<6>})
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
     g_attr_set[dev] = true;
   }
   const size_t smem = static_cast<size_t>(kConvSmemFixed) + static_cast<size_t>(p.stages) * p.a_bytes +
                       static_cast<size_t>(p.b_slots) * p.b_bytes;
-  const auto kernel = in_chunks == 1 ? k_conv_tc<true> : k_conv_tc<false>;
   kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, kConvSms), kConvThreads, smem, st>>>(map, a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
@@ -1011,41 +1201,76 @@ void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void*
       planes, lx, ly, lz, static_cast<uint4*>(out));
 }
 
-int head_blocks(int64_t nv) { return static_cast<int>((nv + 255) / 256); }
+int head_blocks(int64_t nv) { return static_cast<int>(std::min<int64_t>((nv + 255) / 256, kConvSms)); }
 
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
                           double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st) {
   const int nb = head_blocks(nv);
   k_head_backward<<<nb, 256, 0, st>>>(static_cast<const uint4*>(u1), hw, nv, f, g, static_cast<uint4*>(gz), partial);
-  k_head_reduce<<<1, 32, 0, st>>>(partial, nb, nv, loss, grad, hw_off, hb_off);
+  k_head_reduce<<<1, 18 * 32, 0, st>>>(partial, nb, nv, loss, grad, hw_off, hb_off);
 }
 
-int64_t wgrad_partial_floats(int64_t nv, int cout, int cin) {
-  const int64_t nblk = (nv + kWgChunk - 1) / kWgChunk;
-  return 27 * nblk * cout * cin;
+WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout) {
+  WgradPlan p{};
+  p.lz = lz;
+  p.cout_chunks = cout / 8;
+  p.copies = 3 * cout <= 128 ? 3 : 1;
+  p.cin_blocks = cin > 48 ? 2 : 1;
+  p.cin_chunks = cin / 8 / p.cin_blocks;
+  p.groups = p.cin_blocks * (3 / p.copies);
+  p.m = p.copies * cout <= 64 ? 64 : 128;
+  const int cols = 3 * 24 * p.cin_chunks;
+  p.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
+  p.tiles_x = (lx + kWgTx - 1) / kWgTx;
+  p.tx = ((lx + p.tiles_x - 1) / p.tiles_x + 15) / 16 * 16;
+  p.pitch = p.tx + 2;
+  // rows per step: four stages in shared memory, and four steps for every
+  // block (each block's partial is written and read once more)
+  const int row_bytes = 16 * (3 * p.cin_chunks * p.pitch + p.copies * p.cout_chunks * p.tx);
+  int blocks = std::max(kConvSms / p.groups, 1);
+  const int by_smem = std::max(static_cast<int>(kWgSmem / kWgStagesMax) / row_bytes, 1);
+  const int by_steps = std::max(static_cast<int>(static_cast<int64_t>(ly) * lz * p.tiles_x / (4 * blocks)), 1);
+  p.ty = std::min(std::min(by_smem, by_steps), std::min(ly, 256));
+  p.tiles_y = (ly + p.ty - 1) / p.ty;
+  p.ty = (ly + p.tiles_y - 1) / p.tiles_y;
+  p.steps = p.tiles_x * p.tiles_y * lz;
+  blocks = std::min(blocks, std::max(p.steps / 4, 1));
+  p.blocks = blocks;
+  p.copy_bytes = p.ty * p.tx * 16 * p.cout_chunks;
+  p.tx_bytes = p.ty * row_bytes;
+  p.stage_bytes = (p.tx_bytes + 127) / 128 * 128;
+  p.stages = std::min(static_cast<int>(kWgSmem) / p.stage_bytes, kWgStagesMax);
+  return p;
 }
 
-int64_t bias_partial_floats(int64_t nv, int cout) { return ((nv + 2047) / 2048) * cout; }
+int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout) {
+  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout).blocks) * 27 * cin * cout;
+}
 
-void launch_wgrad(const void* x, int x_plane0, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
-                  float* partial, float* gw, float* bpartial, float* gb, cudaStream_t st) {
-  const int64_t nv = static_cast<int64_t>(lx) * ly * lz;
-  const int nblk = static_cast<int>((nv + kWgChunk - 1) / kWgChunk);
-  const size_t smem = (static_cast<size_t>(cout + cin) * kWgV + static_cast<size_t>(cout) * cin) * sizeof(float);
+int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout) {
+  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout).blocks) * cout;
+}
+
+int launch_wgrad(const void* x, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
+                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, cudaStream_t st) {
+  const WgradPlan p = plan_wgrad(lx, ly, lz, cin, cout);
+  if (p.stages < 1 || cout % 16 != 0 || cout > 64 || cin > 96) return -1;
+  CUtensorMap xm, gm;
+  if (encode_planes_map(&xm, x, lx, ly, lz, cin / 8, p.pitch, p.ty, 3, p.cin_chunks) != 0 ||
+      encode_planes_map(&gm, gz, lx, ly, lz, p.cout_chunks, p.tx, p.ty, 1, p.cout_chunks) != 0)
+    return -2;
   static bool attr[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr[dev]) {
-    cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kWgSmem) + 1024);
     attr[dev] = true;
   }
-  k_wgrad<<<dim3(nblk, 27), 256, smem, st>>>(static_cast<const uint4*>(x), x_plane0, cin,
-                                             static_cast<const uint4*>(gz), cout, lx, ly, lz, partial);
-  const int n = 27 * cout * cin_real;
-  k_wgrad_reduce<<<(n + 255) / 256, 256, 0, st>>>(partial, nblk, cout, cin, cin_real, gw);
-  const int nb = static_cast<int>((nv + 2047) / 2048);
-  k_bias_partial<<<nb, 256, 0, st>>>(static_cast<const uint4*>(gz), cout, nv, bpartial);
-  k_bias_reduce<<<1, 128, 0, st>>>(bpartial, nb, cout, gb);
+  k_wgrad_tc<<<dim3(p.blocks, p.groups), kWgThreads, static_cast<size_t>(p.stages) * p.stage_bytes + 1024, st>>>(
+      xm, gm, p, partial, bpartial, status);
+  const int n = 27 * cin * cout + cout;
+  k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(p, partial, bpartial, cin_real, gw, gb);
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
 
 void launch_pack_weights(const float* w, int cout_f, int cin_real, int cin_pad, int transpose, void* pack,
@@ -1058,7 +1283,7 @@ void launch_pack_weights(const float* w, int cout_f, int cin_real, int cin_pad, 
 int64_t pack_elems(int cout_f, int cin_pad, int transpose) {
   const int n_in = transpose ? cout_f : cin_pad;
   const int n_out = transpose ? cin_pad : cout_f;
-  return static_cast<int64_t>(n_in == 8 ? 1 : n_in / 16) * (n_in == 8 ? 6 : 9) * 2 * 3 * n_out * 8;
+  return n_in == 8 ? static_cast<int64_t>(14) * 2 * n_out * 8 : static_cast<int64_t>(9) * n_in * 3 * n_out;
 }
 
 void launch_round_bf16(const float* in, int64_t n, float* out, cudaStream_t st) {

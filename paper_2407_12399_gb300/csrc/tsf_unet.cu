@@ -146,10 +146,11 @@ int ensure_grid(tsf_unet* U, int lx, int ly, int lz, bool train) {
     A(&U->gp1, 2 * n2);
     if (e == cudaSuccess) e = dalloc(&U->gbuf, n1);
     int64_t wp = 0, bp = 0;
-    const int64_t nv_of[NCONV] = {n1, n1, n2, n2, n3, n3, n2, n2, n1, n1};
+    const int level[NCONV] = {1, 1, 2, 2, 4, 4, 2, 2, 1, 1};
     for (int i = 0; i < NCONV; ++i) {
-      wp = std::max(wp, wgrad_partial_floats(nv_of[i], kNet.L[i].cout, kNet.L[i].cin_pad));
-      bp = std::max(bp, bias_partial_floats(nv_of[i], kNet.L[i].cout));
+      const int k = level[i], cin = kNet.L[i].cin_pad, cout = kNet.L[i].cout;
+      wp = std::max(wp, wgrad_partial_floats(lx / k, ly / k, lz / k, cin, cout));
+      bp = std::max(bp, bias_partial_floats(lx / k, ly / k, lz / k, cin, cout));
     }
     if (e == cudaSuccess) e = dalloc(&U->wpart, wp);
     if (e == cudaSuccess) e = dalloc(&U->bpart, bp);
@@ -235,10 +236,13 @@ int forward(tsf_unet* U, float tau, bool head, bool keep) {
   return r;
 }
 
-void wgrad(tsf_unet* U, int layer, const uint4* x, int x_plane0, const uint4* gz, int lx, int ly, int lz) {
+int wgrad(tsf_unet* U, int layer, const uint4* x, const uint4* gz, int lx, int ly, int lz) {
   const Layer& l = kNet.L[layer];
-  launch_wgrad(x, x_plane0, l.cin_pad, l.cin_real, gz, l.cout, lx, ly, lz, U->wpart, U->grad + l.w_off, U->bpart,
-               U->grad + l.b_off, U->st);
+  tsf::note_launch();
+  return launch_wgrad(x, l.cin_pad, l.cin_real, gz, l.cout, lx, ly, lz, U->wpart, U->grad + l.w_off, U->bpart,
+                      U->grad + l.b_off, U->status, U->st) == 0
+             ? TSF_OK
+             : TSF_ECUDA;
 }
 
 // Backward pass of mean((g0 - g)^2) after forward(); parameter gradients in
@@ -260,38 +264,38 @@ int backward(tsf_unet* U, float* keep) {
   launch_head_backward(U->u1, U->rounded + kNet.head_w, n1, U->fbuf, U->gbuf, U->gzA1, U->hpart, U->loss, U->grad,
                        kNet.head_w, kNet.head_b, st);
   put(U->gzA1, 16, n1);
-  wgrad(U, D1B, U->a1d, 0, U->gzA1, lx, ly, lz);
+  if (!r) r = wgrad(U, D1B, U->a1d, U->gzA1, lx, ly, lz);
   if (!r) r = conv(U, D1B, kConvDgrad, U->gzA1, 2, lx, ly, lz, U->gzB1, 0, 0, U->a1d, 0);
   put(U->gzB1, 16, n1);
-  wgrad(U, D1A, U->cat1, 0, U->gzB1, lx, ly, lz);
+  if (!r) r = wgrad(U, D1A, U->cat1, U->gzB1, lx, ly, lz);
   if (!r) r = conv(U, D1A, kConvDgrad, U->gzB1, 2, lx, ly, lz, U->gcat1, 0, 0, nullptr, 0);
   launch_upsample_back(U->gcat1, 0, 4, lx, ly, lz, U->cat1, 0, U->gzA2, st);
   put(U->gzA2, 32, n2);
-  wgrad(U, D2B, U->a2d, 0, U->gzA2, x2, y2, z2);
+  if (!r) r = wgrad(U, D2B, U->a2d, U->gzA2, x2, y2, z2);
   if (!r) r = conv(U, D2B, kConvDgrad, U->gzA2, 4, x2, y2, z2, U->gzB2, 0, 0, U->a2d, 0);
   put(U->gzB2, 32, n2);
-  wgrad(U, D2A, U->cat2, 0, U->gzB2, x2, y2, z2);
+  if (!r) r = wgrad(U, D2A, U->cat2, U->gzB2, x2, y2, z2);
   if (!r) r = conv(U, D2A, kConvDgrad, U->gzB2, 4, x2, y2, z2, U->gcat2, 0, 0, nullptr, 0);
   launch_upsample_back(U->gcat2, 0, 8, x2, y2, z2, U->cat2, 0, U->gzA3, st);
   put(U->gzA3, 64, n3);
-  wgrad(U, E3B, U->a3a, 0, U->gzA3, x3, y3, z3);
+  if (!r) r = wgrad(U, E3B, U->a3a, U->gzA3, x3, y3, z3);
   if (!r) r = conv(U, E3B, kConvDgrad, U->gzA3, 8, x3, y3, z3, U->gzB3, 0, 0, U->a3a, 0);
   put(U->gzB3, 64, n3);
-  wgrad(U, E3A, U->p2, 0, U->gzB3, x3, y3, z3);
+  if (!r) r = wgrad(U, E3A, U->p2, U->gzB3, x3, y3, z3);
   if (!r) r = conv(U, E3A, kConvDgrad, U->gzB3, 8, x3, y3, z3, U->gp2, 0, 0, nullptr, 0);
   launch_skip_back(U->gcat2, 8, U->gp2, U->cat2, 8, 4, x2, y2, z2, U->gzA2, st);
   put(U->gzA2, 32, n2);
-  wgrad(U, E2B, U->a2a, 0, U->gzA2, x2, y2, z2);
+  if (!r) r = wgrad(U, E2B, U->a2a, U->gzA2, x2, y2, z2);
   if (!r) r = conv(U, E2B, kConvDgrad, U->gzA2, 4, x2, y2, z2, U->gzB2, 0, 0, U->a2a, 0);
   put(U->gzB2, 32, n2);
-  wgrad(U, E2A, U->p1, 0, U->gzB2, x2, y2, z2);
+  if (!r) r = wgrad(U, E2A, U->p1, U->gzB2, x2, y2, z2);
   if (!r) r = conv(U, E2A, kConvDgrad, U->gzB2, 4, x2, y2, z2, U->gp1, 0, 0, nullptr, 0);
   launch_skip_back(U->gcat1, 4, U->gp1, U->cat1, 4, 2, lx, ly, lz, U->gzA1, st);
   put(U->gzA1, 16, n1);
-  wgrad(U, E1B, U->a1a, 0, U->gzA1, lx, ly, lz);
+  if (!r) r = wgrad(U, E1B, U->a1a, U->gzA1, lx, ly, lz);
   if (!r) r = conv(U, E1B, kConvDgrad, U->gzA1, 2, lx, ly, lz, U->gzB1, 0, 0, U->a1a, 0);
   put(U->gzB1, 16, n1);
-  wgrad(U, E1A, U->xin, 0, U->gzB1, lx, ly, lz);
+  if (!r) r = wgrad(U, E1A, U->xin, U->gzB1, lx, ly, lz);
   return r;
 }
 

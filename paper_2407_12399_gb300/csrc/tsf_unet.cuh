@@ -12,7 +12,7 @@ namespace tsf {
 namespace unet {
 
 constexpr int kConvStagesMax = 12;             // input planes in flight in a convolution block
-constexpr int kConvBSlotsMax = 6;              // K steps' weights in shared memory
+constexpr int kConvBSlotsMax = 14;             // taps' weights in shared memory
 constexpr size_t kConvSmem = 220 * 1024;       // dynamic shared memory, one block per SM
 constexpr int kConvSmemFixed = 1024;           // ... of which alignment
 constexpr int kConvTx = 126;                   // voxels of a tile along x: a row with its halo is one TMA run
@@ -26,9 +26,9 @@ struct ConvPlan {
   int tx, ty, tz;                   // output voxels of a block
   int pitch, mtiles;                // row pitch tx + 2; operand tiles of 128 flattened positions
   int tiles_x, tiles_y, tiles_z;
-  int kchunks, ksteps, taps;        // input planes per K step, K steps, MMA taps per K step and z-plane
-  int stages, b_slots, b_resident;  // input planes and K steps' weights in flight; all weights stay
-  int a_tx, a_bytes, b_bytes;       // bytes of a stage (loaded, reserved) and of a K step's weights
+  int chunks, taps;                 // input planes; (dy, dx) taps (pairs of taps for a single input plane)
+  int stages, b_slots, b_resident;  // z-planes and taps' weights in shared memory; all weights stay
+  int a_tx, a_bytes, b_bytes;       // bytes of a z-plane (loaded, reserved) and of a tap's weights
   int tmem_cols;
 };
 
@@ -65,10 +65,22 @@ void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void*
 int head_blocks(int64_t nv);
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
                           double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st);
-int64_t wgrad_partial_floats(int64_t nv, int cout, int cin);
-int64_t bias_partial_floats(int64_t nv, int cout);
-void launch_wgrad(const void* x, int x_plane0, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
-                  float* partial, float* gw, float* bpartial, float* gb, cudaStream_t st);
+// Weight gradient of one convolution (k_wgrad_tc): tile, operand blocks and
+// grid (blocks x groups).
+struct WgradPlan {
+  int tx, ty, pitch, tiles_x, tiles_y, lz, steps;  // voxels of a step, row pitch of x, steps = tiles x z-planes
+  int cout_chunks, cin_chunks, cin_blocks;         // planes of gz; planes of x per block, blocks of input channels
+  int copies, groups, m, tmem_cols;                // dy copies of gz; launches side by side; M of the MMAs
+  int copy_bytes, tx_bytes, stage_bytes, stages;
+  int blocks;                                      // blocks per group = partials
+};
+constexpr int kWgTx = 112;                // voxels of a step along x, at most
+constexpr size_t kWgSmem = 208 * 1024;    // stages of a block
+WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout);
+int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout);
+int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout);
+int launch_wgrad(const void* x, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
+                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, cudaStream_t st);
 void launch_pack_weights(const float* w, int cout_f, int cin_real, int cin_pad, int transpose, void* pack,
                          cudaStream_t st);
 int64_t pack_elems(int cout_f, int cin_pad, int transpose);
