@@ -289,14 +289,12 @@ int64_t tsf_kernel_launches(void);
 
 /* Test and tuning knobs of the pairing (process-wide, not in the paper;
  * results never depend on them, only the schedule and the bounds):
- *   1: items from which the union-find rounds run over the whole GPU
- *      (default 65536; below, one block runs them);
- *   2: active items below which one block finishes the rounds (default 8192);
- *   3: cap on the union-find rounds (default 0 = none; a cap that is hit
- *      makes the call fail with TSF_ETIMEOUT);
- *   4: polls a block waits at a grid barrier of the whole-GPU rounds (union-
- *      find and D1 reduction) before it gives up (default 2^24; giving up
- *      makes the call fail with TSF_ETIMEOUT);
+ *   1, 2: no effect (kept for callers that set them);
+ *   3: cap on the steps of a union-find item (default 0 = none; a cap that
+ *      is hit makes the call fail with TSF_ETIMEOUT);
+ *   4: limit of the pairing's device waits and walks: polls at a grid barrier
+ *      of the D1 reduction's whole-GPU rounds, steps of a union-find item
+ *      (default 2^24; giving up makes the call fail with TSF_ETIMEOUT);
  *   5: critical triangles from which the D1 reduction starts with rounds
  *      over the whole GPU (default 262144);
  *   6: active D1 columns below which they go on on warps (default 131072);

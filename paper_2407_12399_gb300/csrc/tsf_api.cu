@@ -221,17 +221,11 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
   if (items > F->cap_items || nodes > F->cap_nodes) {
     int ci = std::max(items, F->cap_items), cn = std::max(nodes, F->cap_nodes);
     dev_free(F->PS.ends);
-    dev_free(F->PS.roots);
-    dev_free(F->PS.listA);
-    dev_free(F->PS.listB);
-    dev_free(F->PS.parent);
-    dev_free(F->PS.reserve);
+    dev_free(F->PS.rec);
+    dev_free(F->PS.skip);
     ck(dev_alloc(&F->PS.ends, 2 * (size_t)ci));
-    ck(dev_alloc(&F->PS.roots, 2 * (size_t)ci));
-    ck(dev_alloc(&F->PS.listA, ci));
-    ck(dev_alloc(&F->PS.listB, ci));
-    ck(dev_alloc(&F->PS.parent, cn));
-    ck(dev_alloc(&F->PS.reserve, cn));
+    ck(dev_alloc(&F->PS.rec, cn));
+    ck(dev_alloc(&F->PS.skip, cn));
     F->cap_items = ci;
     F->cap_nodes = cn;
   }
@@ -764,11 +758,8 @@ int tsf_destroy_field(tsf_field* F) {
   dev_free(F->L.c2_ve);
   dev_free(F->L.c3);
   dev_free(F->PS.ends);
-  dev_free(F->PS.roots);
-  dev_free(F->PS.listA);
-  dev_free(F->PS.listB);
-  dev_free(F->PS.parent);
-  dev_free(F->PS.reserve);
+  dev_free(F->PS.rec);
+  dev_free(F->PS.skip);
   dev_free(F->PS.counter);
   dev_free(F->PO.d0_min);
   dev_free(F->PO.d0_killed);

@@ -98,13 +98,10 @@ void launch_zero_pairs(const Dims& d, const uint32_t* rank, unsigned long long* 
 
 // ---- k_pairs.cu ----------------------------------------------------------
 struct PairScratch {
-  int32_t* ends;      // 2 per item: component endpoints
-  int32_t* parent;    // union-find parents over nodes
-  int32_t* reserve;   // per node reservation
-  int32_t* listA;     // active item lists
-  int32_t* listB;
-  int32_t* roots;     // 2 per item
-  int32_t* counter;   // device counters (>= 4 ints)
+  int32_t* ends;             // 2 per item: component endpoints
+  unsigned long long* rec;   // per node: union-find record and shortcut (k_uf_items)
+  unsigned long long* skip;
+  int32_t* counter;          // control block of the D1 reduction (64 bytes)
 };
 void launch_d0(const Dims& d, const NbrDelta& nd, const CritLists& L, int n0, int n1, const uint8_t* vnext8,
                const uint32_t* cidx, PairScratch& S, PairOut& P, uint32_t* status, cudaStream_t st);
