@@ -87,9 +87,76 @@ __global__ void __launch_bounds__(kTileT) k_tile_sort(int n, const int* __restri
   for (int i = threadIdx.x; i < m; i += kTileT) out[base + i] = I[i];
 }
 
+// Few items: an item's place is the number of items before it, counted by
+// brute force over the whole GPU (n / 256 x n / kRankChunk blocks) in three
+// launches, where a radix or merge sort's dozen small launches wait for one
+// another.  Ranks of equal keys follow the comparator, so the result is the
+// merge sort's.  Measured on 5e3 contributions of a 128^3 iteration: the
+// gradient step's stage 161 us with the radix sorts, 48 us with this; the
+// crossover with the radix sorts lies above kRankMax (n^2 work).
+constexpr int kRankMax = 8192, kRankChunk = 256;
+
 template <class Less>
-static int32_t* merge_sort(int n, int32_t* a, int32_t* b, Less less, cudaStream_t st, const int* n_dev = nullptr) {
+__global__ void __launch_bounds__(256) k_rank_keys(int n, const int* __restrict__ n_dev, Less less,
+                                                   unsigned long long* __restrict__ keys, int32_t* __restrict__ rank) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  rank[i] = 0;
+  if (i < (n_dev ? min(*n_dev, n) : n)) keys[i] = less.key(i);
+}
+
+template <class Less>
+__global__ void __launch_bounds__(256) k_rank_count(int n, const int* __restrict__ n_dev, Less less,
+                                                    const unsigned long long* __restrict__ keys,
+                                                    int32_t* __restrict__ rank) {
+  __shared__ unsigned long long K[kRankChunk];
+  if (n_dev) n = min(*n_dev, n);
+  const int i = blockIdx.x * 256 + threadIdx.x, j0 = blockIdx.y * kRankChunk, m = min(kRankChunk, n - j0);
+  if (m <= 0 || (int)blockIdx.x * 256 >= n) return;
+  for (int j = threadIdx.x; j < m; j += 256) K[j] = keys[j0 + j];
+  __syncthreads();
+  if (i >= n) return;
+  const unsigned long long k = keys[i];
+  int before = 0, equal = 0;
+#pragma unroll 16
+  for (int j = 0; j < m; ++j) {
+    const unsigned long long kj = K[j];
+    before += kj < k ? 1 : 0;
+    equal += kj == k ? 1 : 0;
+  }
+  if (equal > (i >= j0 && i < j0 + m ? 1 : 0))  // others with this key: the comparator decides
+    for (int j = 0; j < m; ++j)
+      if (K[j] == k && j0 + j != i && (less(j0 + j, i) || (j0 + j < i && !less(i, j0 + j)))) ++before;
+  if (before) atomicAdd(rank + i, before);
+}
+
+__global__ void __launch_bounds__(256) k_rank_place(int n, const int* __restrict__ n_dev,
+                                                    const int32_t* __restrict__ rank, int32_t* __restrict__ out) {
+  if (n_dev) n = min(*n_dev, n);
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i < n) out[rank[i]] = i;
+}
+
+// scratch: 3 n words, 8-byte aligned
+template <class Less>
+static int32_t* rank_sort(int n, int32_t* out, Less less, uint32_t* scratch, cudaStream_t st,
+                          const int* n_dev = nullptr) {
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(scratch);
+  int32_t* rank = reinterpret_cast<int32_t*>(keys + n);
+  const unsigned nb = (unsigned)((n + 255) / 256);
+  k_rank_keys<<<nb, 256, 0, st>>>(n, n_dev, less, keys, rank); note_launch();
+  k_rank_count<<<dim3(nb, (unsigned)((n + kRankChunk - 1) / kRankChunk)), 256, 0, st>>>(n, n_dev, less, keys, rank);
+  note_launch();
+  k_rank_place<<<nb, 256, 0, st>>>(n, n_dev, rank, out); note_launch();
+  return out;
+}
+
+// Order of n items by a comparator; rs (may be null): scratch for few items.
+template <class Less>
+static int32_t* merge_sort(int n, int32_t* a, int32_t* b, Less less, cudaStream_t st, const int* n_dev = nullptr,
+                           uint32_t* rs = nullptr) {
   if (n <= 0) return a;
+  if (rs && n <= kRankMax) return rank_sort(n, a, less, rs, st, n_dev);
   k_tile_sort<<<(n + kTile - 1) / kTile, kTileT, 0, st>>>(n, n_dev, a, less); note_launch();
   for (int w = kTile; w < n; w *= 2) {
     k_merge_pass<<<(n + 255) / 256, 256, 0, st>>>(n, n_dev, w, a, b, less); note_launch();
@@ -124,10 +191,19 @@ __global__ void k_gather_u32(int n, const uint32_t* __restrict__ src, const uint
   if (i < n) dst[i] = src[perm[i]];
 }
 
+// A key function as a comparator: equal keys in index order.
+template <class KeyFn>
+struct KeyThenIndex {
+  KeyFn kf;
+  __device__ unsigned long long key(int i) const { return kf(i); }
+  __device__ bool operator()(int a, int b) const { return a < b; }
+};
+
 template <class KeyFn>
 static int32_t* radix_sort64(int n, const int* n_dev, KeyFn kf, uint32_t* rs, int32_t* tmp, int32_t* out,
                              uint32_t* status, cudaStream_t st) {
   if (n <= 0) return out;
+  if (n <= kRankMax) return rank_sort(n, out, KeyThenIndex<KeyFn>{kf}, rs, st, n_dev);
   uint32_t* lo = rs;
   uint32_t* hi = lo + n;
   uint32_t* hi2 = hi + n;
@@ -313,7 +389,7 @@ int build_diagram(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1,
   cudaMemcpyAsync(&np, B.count, sizeof(int), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
   if (np > cap) return -np;
-  int32_t* idx = merge_sort(np, B.idxA, B.idxB, DiagLess{B.tmp_pts}, st);
+  int32_t* idx = merge_sort(np, B.idxA, B.idxB, DiagLess{B.tmp_pts}, st, nullptr, np <= B.cap_rsort ? B.rsort : nullptr);
   k_gather_pts<<<(np + 255) / 256, 256, 0, st>>>(np, idx, B.tmp_pts, out); note_launch();
   return np;
 }
@@ -400,29 +476,34 @@ __device__ __forceinline__ int key_cmp(const Pt& x, const Pt& y) {
 
 // For each current point (in key order) the k-th point with its key is still
 // if the reference list has at least k points with that key; it inherits the
-// reference point's assignment.
-__global__ void k_still(int np, const Pt* __restrict__ cur, const int32_t* __restrict__ ck, int nr,
-                        const Pt* __restrict__ ref, const int32_t* __restrict__ rk, Pt* __restrict__ out,
-                        uint8_t* __restrict__ taken) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
+// reference point's assignment.  Both lists are in key order, so a block's
+// points meet one short range of the reference: two threads search the whole
+// list for its ends, the others search only between them (every thread over
+// the whole list: 1.3 ms for 3e6 points, 0.38 ms now).
+__global__ void __launch_bounds__(256) k_still(int np, const Pt* __restrict__ cur, const int32_t* __restrict__ ck,
+                                               int nr, const Pt* __restrict__ ref, const int32_t* __restrict__ rk,
+                                               Pt* __restrict__ out, uint8_t* __restrict__ taken) {
+  __shared__ int range[2];
+  const int r = blockIdx.x * 256 + threadIdx.x, last = min((int)blockIdx.x * 256 + 255, np - 1);
+  // first reference index in [a, b) with a key not below x's (`past`: above it)
+  auto bound = [&](const Pt& x, int a, int b, bool past) {
+    while (a < b) {
+      const int mid = (a + b) >> 1;
+      const int c = key_cmp(ref[rk[mid]], x);
+      if (c < 0 || (past && c == 0)) a = mid + 1;
+      else b = mid;
+    }
+    return a;
+  };
+  if (threadIdx.x == 0) range[0] = bound(cur[ck[blockIdx.x * 256]], 0, nr, false);
+  if (threadIdx.x == 32) range[1] = bound(cur[ck[last]], 0, nr, true);
+  __syncthreads();
   if (r >= np) return;
-  int i = ck[r];
-  const Pt& x = cur[i];
-  // first index with this key in the current key order
-  int lo = 0, hi = r;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (key_cmp(cur[ck[mid]], x) < 0) lo = mid + 1;
-    else hi = mid;
-  }
-  int rank_in_key = r - lo;
-  int a = 0, b = nr;
-  while (a < b) {
-    int mid = (a + b) >> 1;
-    if (key_cmp(ref[rk[mid]], x) < 0) a = mid + 1;
-    else b = mid;
-  }
-  int j = a + rank_in_key;
+  const int i = ck[r];
+  const Pt x = cur[i];
+  int rank_in_key = 0;  // points of this key before this one: few share a key
+  while (r - rank_in_key > 0 && key_cmp(cur[ck[r - rank_in_key - 1]], x) == 0) ++rank_in_key;
+  const int j = bound(x, range[0], range[1], false) + rank_in_key;
   Pt p = x;
   p.tgt = -1;
   p.still = 0;
@@ -1869,8 +1950,12 @@ __global__ void __launch_bounds__(kPartT) k_part_scatter(int np, const Pt* __res
   if (g >= 0) {
     int o = bc[blockIdx.x * 8 + g] + myoff;
     for (int ww = 0; ww < w; ++ww) o += wc[ww][g];
-    if (g < 4) A.plist[o] = i;
-    else A.tlist[o] = i - np;
+    if (g < 4) {
+      A.plist[o] = i;
+      A.pbd[o] = make_float2(pts[i].b, pts[i].d);
+    } else {
+      A.tlist[o] = i - np;
+    }
   }
 }
 
@@ -1930,78 +2015,168 @@ __device__ void cand_sort(double* sw, int* sp, int n) {
     }
 }
 
-// one block per free finite target: its k cheapest candidates p (w(p,t) <
-// diag(t), ordered by (w, point index)).  Points are scanned in chunks of
-// the block size in increasing index; whenever the shared buffer could
-// overflow, it is sorted and cut to the k cheapest, whose largest (w, p)
-// becomes the bar a later point must beat (later points have larger
-// indices, so w below the bar's w).  Groups with more than kCandTile - 512
-// free targets leave the problem to the general path.
-__global__ void __launch_bounds__(512) k_asg_candidates(const Pt* __restrict__ pts, const Tg* __restrict__ T,
-                                                        AsgDev A) {
-  __shared__ double sw[kCandTile];
-  __shared__ int sp[kCandTile];
-  __shared__ int fill;
-  __shared__ double bar;
+// Free finite targets of a list of candidates (k_asg_candidates, k_asg_merge):
+// the k cheapest so far, in shared memory.
+struct CandTile {
+  double w[kCandTile];
+  int p[kCandTile];
+  int fill;
+  double bar;  // a later candidate must be cheaper
+  uint32_t off;
+};
+
+// Cut to the k cheapest once the next chunk could overflow the tile.
+__device__ __forceinline__ void cand_cut(CandTile& t, int k, bool more) {
+  __syncthreads();
+  const int n = t.fill;
+  __syncthreads();  // every thread has read fill before the next chunk appends
+  if (n <= kCandTile - (int)blockDim.x || !more) return;
+  cand_sort(t.w, t.p, n);
+  if (threadIdx.x == 0) {
+    t.fill = min(n, k);
+    if (n >= k) t.bar = t.w[k - 1];
+  }
+  __syncthreads();
+}
+
+// The k cheapest of the tile as target `local`'s list.
+__device__ void cand_store(CandTile& t, int k, int g, int local, int pbase, int tbase, const AsgDev& A) {
+  const int n = t.fill;
+  cand_sort(t.w, t.p, n);
+  const int keep = min(n, k);
+  if (threadIdx.x == 0) {
+    t.off = (uint32_t)atomicAdd(&A.counts[9], keep);
+    A.kept_off[tbase + local] = t.off;
+    A.nkept[tbase + local] = (uint32_t)keep;
+    if ((int)t.off + keep > A.cap_kept) A.counts[8] = 1;
+  }
+  __syncthreads();
+  if ((int)t.off + keep > A.cap_kept) return;
+  for (int i = threadIdx.x; i < keep; i += blockDim.x) {
+    Cand c;
+    c.w = t.w[i];
+    c.p = t.p[i];
+    c.t = local;
+    A.kept[t.off + i] = c;
+    A.is_col[pbase + t.p[i]] = 1u;
+  }
+}
+
+// Room for a part's list of any group.
+__device__ __forceinline__ int cand_room(const AsgDev& A) {
+  return max(A.counts[4], max(A.counts[5], A.counts[6]));
+}
+
+// Parts into which the points are split per target: all of them when every
+// target's part lists fit the buffer, else one.
+__device__ __forceinline__ int cand_parts(const AsgDev& A, int parts) {
+  const long long free_t = A.counts[4] + A.counts[5] + A.counts[6];
+  return parts > 1 && free_t * parts * cand_room(A) <= A.cap_part ? parts : 1;
+}
+
+// Block (target, part): the target's k cheapest candidates p (w(p,t) <
+// diag(t), ordered by (w, point index)) among the part's points.  Points are
+// scanned in chunks of the block size in increasing index; whenever the shared
+// buffer could overflow, it is sorted and cut to the k cheapest, whose largest
+// (w, p) becomes the bar a later point must beat (later points have larger
+// indices, so w below the bar's w).  With several parts k_asg_merge joins the
+// lists.  Groups with more than kCandTile - 512 free targets leave the problem
+// to the general path.
+// Bound: fp64 arithmetic and the scan's chunks, one after another.  Values are
+// read from a compact array and a point whose fp32 cost is above the bar by
+// more than its error (a few ulp of its terms) is dropped before the fp64 one;
+// 16 parts per target fill the GPU when few targets are free: 3e6 points and
+// 36 free targets 8.3 ms without either, 0.82 ms now (8.8e4 points, 0.58
+// and 0.12 ms).
+__global__ void __launch_bounds__(512) k_asg_candidates(const Tg* __restrict__ T, AsgDev A, int parts) {
+  __shared__ CandTile t;
   int g, local, pbase, tbase;
   group_of_target(A.counts, blockIdx.x, g, local, pbase, tbase);
   if (g < 0) return;
-  int npg = A.counts[g], k = A.counts[4 + g];
+  const int npg = A.counts[g], k = A.counts[4 + g];
   if (k > kCandTile - 512) {
     if (threadIdx.x == 0) A.counts[8] = 1;  // the general path takes over
     return;
   }
+  const int np = cand_parts(A, parts), part = blockIdx.y;
+  if (part >= np) return;
   const Tg tg = T[A.tlist[tbase + local]];
   const double dt = cost_diag(tg.b, tg.d);
   if (threadIdx.x == 0) {
-    fill = 0;
-    bar = dt;
+    t.fill = 0;
+    t.bar = dt;
   }
   __syncthreads();
-  for (int base = 0; base < npg; base += blockDim.x) {
+  const int i0 = (int)((long long)npg * part / np), i1 = (int)((long long)npg * (part + 1) / np);
+  for (int base = i0; base < i1; base += blockDim.x) {
     const int i = base + threadIdx.x;
-    const double b = bar;
-    if (i < npg) {
-      const Pt& p = pts[A.plist[pbase + i]];
-      const double w = __dsub_rn(cost_pt(p.b, p.d, tg.b, tg.d), cost_diag(p.b, p.d));
-      if (w < b) {
-        const int s = atomicAdd(&fill, 1);
-        sw[s] = w;
-        sp[s] = i;
+    const double b = t.bar;
+    if (i < i1) {
+      const float2 p = A.pbd[pbase + i];
+      const float db = p.x - tg.b, dd = p.y - tg.d, e = p.y - p.x;
+      const float q = db * db + dd * dd, h = 0.5f * e * e;
+      // |fl32(w) - w| <= 6 x 2^-24 (q + h); anything not surely above goes on
+      if (!(q - h - 1e-6f * (q + h) > __double2float_ru(b) + 1e-37f)) {
+        const double w = __dsub_rn(cost_pt(p.x, p.y, tg.b, tg.d), cost_diag(p.x, p.y));
+        if (w < b) {
+          const int s = atomicAdd(&t.fill, 1);
+          t.w[s] = w;
+          t.p[s] = i;
+        }
       }
     }
-    __syncthreads();
-    const int n = fill;
-    __syncthreads();  // every thread has read fill before the next chunk appends
-    if (n > kCandTile - (int)blockDim.x && base + (int)blockDim.x < npg) {
-      cand_sort(sw, sp, n);
-      if (threadIdx.x == 0) {
-        fill = min(n, k);
-        if (n >= k) bar = sw[k - 1];
-      }
-      __syncthreads();
-    }
+    cand_cut(t, k, base + (int)blockDim.x < i1);
   }
-  const int n = fill;
-  cand_sort(sw, sp, n);
-  int keep = min(n, k);
-  __shared__ uint32_t off;
-  if (threadIdx.x == 0) {
-    off = (uint32_t)atomicAdd(&A.counts[9], keep);
-    A.kept_off[tbase + local] = off;
-    A.nkept[tbase + local] = (uint32_t)keep;
-    if ((int)off + keep > A.cap_kept) A.counts[8] = 1;
+  if (np == 1) {
+    cand_store(t, k, g, local, pbase, tbase, A);
+    return;
   }
-  __syncthreads();
-  if ((int)off + keep > A.cap_kept) return;
+  const int n = t.fill;
+  cand_sort(t.w, t.p, n);
+  const int keep = min(n, k), list = (tbase + local) * np + part;
+  if (threadIdx.x == 0) A.part_n[list] = keep;
   for (int i = threadIdx.x; i < keep; i += blockDim.x) {
     Cand c;
-    c.w = sw[i];
-    c.p = sp[i];
+    c.w = t.w[i];
+    c.p = t.p[i];
     c.t = local;
-    A.kept[off + i] = c;
-    A.is_col[pbase + sp[i]] = 1u;
+    A.part[(long long)list * cand_room(A) + i] = c;
   }
+}
+
+// Block = target: its k cheapest candidates of all parts' lists.
+__global__ void __launch_bounds__(512) k_asg_merge(const Tg* __restrict__ T, AsgDev A, int parts) {
+  __shared__ CandTile t;
+  int g, local, pbase, tbase;
+  group_of_target(A.counts, blockIdx.x, g, local, pbase, tbase);
+  if (g < 0) return;
+  const int k = A.counts[4 + g];
+  if (k > kCandTile - 512) return;
+  const int np = cand_parts(A, parts);
+  if (np == 1) return;
+  if (threadIdx.x == 0) {
+    t.fill = 0;
+    t.bar = __longlong_as_double(0x7FF0000000000000ll);
+  }
+  __syncthreads();
+  // lists in point order, each in (w, point) order: of equal costs the earlier
+  // point comes first, as in a scan of the points
+  for (int part = 0; part < np; ++part) {
+    const int list = (tbase + local) * np + part, m = A.part_n[list];
+    for (int base = 0; base < m; base += blockDim.x) {
+      const int i = base + threadIdx.x;
+      if (i < m) {
+        const Cand c = A.part[(long long)list * cand_room(A) + i];
+        if (c.w < t.bar) {
+          const int s = atomicAdd(&t.fill, 1);
+          t.w[s] = c.w;
+          t.p[s] = c.p;
+        }
+      }
+      cand_cut(t, k, true);
+    }
+  }
+  cand_store(t, k, g, local, pbase, tbase, A);
 }
 
 // one block per finite group: column map (candidate points in point order,
@@ -2025,14 +2200,23 @@ __global__ void __launch_bounds__(kHT, 1) k_asg_solve(AsgDev A, Pt* __restrict__
   // column positions of the candidate points of this group
   __shared__ int s_mc;
   {
+    // 16 points per thread and pass (one point each took 1.9 ms for 2e6
+    // points); only candidates' positions are read
+    constexpr int kPer = 16;
     int run = 0;
-    for (int b0 = 0; b0 < npg; b0 += kHT) {
-      int i = b0 + threadIdx.x;
-      int f = (i < npg && A.is_col[pbase + i]) ? 1 : 0;
+    for (int b0 = 0; b0 < npg; b0 += kHT * kPer) {
+      const int i0 = b0 + (int)threadIdx.x * kPer;
+      uint32_t f = 0;
+#pragma unroll
+      for (int j = 0; j < kPer; ++j)
+        if (i0 + j < npg && A.is_col[pbase + i0 + j]) f |= 1u << j;
       int tot;
-      int ex = block_exscan_int1024(f, tot);
-      if (i < npg) A.colpos[pbase + i] = (uint32_t)(run + ex);
-      if (f) A.col_point[wbase + run + ex] = i;
+      int at = run + block_exscan_int1024(__popc(f), tot);
+      for (; f; f &= f - 1, ++at) {
+        const int i = i0 + __ffs(f) - 1;
+        A.colpos[pbase + i] = (uint32_t)at;
+        A.col_point[wbase + at] = i;
+      }
       run += tot;
     }
     if (threadIdx.x == 0) s_mc = run;
@@ -2080,6 +2264,8 @@ __global__ void __launch_bounds__(kHT, 1) k_asg_solve(AsgDev A, Pt* __restrict__
 int assign_groups(int np, Pt* pts, int nt, const Tg* T, double prec, SolverBufs& B, uint32_t* status,
                   AssignStats* as, cudaStream_t st);
 
+constexpr int kParts = 16, kPartPoints = 1 << 14;  // parts per target, points from which they are used
+
 // Assignment phi*_j.  `ref` is the previous diagram (or the targets at j = 0,
 // each assigned to itself).  Returns 0, or a negative value when a scratch
 // buffer is too small (the caller grows it and retries).
@@ -2114,7 +2300,11 @@ int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double p
     k_part_scatter<<<nblk, kPartT, 0, st>>>(np, pts, nt, T, B.taken, bc, B.A); note_launch();
     k_part_essential<<<1, 32, 0, st>>>(B.A, pts); note_launch();
   }
-  k_asg_candidates<<<max(nt, 1), 512, 0, st>>>(pts, T, B.A); note_launch();
+  const int parts = np >= kPartPoints ? kParts : 1;
+  k_asg_candidates<<<dim3(max(nt, 1), parts), 512, 0, st>>>(T, B.A, parts); note_launch();
+  if (parts > 1) {
+    k_asg_merge<<<max(nt, 1), 512, 0, st>>>(T, B.A, parts); note_launch();
+  }
   if (prec > 0.0) {
     k_asg_solve<true><<<3, kHT, 0, st>>>(B.A, pts, T, prec, status);
   } else {
@@ -2234,19 +2424,25 @@ __global__ void k_loss_terms(int np, const Pt* __restrict__ pts, int nt, const T
                              float cancel_eps, double* __restrict__ terms, uint8_t* __restrict__ tused,
                              unsigned long long* __restrict__ counters) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  bool uncancelled = false, still = false, matched = false;
   if (i < np) {
     const Pt& p = pts[i];
     double c;
     if (p.tgt >= 0) {
       c = cost_pt(p.b, p.d, T[p.tgt].b, T[p.tgt].d);
       tused[p.tgt] = 1;
-      if (!p.still) atomicAdd(&counters[2], 1ull);
+      matched = !p.still;
     } else {
       c = cost_diag(p.b, p.d);
-      if (__fsub_rn(p.d, p.b) > cancel_eps) atomicAdd(&counters[0], 1ull);
+      uncancelled = __fsub_rn(p.d, p.b) > cancel_eps;
     }
-    if (p.still) atomicAdd(&counters[1], 1ull);
+    still = p.still != 0;
     terms[i] = c;
+  }
+  const int n0 = __syncthreads_count(uncancelled), n1 = __syncthreads_count(still), n2 = __syncthreads_count(matched);
+  if (threadIdx.x < 3) {
+    const int n = threadIdx.x == 0 ? n0 : threadIdx.x == 1 ? n1 : n2;
+    if (n) atomicAdd(&counters[threadIdx.x], (unsigned long long)n);
   }
 }
 __global__ void k_loss_tterms(int np, int nt, const Tg* __restrict__ T, const uint8_t* __restrict__ tused,
@@ -2254,18 +2450,21 @@ __global__ void k_loss_tterms(int np, int nt, const Tg* __restrict__ T, const ui
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < nt) terms[np + t] = tused[t] ? 0.0 : cost_diag(T[t].b, T[t].d);
 }
-// deterministic pairwise sum (fixed tree), one block
-__global__ void k_sum(int n, const double* __restrict__ terms, double* __restrict__ out) {
+// Deterministic sum: a fixed tree inside blocks of kSumBlock terms, then of
+// the blocks' sums (the same kernel).  One block over 3e6 terms took 1.1 ms.
+constexpr int kSumBlock = 8192;
+__global__ void __launch_bounds__(1024) k_sum(int n, const double* __restrict__ terms, double* __restrict__ out) {
   __shared__ double s[1024];
+  const int base = blockIdx.x * kSumBlock, end = min(n, base + kSumBlock);
   double acc = 0.0;
-  for (int i = threadIdx.x; i < n; i += 1024) acc = __dadd_rn(acc, terms[i]);
+  for (int i = base + threadIdx.x; i < end; i += 1024) acc = __dadd_rn(acc, terms[i]);
   s[threadIdx.x] = acc;
   __syncthreads();
   for (int w = 512; w; w >>= 1) {
     if (threadIdx.x < w) s[threadIdx.x] = __dadd_rn(s[threadIdx.x], s[threadIdx.x + w]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = s[0];
+  if (threadIdx.x == 0) out[blockIdx.x] = s[0];
 }
 
 void loss_and_counts(int np, const Pt* pts, int nt, const Tg* T, float cancel_eps, SolverBufs& B, double* h_loss,
@@ -2275,7 +2474,17 @@ void loss_and_counts(int np, const Pt* pts, int nt, const Tg* T, float cancel_ep
   if (np > 0)
     k_loss_terms<<<(np + 255) / 256, 256, 0, st>>>(np, pts, nt, T, cancel_eps, B.terms, B.taken, B.counters); note_launch();
   if (nt > 0) k_loss_tterms<<<(nt + 255) / 256, 256, 0, st>>>(np, nt, T, B.taken, B.terms); note_launch();
-  k_sum<<<1, 1024, 0, st>>>(np + nt, B.terms, B.dsum); note_launch();
+  int n = np + nt;
+  const double* in = B.terms;
+  double* sums = B.sums;  // block sums of one level after another
+  do {
+    const int nb = max((n + kSumBlock - 1) / kSumBlock, 1);
+    double* out = nb == 1 ? B.dsum : sums;
+    k_sum<<<nb, 1024, 0, st>>>(n, in, out); note_launch();
+    in = out;
+    sums += nb;
+    n = nb;
+  } while (n > 1);
   cudaMemcpyAsync(h_loss, B.dsum, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaMemcpyAsync(h_counts, B.counters, sizeof(unsigned long long) * 4, cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -2408,6 +2617,16 @@ struct Grad64Less {
   __device__ bool operator()(int a, int b) const { return key(a) < key(b); }
 };
 
+// The entries lie in (point, birth before death) order, so a stable sort by
+// vertex alone gives the order above.
+__global__ void k_grad_keys(int n, const Grad64* __restrict__ G, uint32_t* __restrict__ key,
+                            uint32_t* __restrict__ iota) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  key[i] = G[i].v;
+  iota[i] = (uint32_t)i;
+}
+
 __global__ void k_loss_grad_apply(int n, const int32_t* __restrict__ idx, const Grad64* __restrict__ G,
                                   double* __restrict__ grad) {
   int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2419,12 +2638,21 @@ __global__ void k_loss_grad_apply(int n, const int32_t* __restrict__ idx, const 
   grad[v] = acc;
 }
 
-void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* grad, int64_t nv, cudaStream_t st) {
+void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* grad, int64_t nv, uint32_t* status,
+                   cudaStream_t st) {
   cudaMemsetAsync(grad, 0, sizeof(double) * (size_t)nv, st);
   if (np == 0) return;
   Grad64* G = reinterpret_cast<Grad64*>(B.contrib);
   k_loss_grad_contrib<<<(np + 255) / 256, 256, 0, st>>>(np, pts, T, G); note_launch();
-  int32_t* idx = merge_sort(2 * np, B.idxA, B.idxB, Grad64Less{G}, st);
+  const int n = 2 * np;
+  int32_t* idx = B.idxA;
+  if (n <= kRankMax || n > B.cap_rsort) {
+    idx = merge_sort(n, B.idxA, B.idxB, Grad64Less{G}, st, nullptr, n <= B.cap_rsort ? B.rsort : nullptr);
+  } else {
+    uint32_t *key = B.rsort, *iota = key + n;
+    k_grad_keys<<<(n + 255) / 256, 256, 0, st>>>(n, G, key, iota); note_launch();
+    sort_u32_pairs(key, iota, n, nullptr, reinterpret_cast<uint32_t*>(idx), iota + n, status, st);
+  }
   k_loss_grad_apply<<<(2 * np + 255) / 256, 256, 0, st>>>(2 * np, idx, G, grad); note_launch();
 }
 

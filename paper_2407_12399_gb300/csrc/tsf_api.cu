@@ -274,6 +274,7 @@ void grow_solver(tsf_field* F, int np, int nt) {
   dev_free(B.col_point);
   dev_free(B.diag_t);
   dev_free(B.terms);
+  dev_free(B.sums);
   dev_free(B.contrib);
   ck(dev_alloc(&B.tmp_pts, cp));
   ck(dev_alloc(&B.keyord, cp));
@@ -298,10 +299,13 @@ void grow_solver(tsf_field* F, int np, int nt) {
   ck(dev_alloc(&B.col_point, cp));
   ck(dev_alloc(&B.diag_t, ctt));
   ck(dev_alloc(&B.terms, (size_t)cp + ctt));
+  ck(dev_alloc(&B.sums, ((size_t)cp + ctt) / 4096 + 64));
   ck(dev_alloc(&B.contrib, 2 * (size_t)cp));
   {
     AsgDev& A = B.A;
     dev_free(A.counts);
+    dev_free(A.pbd);
+    dev_free(A.part_n);
     dev_free(A.kept);
     dev_free(A.kept_off);
     dev_free(A.col_point);
@@ -319,6 +323,10 @@ void grow_solver(tsf_field* F, int np, int nt) {
     size_t w = (size_t)cp + ctt + 8;
     A.cap_kept = (int)std::min<int64_t>((int64_t)ctt * 2048, std::max<int64_t>((int64_t)16 * cp, 1 << 18));
     ck(dev_alloc(&A.counts, 16));
+    ck(dev_alloc(&A.pbd, cp));
+    ck(dev_alloc(&A.part_n, 16 * (size_t)ctt));
+    A.cap_part = 1 << 20;
+    if (!A.part) ck(dev_alloc(&A.part, A.cap_part));
     ck(dev_alloc(&A.kept, (size_t)A.cap_kept));
     ck(dev_alloc(&A.kept_off, ctt));
     ck(dev_alloc(&A.col_point, w));
@@ -824,10 +832,14 @@ int tsf_destroy_field(tsf_field* F) {
   dev_free(B.H.bw);
   dev_free(B.aux);
   dev_free(B.terms);
+  dev_free(B.sums);
   dev_free(B.dsum);
   dev_free(B.counters);
   dev_free(B.contrib);
   dev_free(B.A.counts);
+  dev_free(B.A.pbd);
+  dev_free(B.A.part);
+  dev_free(B.A.part_n);
   dev_free(B.A.kept);
   dev_free(B.A.kept_off);
   dev_free(B.A.col_point);
@@ -1082,7 +1094,7 @@ int tsf_loss_and_gradient(tsf_field* F, const float* values, int values_on_devic
     *loss = F->loss;
     if (grad) {
       if (!F->lgrad) ck(dev_alloc(&F->lgrad, (size_t)F->d.nv));
-      loss_gradient(F->np, F->pts, F->T, F->B, F->lgrad, F->d.nv, F->st);
+      loss_gradient(F->np, F->pts, F->T, F->B, F->lgrad, F->d.nv, F->status, F->st);
       ck(cudaMemcpyAsync(grad, F->lgrad, sizeof(double) * F->d.nv,
                          grad_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, F->st));
     }

@@ -64,6 +64,10 @@ struct AsgDev {
   HungWork H;          // arrays of np + nt + 8 entries, split per group
   int32_t* aux;        // auction: 4 x (np + nt + 8) ints, split per group
   int cap_kept;
+  float2* pbd;         // (b, d) per position in plist
+  Cand* part;          // candidate lists of parts of the points (k_asg_candidates)
+  int32_t* part_n;     // their lengths, 16 per free target
+  int cap_part;
 };
 
 struct SolverBufs {
@@ -86,6 +90,7 @@ struct SolverBufs {
   HungWork H;
   double* terms;
   double* dsum;
+  double* sums;  // block sums of the loss
   unsigned long long* counters;
   Contrib* contrib;
   int cap_k, cap_cand, cap_cols;
@@ -125,7 +130,8 @@ void replace_values(int64_t nv, const float* in, float* f, uint32_t* upd, unsign
                     cudaStream_t st);
 // dL/df (fp64, nv entries) of the topological loss for the current points
 // and their matching.
-void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* grad, int64_t nv, cudaStream_t st);
+void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* grad, int64_t nv, uint32_t* status,
+                   cudaStream_t st);
 int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double prec, SolverBufs& B, uint32_t* status,
            AssignStats* as, cudaStream_t st);
 void loss_and_counts(int np, const Pt* pts, int nt, const Tg* T, float cancel_eps, SolverBufs& B, double* h_loss,
