@@ -9,23 +9,23 @@
 // The old order's sorted keys (kept from the previous ordering) give the
 // second count by a binary search, even though the updated vertices' old
 // values are gone.
-#include <algorithm>
-#include <atomic>
-
 #include "../../include/tsf.h"
-#include "tsf_group.cuh"
 #include "tsf_kernels.cuh"
 
 namespace tsf {
 
-constexpr int kOT = 1024;  // threads of the one-block kernels
-
-// The old ranks of the updated vertices as a bitmap over positions.
-__global__ void k_order_mark(const uint32_t* __restrict__ upd, int nu, const uint32_t* __restrict__ rank,
-                             uint32_t* __restrict__ ubits) {
+// The old ranks of the updated vertices as a bitmap over positions, and their
+// new keys value_key << 32 | id in K (in the order of upd).
+__global__ void k_order_mark(const uint32_t* __restrict__ upd, int nu, const float* __restrict__ f,
+                             const uint32_t* __restrict__ rank, uint32_t* __restrict__ ubits,
+                             unsigned long long* __restrict__ K, uint32_t* status) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < nu) {
-    uint32_t r = __ldg(rank + upd[q]);
+    const uint32_t u = upd[q];
+    const uint32_t r = __ldg(rank + u);
+    const float x = __ldg(f + u);
+    if (!isfinite(x)) atomicOr(status, kErrNaN);
+    K[q] = ((unsigned long long)value_key(x) << 32) | u;
     atomicOr(ubits + (r >> 5), 1u << (r & 31));
   }
 }
@@ -62,50 +62,56 @@ __global__ void __launch_bounds__(kCntT) k_order_count(const uint32_t* __restric
   if (w < nw) ucnt[w] = wsum[wi] + inc - c;
 }
 
-// One block: boff[b] = set bits in the counting blocks before b, and B = the
-// updated vertices' new keys value_key << 32 | id, ascending (bitonic sort
-// in shared memory).
-__global__ void __launch_bounds__(kOT) k_order_prep(const uint32_t* __restrict__ upd, int nu,
-                                                    const float* __restrict__ f, const uint32_t* __restrict__ btot,
-                                                    int nblk, uint32_t* __restrict__ boff,
-                                                    unsigned long long* __restrict__ B, uint32_t* status) {
-  extern __shared__ __align__(16) unsigned long long sb[];
-  __shared__ uint32_t part[kOT];
-  const int tid = threadIdx.x;
-  const int per = (nblk + kOT - 1) / kOT;
-  const int b0 = tid * per, b1 = b0 + per < nblk ? b0 + per : nblk;
-  uint32_t mine = 0;
-  for (int b = b0; b < b1; ++b) mine += btot[b];
-  part[tid] = mine;
-  __syncthreads();
-  for (int o = 1; o < kOT; o <<= 1) {  // inclusive scan of the runs' totals
-    uint32_t x = tid >= o ? part[tid - o] : 0u;
+// B = K ascending, by rank counting: a block ranks 32 keys, one per lane, and
+// each of its warps counts the smaller ones in its share of K (a broadcast
+// load per step, no dependence between steps).  The keys are distinct, as the
+// vertices are.  The last block also turns the counting blocks' totals into
+// boff[b] = set bits before block b.  Bound by the n^2 comparisons: 6 us for
+// 4096 keys; a bitonic sort by one block took 46 us.
+constexpr int kRankT = 256;
+constexpr int kRankW = kRankT / 32;
+__global__ void __launch_bounds__(kRankT) k_order_rank(const unsigned long long* __restrict__ K, int nu,
+                                                       unsigned long long* __restrict__ B,
+                                                       const uint32_t* __restrict__ btot, int nblk,
+                                                       uint32_t* __restrict__ boff) {
+  __shared__ int cnt[kRankW][32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (blockIdx.x == gridDim.x - 1) {
+    uint32_t* part = reinterpret_cast<uint32_t*>(&cnt[0][0]);
+    const int per = (nblk + kRankT - 1) / kRankT;
+    const int b0 = min(tid * per, nblk), b1 = min(b0 + per, nblk);
+    uint32_t mine = 0;
+    for (int b = b0; b < b1; ++b) mine += btot[b];
+    part[tid] = mine;
     __syncthreads();
-    part[tid] += x;
-    __syncthreads();
-  }
-  uint32_t run = part[tid] - mine;
-  for (int b = b0; b < b1; ++b) {
-    boff[b] = run;
-    run += btot[b];
-  }
-  int n2 = 1;
-  while (n2 < nu) n2 <<= 1;
-  bool bad = false;
-  for (int i = tid; i < n2; i += kOT) {
-    unsigned long long k = 0ull;
-    if (i < nu) {
-      uint32_t u = upd[i];
-      float x = __ldg(f + u);
-      bad |= !isfinite(x);
-      k = ((unsigned long long)value_key(x) << 32) | u;
+    for (int o = 1; o < kRankT; o <<= 1) {  // inclusive scan of the runs' totals
+      const uint32_t x = tid >= o ? part[tid - o] : 0u;
+      __syncthreads();
+      part[tid] += x;
+      __syncthreads();
     }
-    sb[i] = k;
+    uint32_t run = part[tid] - mine;
+    for (int b = b0; b < b1; ++b) {
+      boff[b] = run;
+      run += btot[b];
+    }
+    return;
   }
-  if (bad) atomicOr(status, kErrNaN);
+  const int q = blockIdx.x * 32 + lane;
+  const unsigned long long k = q < nu ? __ldg(K + q) : 0ull;
+  const int per = (nu + kRankW - 1) / kRankW;
+  const int j1 = min((w + 1) * per, nu);
+  int c = 0;
+#pragma unroll 8
+  for (int j = w * per; j < j1; ++j) c += __ldg(K + j) < k ? 1 : 0;
+  cnt[w][lane] = c;
   __syncthreads();
-  group_sort_desc<kOT>(sb, n2);  // keys are > 0, the padding sorts last
-  for (int i = tid; i < nu; i += kOT) B[i] = sb[nu - 1 - i];
+  if (w == 0 && q < nu) {
+    c = 0;
+#pragma unroll
+    for (int i = 0; i < kRankW; ++i) c += cnt[i][lane];
+    B[c] = k;
+  }
 }
 
 __device__ __forceinline__ int count_below(const unsigned long long* __restrict__ s, int n, unsigned long long x) {
@@ -127,18 +133,40 @@ __device__ __forceinline__ int updated_below(const uint32_t* __restrict__ ubits,
 constexpr int kKeepT = 256, kKeepC = 16;  // threads, positions per lane
 constexpr int kKeepTile = kKeepT * kKeepC;
 
-// The kept vertices: each lane walks old positions i0, i0 + 32, ... and
-// advances its count of smaller new keys (non-decreasing in i).
-__global__ void __launch_bounds__(kKeepT) k_order_keep(int64_t n, const uint32_t* __restrict__ order,
-                                                       const uint32_t* __restrict__ skey,
-                                                       const uint32_t* __restrict__ ubits,
-                                                       const uint32_t* __restrict__ ucnt,
-                                                       const uint32_t* __restrict__ boff, int nu,
-                                                       const unsigned long long* __restrict__ B,
-                                                       uint32_t* __restrict__ order2, uint32_t* __restrict__ skey2,
-                                                       uint32_t* __restrict__ rank) {
+// The new order.  The first blocks place the updated vertices, one thread
+// each (a binary search of the old order, latency bound: it runs beside the
+// copy below); in the others each lane walks kept positions i0, i0 + 32, ...
+// and advances its count of smaller new keys (non-decreasing in i).
+__global__ void __launch_bounds__(kKeepT) k_order_place(int64_t n, const uint32_t* __restrict__ order,
+                                                        const uint32_t* __restrict__ skey,
+                                                        const uint32_t* __restrict__ ubits,
+                                                        const uint32_t* __restrict__ ucnt,
+                                                        const uint32_t* __restrict__ boff, int nu,
+                                                        const unsigned long long* __restrict__ B,
+                                                        uint32_t* __restrict__ order2, uint32_t* __restrict__ skey2,
+                                                        uint32_t* __restrict__ rank) {
+  const int moved_blocks = (nu + kKeepT - 1) / kKeepT;
+  if ((int)blockIdx.x < moved_blocks) {
+    const int q = blockIdx.x * kKeepT + threadIdx.x;
+    if (q >= nu) return;
+    const unsigned long long key = B[q];
+    int64_t lo = 0, hi = n;  // old positions whose (old key, id) is below key
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      const unsigned long long k = ((unsigned long long)__ldg(skey + mid) << 32) | __ldg(order + mid);
+      if (k < key) lo = mid + 1;
+      else hi = mid;
+    }
+    const int la = lo < n ? updated_below(ubits, ucnt, boff, lo) : nu;
+    const uint32_t ni = (uint32_t)(q + lo - la);
+    const uint32_t u = (uint32_t)key;
+    order2[ni] = u;
+    skey2[ni] = (uint32_t)(key >> 32);
+    rank[u] = ni;
+    return;
+  }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t i0 = (int64_t)blockIdx.x * kKeepTile + (int64_t)w * (32 * kKeepC) + lane;
+  const int64_t i0 = (int64_t)(blockIdx.x - moved_blocks) * kKeepTile + (int64_t)w * (32 * kKeepC) + lane;
   if (i0 >= n) return;
   int b = count_below(B, nu, ((unsigned long long)__ldg(skey + i0) << 32) | __ldg(order + i0));
 #pragma unroll 4
@@ -147,7 +175,7 @@ __global__ void __launch_bounds__(kKeepT) k_order_keep(int64_t n, const uint32_t
     if (i >= n) break;
     uint32_t v = __ldg(order + i);
     uint32_t kk = __ldg(skey + i);
-    if ((__ldg(ubits + (i >> 5)) >> (i & 31)) & 1u) continue;  // updated: placed by k_order_moved
+    if ((__ldg(ubits + (i >> 5)) >> (i & 31)) & 1u) continue;  // updated: placed by its own thread
     unsigned long long key = ((unsigned long long)kk << 32) | v;
     while (b < nu && __ldg(B + b) < key) ++b;
     uint32_t ni = (uint32_t)(i - updated_below(ubits, ucnt, boff, i) + b);
@@ -155,30 +183,6 @@ __global__ void __launch_bounds__(kKeepT) k_order_keep(int64_t n, const uint32_t
     skey2[ni] = kk;
     rank[v] = ni;
   }
-}
-
-// The updated vertices, one thread each.
-__global__ void k_order_moved(int64_t n, const uint32_t* __restrict__ order, const uint32_t* __restrict__ skey,
-                              const uint32_t* __restrict__ ubits, const uint32_t* __restrict__ ucnt,
-                              const uint32_t* __restrict__ boff, int nu, const unsigned long long* __restrict__ B,
-                              uint32_t* __restrict__ order2,
-                              uint32_t* __restrict__ skey2, uint32_t* __restrict__ rank) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nu) return;
-  unsigned long long key = B[q];
-  int64_t lo = 0, hi = n;  // old positions whose (old key, id) is below key
-  while (lo < hi) {
-    int64_t mid = (lo + hi) >> 1;
-    unsigned long long k = ((unsigned long long)__ldg(skey + mid) << 32) | __ldg(order + mid);
-    if (k < key) lo = mid + 1;
-    else hi = mid;
-  }
-  int la = lo < n ? updated_below(ubits, ucnt, boff, lo) : nu;
-  uint32_t ni = (uint32_t)(q + lo - la);
-  uint32_t u = (uint32_t)key;
-  order2[ni] = u;
-  skey2[ni] = (uint32_t)(key >> 32);
-  rank[u] = ni;
 }
 
 void vertex_order_incremental(const float* f, int64_t n, const uint32_t* upd, int nu, const uint32_t* order,
@@ -190,21 +194,13 @@ void vertex_order_incremental(const float* f, int64_t n, const uint32_t* upd, in
   const int nblk = (int)((nw + kCntT - 1) / kCntT);
   uint32_t* btot = ucnt + nw;  // ucnt holds nw + 2 * nblk words
   uint32_t* boff = btot + nblk;
-  const size_t smem = sizeof(unsigned long long) * (size_t)kIncOrderMax;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  static std::atomic<bool> attr[64] = {};  // fields may be driven from several host threads
-  if (dev >= 0 && dev < 64 && !attr[dev].load(std::memory_order_acquire)) {
-    cudaFuncSetAttribute(k_order_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr[dev].store(true, std::memory_order_release);
-  }
+  unsigned long long* K = B + kIncOrderMax;
   cudaMemsetAsync(ubits, 0, sizeof(uint32_t) * (size_t)nw, st);
-  k_order_mark<<<(nu + 255) / 256, 256, 0, st>>>(upd, nu, rank, ubits); note_launch();
+  k_order_mark<<<(nu + 255) / 256, 256, 0, st>>>(upd, nu, f, rank, ubits, K, status); note_launch();
   k_order_count<<<nblk, kCntT, 0, st>>>(ubits, nw, ucnt, btot); note_launch();
-  k_order_prep<<<1, kOT, smem, st>>>(upd, nu, f, btot, nblk, boff, B, status); note_launch();
-  k_order_keep<<<(unsigned)((n + kKeepTile - 1) / kKeepTile), kKeepT, 0, st>>>(n, order, skey, ubits, ucnt, boff, nu,
-                                                                              B, order2, skey2, rank); note_launch();
-  k_order_moved<<<(nu + 255) / 256, 256, 0, st>>>(n, order, skey, ubits, ucnt, boff, nu, B, order2, skey2, rank);
+  k_order_rank<<<(nu + 31) / 32 + 1, kRankT, 0, st>>>(K, nu, B, btot, nblk, boff); note_launch();
+  const int64_t place = (nu + kKeepT - 1) / kKeepT + (n + kKeepTile - 1) / kKeepTile;
+  k_order_place<<<(unsigned)place, kKeepT, 0, st>>>(n, order, skey, ubits, ucnt, boff, nu, B, order2, skey2, rank);
   note_launch();
 }
 

@@ -456,7 +456,10 @@ int compute_diagram(tsf_field* F, bool incremental) {
   stage_end(F, kGrad);
   F->records_valid = true;
   stage_begin(F, kCrit);
-  launch_crit_count(F->d, F->order, F->rec, F->tile_counts, F->totals, st);
+  // the critical cells of each position, packed; the list of recomputed stars
+  // is done with
+  uint16_t* pack = reinterpret_cast<uint16_t*>(F->glist);
+  launch_crit_count(F->d, F->order, F->rec, pack, F->tile_counts, F->totals, st);
   int4 tot;
   uint32_t s = 0;
   ck(cudaMemcpyAsync(&tot, F->totals, sizeof(int4), cudaMemcpyDeviceToHost, st));
@@ -474,8 +477,7 @@ int compute_diagram(tsf_field* F, bool incremental) {
   F->n2 = tot.z;
   F->n3 = tot.w;
   grow_crit(F, F->n0, F->n1, F->n2, F->n3);
-  launch_crit_write(F->d, F->order, F->rank, F->rec, F->tile_counts, F->L, F->cidx, F->c1base, F->c2base, F->status,
-                    st);
+  launch_crit_write(F->d, F->order, F->rank, F->rec, pack, F->tile_counts, F->L, F->cidx, F->c1base, F->c2base, st);
   stage_end(F, kCrit);
   stage_begin(F, kD0);
   launch_d0(F->d, F->nd, F->L, F->n0, F->n1, F->vnext8, F->cidx, F->PS, F->PO, F->status, st);
@@ -890,7 +892,7 @@ int tsf_create_field(int lx, int ly, int lz, const float* values, int values_on_
     ck(dev_alloc(&F->skey2, nv));
     ck(dev_alloc(&F->ubits, (size_t)(nv / 32 + 1)));
     ck(dev_alloc(&F->ucnt, (size_t)order_count_words(nv)));
-    ck(dev_alloc(&F->ordB, kIncOrderMax));
+    ck(dev_alloc(&F->ordB, 2 * (size_t)kIncOrderMax));
     ck(dev_alloc(&F->rec, nv));
     ck(dev_alloc(&F->tab, nv));
     ck(dev_alloc(&F->vnext8, nv));

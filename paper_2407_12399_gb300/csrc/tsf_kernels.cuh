@@ -71,7 +71,7 @@ void vertex_order(const float* f, int64_t n, uint32_t* order, uint32_t* rank, ui
 constexpr int kIncOrderMax = 8192;
 // New order2/skey2/rank from the old order/skey/rank and the nu vertices upd[]
 // whose values changed.  Scratch: ubits (n/32 + 1 words), ucnt
-// (order_count_words(n) words), B (kIncOrderMax double words).
+// (order_count_words(n) words), B (2 kIncOrderMax double words).
 void vertex_order_incremental(const float* f, int64_t n, const uint32_t* upd, int nu, const uint32_t* order,
                               const uint32_t* skey, uint32_t* order2, uint32_t* skey2, uint32_t* rank,
                               uint32_t* ubits, uint32_t* ucnt, unsigned long long* B, uint32_t* status,
@@ -88,11 +88,13 @@ void launch_gradient_incremental(const Dims& d, const uint32_t* rank, const floa
                                  uint32_t* mark, uint32_t gen, uint32_t* list, unsigned long long* count, Rec* rec,
                                  uint8_t* vnext8, D1Tab* tab, uint32_t* status, cudaStream_t st);
 int crit_tiles(int64_t nv);
-void launch_crit_count(const Dims& d, const uint32_t* order, const Rec* rec, int4* tile_counts, int4* totals,
-                       cudaStream_t st);
+// pack (n words of 16 bits): each position's critical cells, from the count for
+// the write.
+void launch_crit_count(const Dims& d, const uint32_t* order, const Rec* rec, uint16_t* pack, int4* tile_counts,
+                       int4* totals, cudaStream_t st);
 void launch_crit_write(const Dims& d, const uint32_t* order, const uint32_t* rank, const Rec* rec,
-                       const int4* tile_off, const CritLists& L, uint32_t* cidx, uint32_t* c1base, uint32_t* c2base,
-                       uint32_t* status, cudaStream_t st);
+                       const uint16_t* pack, const int4* tile_off, const CritLists& L, uint32_t* cidx,
+                       uint32_t* c1base, uint32_t* c2base, cudaStream_t st);
 void launch_zero_pairs(const Dims& d, const uint32_t* rank, unsigned long long* out, int64_t cap,
                        unsigned long long* count, uint32_t* status, cudaStream_t st);
 
