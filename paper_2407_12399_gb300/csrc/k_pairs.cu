@@ -119,26 +119,6 @@ __device__ __forceinline__ void uf_clear(int64_t t, int64_t threads, int nn, Pai
   }
 }
 
-// One thread per endpoint of each critical edge; also clears the union-find.
-__global__ void k_d0_trace(int n1, int n0, int64_t nv, CritLists L, const uint8_t* __restrict__ vnext8,
-                           const uint32_t* __restrict__ cidx, NbrDelta nd, PairScratch S, PairOut P,
-                           uint32_t* status) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uf_clear(t, (int64_t)gridDim.x * blockDim.x, n0, S);
-  if (t >= 2 * (int64_t)n1) return;
-  uint32_t vn = L.c1_vn[t >> 1];
-  uint32_t v = vn >> 4;
-  if (!(t & 1)) {
-    P.d0_min[t >> 1] = -1;
-    P.d0_killed[t >> 1] = 0;
-    P.d0mask[v] = 0u;
-  }
-  if (t & 1) v = (uint32_t)((int32_t)v + nd.d[vn & 15u]);
-  int32_t a = trace_down(v, vnext8, cidx, nd, nv);
-  if (a < 0) atomicOr(status, kErrTrace);
-  S.ends[t] = a < 0 ? 0 : a;
-}
-
 __device__ __forceinline__ Rec ld_rec(const Rec* rec, uint32_t v) {
   const uint4* p = reinterpret_cast<const uint4*>(rec + v);
   uint4 a = __ldg(p), b = __ldg(p + 1);
@@ -148,46 +128,87 @@ __device__ __forceinline__ Rec ld_rec(const Rec* rec, uint32_t v) {
   return r;
 }
 
+// The integral lines of both stages run in one launch (the stages do not
+// depend on each other and each is bound by its longest lines), D2's first as
+// they take longer.  Both stages, one after the other with D2's walk holding a
+// whole record in local memory / now: 0.266 / 0.097 ms for the 128^3 filament
+// field, 0.59 / 0.23 for the 97 x 61 x 130 field, 3.69 / 1.26 for a 256^3 one.
+struct TraceArgs {
+  Dims d;
+  NbrDelta nd;
+  CritLists L;
+  int n0, n1, n2, n3;
+  const uint32_t* rank;
+  const Rec* rec;
+  const uint8_t* vnext8;
+  const uint32_t* cidx;
+  PairScratch S0, S2;
+  PairOut P;
+};
+constexpr int kTraceT = 128;
+
+// D0: one thread per endpoint of each critical edge; also clears the
+// union-find.
+__device__ void d0_trace(const TraceArgs& A, int64_t t, int64_t threads, uint32_t* status) {
+  uf_clear(t, threads, A.n0, A.S0);
+  if (t >= 2 * (int64_t)A.n1) return;
+  uint32_t vn = A.L.c1_vn[t >> 1];
+  uint32_t v = vn >> 4;
+  if (!(t & 1)) {
+    A.P.d0_min[t >> 1] = -1;
+    A.P.d0_killed[t >> 1] = 0;
+    A.P.d0mask[v] = 0u;
+  }
+  if (t & 1) v = (uint32_t)((int32_t)v + A.nd.d[vn & 15u]);
+  int32_t a = trace_down(v, A.vnext8, A.cidx, A.nd, A.d.nv);
+  if (a < 0) atomicOr(status, kErrTrace);
+  A.S0.ends[t] = a < 0 ? 0 : a;
+}
+
+// Code of tetrahedron tau in a record in memory: the two words that hold its
+// seven bits (rec_tet_code of the whole record, whose words a run-time index
+// would send through local memory).
+__device__ __forceinline__ int ld_tet_code(const Rec* __restrict__ rec, uint32_t w, int tau) {
+  const int off = 56 + 7 * tau;
+  const uint32_t* p = rec[w].w + (off >> 5);  // off <= 217: word 7 is the last
+  return (int)(__funnelshift_r(__ldg(p), __ldg(p + 1), off & 31) & 127u);
+}
+
 // Ascending integral line in the dual: from tetrahedron (w, tau) follow the
 // record codes to a maximum (its index) or to the outside (returns n3).
+// Bound: one dependent L2 or memory access per star crossed, the steps inside
+// a star hit L1.
 __device__ int32_t trace_up(uint32_t w, int tau, const Rec* __restrict__ rec, const uint32_t* __restrict__ cidx,
                             const int32_t* nd, int n3, const UpStep* up, int64_t nv) {
-  Rec r = ld_rec(rec, w);
   for (int64_t s = 0; s <= 25 * nv; ++s) {
-    int code = rec_tet_code(r, tau);
-    if (code == kCodeMax) return (int32_t)cidx[w];
-    if (code == kCodeOut) return n3;
+    const int code = ld_tet_code(rec, w, tau);
     if (code < 24) {
       tau = code;
       continue;
     }
-    if (code >= 96) return -1;
-    UpStep u = up[code - 24];
+    if (code >= 96) return code == kCodeMax ? (int32_t)cidx[w] : code == kCodeOut ? n3 : -1;
+    const UpStep u = up[code - 24];
     tau = u.tau;
     w = (uint32_t)((int32_t)w + nd[u.c]);
-    r = ld_rec(rec, w);
   }
   return -1;
 }
 
-// One thread per (critical triangle, side): the ascending dual line from the
-// tetrahedron on that side to a maximum or the outside.  Also clears the
+// D2: one thread per (critical triangle, side): the ascending dual line from
+// the tetrahedron on that side to a maximum or the outside.  Also clears the
 // union-find.
-__global__ void k_d2_trace(Dims d, int n2, int n3, CritLists L, const uint32_t* __restrict__ rank,
-                           const Rec* __restrict__ rec, const uint32_t* __restrict__ cidx, NbrDelta nd,
-                           PairScratch S, int32_t* __restrict__ d2_max, uint32_t* status) {
-  __shared__ UpStep sup[72];
-  __shared__ int32_t snd[14];
-  if (threadIdx.x < 14) snd[threadIdx.x] = nd.d[threadIdx.x];
-  if (threadIdx.x < 72) sup[threadIdx.x] = c_up.s[threadIdx.x];
-  __syncthreads();
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uf_clear(tt, (int64_t)gridDim.x * blockDim.x, n3 + 1, S);
-  if (tt >= 2 * (int64_t)n2) return;
+__device__ void d2_trace(const TraceArgs& A, int64_t tt, int64_t threads, const int32_t* snd, const UpStep* sup,
+                         uint32_t* status) {
+  const Dims& d = A.d;
+  const int n3 = A.n3;
+  const Rec* __restrict__ rec = A.rec;
+  const uint32_t* __restrict__ cidx = A.cidx;
+  uf_clear(tt, threads, n3 + 1, A.S2);
+  if (tt >= 2 * (int64_t)A.n2) return;
   int i = (int)(tt >> 1), k = (int)(tt & 1);
-  if (!k) d2_max[i] = -1;
+  if (!k) A.P.d2_max[i] = -1;
   const Geo& G = c_geo;
-  uint32_t ve = L.c2_ve[i];
+  uint32_t ve = A.L.c2_ve[i];
   uint32_t v = ve >> 6;
   int e = (int)(ve & 63u);
   int a = G.edge[e][0], b = G.edge[e][1];
@@ -203,7 +224,7 @@ __global__ void k_d2_trace(Dims d, int n2, int n3, CritLists L, const uint32_t* 
     res = n3;
   } else {
     uint32_t wc = vid(d, nx, ny, nz);
-    if (rank[wc] < rank[v]) {
+    if (__ldg(A.rank + wc) < __ldg(A.rank + v)) {
       res = trace_up(v, t, rec, cidx, snd, n3, sup, d.nv);
     } else {
       int i0 = nbr_index(G, -G.off[c][0], -G.off[c][1], -G.off[c][2]);
@@ -217,7 +238,22 @@ __global__ void k_d2_trace(Dims d, int n2, int n3, CritLists L, const uint32_t* 
     atomicOr(status, kErrTrace);
     res = n3;
   }
-  S.ends[tt] = res;
+  A.S2.ends[tt] = res;
+}
+
+__global__ void __launch_bounds__(kTraceT) k_traces(const __grid_constant__ TraceArgs A, unsigned blocks2,
+                                                    uint32_t* status) {
+  __shared__ UpStep sup[72];
+  __shared__ int32_t snd[14];
+  if (blockIdx.x < blocks2) {
+    if (threadIdx.x < 14) snd[threadIdx.x] = A.nd.d[threadIdx.x];
+    if (threadIdx.x < 72) sup[threadIdx.x] = c_up.s[threadIdx.x];
+    __syncthreads();
+    d2_trace(A, (int64_t)blockIdx.x * kTraceT + threadIdx.x, (int64_t)blocks2 * kTraceT, snd, sup, status);
+  } else {
+    d0_trace(A, (int64_t)(blockIdx.x - blocks2) * kTraceT + threadIdx.x,
+             (int64_t)(gridDim.x - blocks2) * kTraceT, status);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -240,7 +276,7 @@ __global__ void k_d2_trace(Dims d, int n2, int n3, CritLists L, const uint32_t* 
 // Bound: dependent L2 round trips along the deepest walk.  Rounds of
 // reservations (one block, or the whole GPU behind barriers) took 0.34 ms for
 // stage D0 of the 97 x 61 x 130 field and 1.42 ms for a 256^3 one, now 0.14
-// and 0.75 ms (traces included).
+// and 0.75 ms (traces included, each stage on its own).
 __device__ __forceinline__ unsigned long long uf_word(int pr, int node) {
   return ((unsigned long long)(uint32_t)pr << 32) | (uint32_t)node;
 }
@@ -266,13 +302,25 @@ __device__ __forceinline__ int uf_walk(const PairScratch& S, int x, int pr, int 
   return x;
 }
 
-// n items (priority i, or n-1-i when `reverse`), nn nodes.  Younger node =
-// larger index (reverse = false) or smaller index (reverse = true).
-__global__ void __launch_bounds__(256) k_uf_items(int n, int nn, bool reverse, PairScratch S, int limit,
-                                                  uint32_t* status) {
-  const int threads = gridDim.x * blockDim.x;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += threads) {  // in priority order
-    const int i = reverse ? n - 1 - t : t;
+// n items (priority i, or n-1-i for D2), nn nodes.  Younger node = larger
+// index (D0) or smaller index (D2).  No blocks and no nodes: nothing to do.
+struct UfSide {
+  int n, nn;
+  unsigned blocks;  // of k_uf_items
+  PairScratch S;
+  int32_t* kill;
+};
+
+// Both stages in one launch, D2's blocks first.
+__global__ void __launch_bounds__(256) k_uf_items(const __grid_constant__ UfSide U2, const __grid_constant__ UfSide U0,
+                                                  int limit, uint32_t* status) {
+  const bool two = blockIdx.x < U2.blocks;
+  const UfSide& U = two ? U2 : U0;
+  const PairScratch S = U.S;
+  const int n = U.n, nn = U.nn;
+  const int threads = U.blocks * 256;
+  for (int t = (blockIdx.x - (two ? 0u : U2.blocks)) * 256 + threadIdx.x; t < n; t += threads) {  // in priority order
+    const int i = two ? n - 1 - t : t;
     int pr = t, a = S.ends[2 * i], b = S.ends[2 * i + 1];
     for (int step = 0;; ++step) {
       if (step >= limit) {
@@ -282,7 +330,7 @@ __global__ void __launch_bounds__(256) k_uf_items(int n, int nn, bool reverse, P
       a = uf_walk(S, a, pr, nn);
       b = uf_walk(S, b, pr, nn);
       if (a == b) break;  // closes a cycle
-      const int young = reverse ? min(a, b) : max(a, b), old = a + b - young;
+      const int young = two ? min(a, b) : max(a, b), old = a + b - young;
       const unsigned long long was = atomicMin(S.rec + young, uf_word(pr, old));
       if (was == kUfNone) break;
       const int wp = (int)(was >> 32);
@@ -293,16 +341,19 @@ __global__ void __launch_bounds__(256) k_uf_items(int n, int nn, bool reverse, P
   }
 }
 
-// kill[i] = node killed by item i; with d0 set also the marks of killed edges.
-__global__ void k_uf_kills(int n, int nn, bool reverse, PairScratch S, int32_t* __restrict__ kill, bool d0, CritLists L,
-                           PairOut P) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= nn) return;
-  const unsigned long long r = S.rec[x];
+// kill[i] = node killed by item i; for D0 also the marks of killed edges.
+__global__ void __launch_bounds__(256) k_uf_kills(const __grid_constant__ UfSide U2, const __grid_constant__ UfSide U0,
+                                                  CritLists L, PairOut P) {
+  const unsigned blocks2 = (unsigned)(U2.nn + 255) / 256;
+  const bool two = blockIdx.x < blocks2;
+  const UfSide& U = two ? U2 : U0;
+  const int x = (blockIdx.x - (two ? 0u : blocks2)) * 256 + threadIdx.x;
+  if (x >= U.nn) return;
+  const unsigned long long r = U.S.rec[x];
   if (r == kUfNone) return;
-  const int pr = (int)(r >> 32), i = reverse ? n - 1 - pr : pr;
-  kill[i] = x;
-  if (d0) {
+  const int pr = (int)(r >> 32), i = two ? U.n - 1 - pr : pr;
+  U.kill[i] = x;
+  if (!two) {
     P.d0_killed[i] = 1;
     const uint32_t vn = L.c1_vn[i];
     atomicOr(&P.d0mask[vn >> 4], 1u << (vn & 15u));
@@ -311,7 +362,7 @@ __global__ void k_uf_kills(int n, int nn, bool reverse, PairScratch S, int32_t* 
 
 // Threads in flight: enough to hide the round trips, few enough that the items
 // run nearly in priority order (an item far ahead claims lows that earlier
-// items take back).  Stages D0 and D2 of the 97 x 61 x 130 field (8e4 items):
+// items take back).  Stages D0 and D2, each on its own with its traces, of the 97 x 61 x 130 field (8e4 items):
 // 0.29 and 0.44 ms with 2^12 threads, 0.14 and 0.37 with 2^14, 0.19 and 0.45
 // with 2^16; of a 256^3 field (2.6e6 items): 1.58 and 3.75 ms with 2^14, 0.75
 // and 2.95 with 2^16, 0.76 and 3.02 with all.
@@ -323,25 +374,23 @@ static int uf_limit() {
   return (int)(cap > 0 ? std::min(limit, cap) : limit);
 }
 
-void launch_d0(const Dims& d, const NbrDelta& nd, const CritLists& L, int n0, int n1, const uint8_t* vnext8,
-               const uint32_t* cidx, PairScratch& S, PairOut& P, uint32_t* status, cudaStream_t st) {
-  if (n1 > 0) {
-    k_d0_trace<<<(unsigned)((2 * (int64_t)n1 + 255) / 256), 256, 0, st>>>(n1, n0, d.nv, L, vnext8, cidx, nd, S, P,
-                                                                         status); note_launch();
-    k_uf_items<<<uf_blocks(n1), 256, 0, st>>>(n1, n0, false, S, uf_limit(), status); note_launch();
-    k_uf_kills<<<(n0 + 255) / 256, 256, 0, st>>>(n1, n0, false, S, P.d0_min, true, L, P); note_launch();
-  }
+void launch_traces(const Dims& d, const NbrDelta& nd, const CritLists& L, int n0, int n1, int n2, int n3,
+                   const uint32_t* rank, const Rec* rec, const uint8_t* vnext8, const uint32_t* cidx, PairScratch& S0,
+                   PairScratch& S2, PairOut& P, uint32_t* status, cudaStream_t st) {
+  const TraceArgs A{d, nd, L, n0, n1, n2, n3, rank, rec, vnext8, cidx, S0, S2, P};
+  const unsigned b2 = (unsigned)((2 * (int64_t)n2 + kTraceT - 1) / kTraceT);
+  const unsigned b0 = (unsigned)((2 * (int64_t)n1 + kTraceT - 1) / kTraceT);
+  if (b0 + b2 == 0) return;
+  k_traces<<<b2 + b0, kTraceT, 0, st>>>(A, b2, status); note_launch();
 }
 
-void launch_d2(const Dims& d, const NbrDelta& nd, const CritLists& L, int n2, int n3, const uint32_t* rank,
-               const Rec* rec, const uint32_t* cidx, PairScratch& S, PairOut& P, uint32_t* status,
-               cudaStream_t st) {
-  if (n2 > 0) {
-    k_d2_trace<<<(unsigned)((2 * (int64_t)n2 + 127) / 128), 128, 0, st>>>(d, n2, n3, L, rank, rec, cidx, nd, S,
-                                                                         P.d2_max, status); note_launch();
-    k_uf_items<<<uf_blocks(n2), 256, 0, st>>>(n2, n3 + 1, true, S, uf_limit(), status); note_launch();
-    k_uf_kills<<<(n3 + 256) / 256, 256, 0, st>>>(n2, n3 + 1, true, S, P.d2_max, false, L, P); note_launch();
-  }
+void launch_union_find(const CritLists& L, int n0, int n1, int n2, int n3, PairScratch& S0, PairScratch& S2,
+                       PairOut& P, uint32_t* status, cudaStream_t st) {
+  if (n1 == 0 && n2 == 0) return;
+  const UfSide U2{n2, n2 ? n3 + 1 : 0, (unsigned)uf_blocks(n2), S2, P.d2_max};
+  const UfSide U0{n1, n1 ? n0 : 0, (unsigned)uf_blocks(n1), S0, P.d0_min};
+  k_uf_items<<<U2.blocks + U0.blocks, 256, 0, st>>>(U2, U0, uf_limit(), status); note_launch();
+  k_uf_kills<<<(U2.nn + 255) / 256 + (U0.nn + 255) / 256, 256, 0, st>>>(U2, U0, L, P); note_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -495,6 +544,46 @@ __global__ void k_d1_gather(int n2, const uint32_t* __restrict__ flag, const uin
     if (flag[i]) cols[pos[i]] = i;
     if (i == n2 - 1) *ncols = (int32_t)(pos[i] + flag[i]);
   }
+}
+
+// The same by one block, for up to kSelectOne triangles (four launches less:
+// 22 us before on 2e3 triangles).
+constexpr int kSelectT = 1024, kSelectOne = 8 * kSelectT;
+__global__ void __launch_bounds__(kSelectT) k_d1_select_one(int n2, const int32_t* __restrict__ d2_max,
+                                                            int32_t* __restrict__ cols, int32_t* __restrict__ d1_edge,
+                                                            int32_t* __restrict__ ncols) {
+  __shared__ int wsum[kSelectT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int per = (n2 + kSelectT - 1) / kSelectT;
+  const int i0 = min(tid * per, n2), i1 = min(i0 + per, n2);
+  uint32_t keep = 0;
+  for (int i = i0; i < i1; ++i) {
+    d1_edge[i] = -1;
+    if (d2_max[i] < 0) keep |= 1u << (i - i0);
+  }
+  const int c = __popc(keep);
+  int inc = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  if (lane == 31) wsum[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    const int x = wsum[lane];
+    int xi = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, xi, o);
+      if (lane >= o) xi += y;
+    }
+    wsum[lane] = xi - x;
+    if (lane == 31) *ncols = xi;
+  }
+  __syncthreads();
+  int at = wsum[w] + inc - c;
+  for (; keep; keep &= keep - 1) cols[at++] = i0 + __ffs((int)keep) - 1;
 }
 
 // Growable array in the pool (a column's heap or its Morse boundary).
@@ -825,6 +914,12 @@ constexpr int kOutCap = 28;
 constexpr int kLargeD1 = 1 << 19;
 constexpr int kChainLarge = 1, kRoundsLarge = 128;  // defaults of knobs 10 and 11, large diagrams
 constexpr int kChainSmall = 2, kRoundsSmall = 16;   // ... small diagrams
+// Below 2^13 critical triangles every column can have its block at once, so
+// phase A only keeps the columns that end after a few rounds.  Stage time at
+// 4 / 16 rounds: 0.101 / 0.155 ms for a 32^3 field (3.5e3 triangles),
+// 0.46 / 0.53 for the 128^3 filament field (2e3), but 1.22 / 0.77 for the
+// 97 x 61 x 130 field (8e4).
+constexpr int kTinyD1 = 1 << 13, kRoundsTiny = 4;
 
 // Round loop of one column.  Phase A (max_rounds > 0): every column, one
 // group of GS threads (a half or a whole warp; NT / GS columns per block);
@@ -1155,6 +1250,10 @@ void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st) {
     cudaMemsetAsync(W.flags + 1, 0, sizeof(int32_t), st);
     return;
   }
+  if (n2 <= kSelectOne) {
+    k_d1_select_one<<<1, kSelectT, 0, st>>>(n2, P.d2_max, W.cols, P.d1_edge, W.flags + 1); note_launch();
+    return;
+  }
   uint32_t* flag = reinterpret_cast<uint32_t*>(W.lowc);  // scratch (n2 entries available)
   uint32_t* pos = reinterpret_cast<uint32_t*>(W.hsize);
   uint32_t* sums = reinterpret_cast<uint32_t*>(W.hcap);
@@ -1185,7 +1284,7 @@ void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int 
   }
   const int64_t mr = g_morse_rounds.load();
   const int roundsA =
-      mr > 0 ? (int)std::min<int64_t>(mr, 1 << 20) : (n2 >= kLargeD1 ? kRoundsLarge : kRoundsSmall);
+      mr > 0 ? (int)std::min<int64_t>(mr, 1 << 20) : (n2 >= kLargeD1 ? kRoundsLarge : n2 >= kTinyD1 ? kRoundsSmall : kRoundsTiny);
   cudaMemsetAsync(W.pool_head, 0, 4, st);
   cudaMemsetAsync(W.stats, 0, kD1Stats * sizeof(unsigned long long), st);
   cudaMemsetAsync(W.nbig, 0, sizeof(int32_t), st);

@@ -82,8 +82,9 @@ struct tsf_field {
   CritLists L{};
   int n0 = 0, n1 = 0, n2 = 0, n3 = 0;
   int cap_c0 = 0, cap_c1 = 0, cap_c2 = 0, cap_c3 = 0;
-  PairScratch PS{};
-  int cap_items = 0, cap_nodes = 0;
+  PairScratch S0{}, S2{};  // D0's and D2's
+  int cap_items0 = 0, cap_nodes0 = 0, cap_items2 = 0, cap_nodes2 = 0;
+  D1Ctl* d1ctl = nullptr;
   PairOut PO{};
   D1Work W{};
   int cap_cols = 0;
@@ -148,6 +149,23 @@ void profile_resolve(tsf_field* F) {
     }
   }
   F->ev_pending.clear();
+}
+
+void grow_pairs(PairScratch& S, int& cap_items, int items, int& cap_nodes, int nodes) {
+  if (items > cap_items) {
+    dev_free(S.ends);
+    cap_items = 0;
+    ck(dev_alloc(&S.ends, 2 * (size_t)items));
+    cap_items = items;
+  }
+  if (nodes > cap_nodes) {
+    dev_free(S.rec);
+    dev_free(S.skip);
+    cap_nodes = 0;
+    ck(dev_alloc(&S.rec, nodes));
+    ck(dev_alloc(&S.skip, nodes));
+    cap_nodes = nodes;
+  }
 }
 
 void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
@@ -216,19 +234,8 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
   F->L.cap1 = F->cap_c1;
   F->L.cap2 = F->cap_c2;
   F->L.cap3 = F->cap_c3;
-  int items = std::max(F->cap_c1, F->cap_c2);
-  int nodes = std::max(F->cap_c0, F->cap_c3 + 1);
-  if (items > F->cap_items || nodes > F->cap_nodes) {
-    int ci = std::max(items, F->cap_items), cn = std::max(nodes, F->cap_nodes);
-    dev_free(F->PS.ends);
-    dev_free(F->PS.rec);
-    dev_free(F->PS.skip);
-    ck(dev_alloc(&F->PS.ends, 2 * (size_t)ci));
-    ck(dev_alloc(&F->PS.rec, cn));
-    ck(dev_alloc(&F->PS.skip, cn));
-    F->cap_items = ci;
-    F->cap_nodes = cn;
-  }
+  grow_pairs(F->S0, F->cap_items0, F->cap_c1, F->cap_nodes0, F->cap_c0);
+  grow_pairs(F->S2, F->cap_items2, F->cap_c2, F->cap_nodes2, F->cap_c3 + 1);
 }
 
 void grow_solver(tsf_field* F, int np, int nt) {
@@ -480,10 +487,11 @@ int compute_diagram(tsf_field* F, bool incremental) {
   launch_crit_write(F->d, F->order, F->rank, F->rec, pack, F->tile_counts, F->L, F->cidx, F->c1base, F->c2base, st);
   stage_end(F, kCrit);
   stage_begin(F, kD0);
-  launch_d0(F->d, F->nd, F->L, F->n0, F->n1, F->vnext8, F->cidx, F->PS, F->PO, F->status, st);
+  launch_traces(F->d, F->nd, F->L, F->n0, F->n1, F->n2, F->n3, F->rank, F->rec, F->vnext8, F->cidx, F->S0, F->S2,
+                F->PO, F->status, st);
   stage_end(F, kD0);
   stage_begin(F, kD2);
-  launch_d2(F->d, F->nd, F->L, F->n2, F->n3, F->rank, F->rec, F->cidx, F->PS, F->PO, F->status, st);
+  launch_union_find(F->L, F->n0, F->n1, F->n2, F->n3, F->S0, F->S2, F->PO, F->status, st);
   stage_end(F, kD2);
   // D1, growing the column pool until it suffices (D0 and D2 report through
   // the same status word, read after the first attempt)
@@ -514,7 +522,7 @@ int compute_diagram(tsf_field* F, bool incremental) {
                     F->PO, F->status, st);
     stage_end(F, kD1Morse);
     stage_begin(F, kD1Reduce);
-    launch_d1_reduce(F->n1, F->n2, F->W, F->PO, F->status, reinterpret_cast<D1Ctl*>(F->PS.counter), st);
+    launch_d1_reduce(F->n1, F->n2, F->W, F->PO, F->status, F->d1ctl, st);
     stage_end(F, kD1Reduce);
     int32_t ncols = 0;
     for (auto& x : F->d1_stats) x = 0;
@@ -767,10 +775,12 @@ int tsf_destroy_field(tsf_field* F) {
   dev_free(F->L.c1_vn);
   dev_free(F->L.c2_ve);
   dev_free(F->L.c3);
-  dev_free(F->PS.ends);
-  dev_free(F->PS.rec);
-  dev_free(F->PS.skip);
-  dev_free(F->PS.counter);
+  for (PairScratch* S : {&F->S0, &F->S2}) {
+    dev_free(S->ends);
+    dev_free(S->rec);
+    dev_free(S->skip);
+  }
+  dev_free(F->d1ctl);
   dev_free(F->PO.d0_min);
   dev_free(F->PO.d0_killed);
   dev_free(F->PO.d0mask);
@@ -908,7 +918,7 @@ int tsf_create_field(int lx, int ly, int lz, const float* values, int values_on_
     ck(dev_alloc(&F->totals, 1));
     ck(dev_alloc(&F->status, 1));
     ck(dev_alloc(&F->counter, 1));
-    ck(dev_alloc(&F->PS.counter, 16));
+    ck(dev_alloc(&F->d1ctl, 1));
     ck(cudaMallocHost((void**)&F->h_flags, 16));
     ck(cudaMemcpyAsync(F->f, values, sizeof(float) * nv,
                        values_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, F->st));

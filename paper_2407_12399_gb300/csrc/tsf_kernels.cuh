@@ -103,13 +103,13 @@ struct PairScratch {
   int32_t* ends;             // 2 per item: component endpoints
   unsigned long long* rec;   // per node: union-find record and shortcut (k_uf_items)
   unsigned long long* skip;
-  int32_t* counter;          // control block of the D1 reduction (64 bytes)
 };
-void launch_d0(const Dims& d, const NbrDelta& nd, const CritLists& L, int n0, int n1, const uint8_t* vnext8,
-               const uint32_t* cidx, PairScratch& S, PairOut& P, uint32_t* status, cudaStream_t st);
-void launch_d2(const Dims& d, const NbrDelta& nd, const CritLists& L, int n2, int n3, const uint32_t* rank,
-               const Rec* rec, const uint32_t* cidx, PairScratch& S, PairOut& P, uint32_t* status,
-               cudaStream_t st);
+// D0 and D2 pairs: the integral lines of both, then both union-finds.
+void launch_traces(const Dims& d, const NbrDelta& nd, const CritLists& L, int n0, int n1, int n2, int n3,
+                   const uint32_t* rank, const Rec* rec, const uint8_t* vnext8, const uint32_t* cidx, PairScratch& S0,
+                   PairScratch& S2, PairOut& P, uint32_t* status, cudaStream_t st);
+void launch_union_find(const CritLists& L, int n0, int n1, int n2, int n3, PairScratch& S0, PairScratch& S2,
+                       PairOut& P, uint32_t* status, cudaStream_t st);
 
 // Control block of the whole-GPU D1 reduction rounds.
 struct D1Ctl {
