@@ -299,15 +299,14 @@ int64_t tsf_kernel_launches(void);
  *   5: critical triangles from which the D1 reduction starts with rounds
  *      over the whole GPU (default 262144);
  *   6: active D1 columns below which they go on on warps (default 131072);
- *   7: schedule of the D1 Morse boundaries' first phase: 0 the default
- *      (half a warp per column, registers capped for 32 warps per SM; 64 +
- *      128 frontier and stage entries for diagrams of at least 2^19
- *      critical triangles, else 32 + 64), 1 and 2 one warp per column with
- *      128 + 256 and 256 + 512 entries, 3 one warp with 64 + 128 without
- *      the register cap, 4 the same with it, 5 half a warp with 32 + 64, 6
- *      a quarter of a warp with 16 + 32, 7 half a warp with 64 + 128 at any
- *      size (columns that outgrow their buffers continue in the second
- *      phase);
+ *   7: schedule of the D1 Morse boundaries' first phase, as threads per
+ *      column and its frontier + stage entries (columns that outgrow them
+ *      continue in the second phase): 0 the default (8 for diagrams of at
+ *      least 2^19 critical triangles, 4 below 2^13, else 6), 1 and 2 one
+ *      warp with 128 + 256 and 256 + 512, 3 one warp with 64 + 128 without
+ *      the register cap, 4 the same with it, 5 half a warp with 32 + 64, 6 a
+ *      quarter of a warp with 16 + 32, 7 half a warp with 64 + 128, 8 a
+ *      quarter of a warp with 32 + 64;
  *   8: register budget of the lower-star gradient kernels, as blocks of
  *      128 threads per SM: 0 the default (6), 1 no cap, 2 five;
  *   9: entries of a column that a warp of the D1 reduction keeps in shared
@@ -317,7 +316,7 @@ int64_t tsf_kernel_launches(void);
  *      for diagrams of at least 2^19 critical triangles, else 2; at most 8);
  *  11: rounds of the D1 Morse boundaries' first phase before a column
  *      moves to a block of the second (0: the default, 128 for diagrams of
- *      at least 2^19 critical triangles, else 16);
+ *      at least 2^19 critical triangles, 4 below 2^13, else 16);
  *  12: additions a D1 column makes on a warp before it goes to a block (0:
  *      the default, 24);
  *  13: groups of 1024 rows that such a block keeps in shared memory (0: all

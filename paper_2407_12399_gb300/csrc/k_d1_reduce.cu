@@ -874,7 +874,7 @@ __global__ void k_d1_edges(int n1, D1Work W, int32_t* d1_edge) {
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-static int d1_sms() {
+int d1_sms() {
   static std::atomic<int> sms[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);

@@ -536,13 +536,23 @@ __global__ void k_d1_select(int n2, const int32_t* __restrict__ d2_max, uint32_t
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n2) flag[i] = d2_max[i] < 0 ? 1u : 0u;
 }
+// Every column starts with kOut0 words of the pool of its own, from j kOut0 on.
+constexpr uint32_t kOut0 = 64;
+__device__ __forceinline__ uint32_t d1_reserved(int ncols) {
+  return (uint32_t)min((unsigned long long)kOut0 * (unsigned)ncols, 1ull << 31);
+}
+
 __global__ void k_d1_gather(int n2, const uint32_t* __restrict__ flag, const uint32_t* __restrict__ pos,
-                            int32_t* __restrict__ cols, int32_t* __restrict__ d1_edge, int32_t* __restrict__ ncols) {
+                            int32_t* __restrict__ cols, int32_t* __restrict__ d1_edge, int32_t* __restrict__ ncols,
+                            uint32_t* __restrict__ pool_head) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n2) {
     d1_edge[i] = -1;
     if (flag[i]) cols[pos[i]] = i;
-    if (i == n2 - 1) *ncols = (int32_t)(pos[i] + flag[i]);
+    if (i == n2 - 1) {
+      *ncols = (int32_t)(pos[i] + flag[i]);
+      *pool_head = d1_reserved(*ncols);
+    }
   }
 }
 
@@ -551,7 +561,8 @@ __global__ void k_d1_gather(int n2, const uint32_t* __restrict__ flag, const uin
 constexpr int kSelectT = 1024, kSelectOne = 8 * kSelectT;
 __global__ void __launch_bounds__(kSelectT) k_d1_select_one(int n2, const int32_t* __restrict__ d2_max,
                                                             int32_t* __restrict__ cols, int32_t* __restrict__ d1_edge,
-                                                            int32_t* __restrict__ ncols) {
+                                                            int32_t* __restrict__ ncols,
+                                                            uint32_t* __restrict__ pool_head) {
   __shared__ int wsum[kSelectT / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int per = (n2 + kSelectT - 1) / kSelectT;
@@ -579,7 +590,10 @@ __global__ void __launch_bounds__(kSelectT) k_d1_select_one(int n2, const int32_
       if (lane >= o) xi += y;
     }
     wsum[lane] = xi - x;
-    if (lane == 31) *ncols = xi;
+    if (lane == 31) {
+      *ncols = xi;
+      *pool_head = d1_reserved(xi);
+    }
   }
   __syncthreads();
   int at = wsum[w] + inc - c;
@@ -713,7 +727,7 @@ __global__ void k_d1_morse(D1Ctx c, D1Work W, uint32_t* status) {
 // a column's updates come from its own group, so they live in the group's
 // shared memory: the frontier, sorted by descending key = value_key << 32 |
 // vertex (the rank order), one entry per star.  Each round the group takes
-// the NT highest entries, one per thread; every visit appends its updates of
+// the GS highest entries, one per thread; every visit appends its updates of
 // target stars to a stage; the stage is sorted, merged into the rest of the
 // frontier and equal keys are combined (xor of masks, zero masks dropped).
 // The projection is linear, so a star that receives entries after it was
@@ -738,107 +752,112 @@ __device__ __forceinline__ unsigned long long star_key(uint32_t vkey, uint32_t v
   return ((unsigned long long)vkey << 32) | v;
 }
 
-// Target stars of the link edges left by a visit, with compile-time
-// geometry: edge (a, b) goes to the lower star of whichever endpoint ranks
-// higher (P: a, Q: b), as the direction towards the other endpoint.
-template <int LE>
-__device__ __forceinline__ void link_edge_target(uint64_t P, uint64_t Q, uint32_t (&tm)[14]) {
-  constexpr int a = geo_edge(LE, 0), b = geo_edge(LE, 1);
-  constexpr int dab = geo_dir(a, b), dba = geo_dir(b, a);
-  tm[a] ^= (uint32_t)((P >> LE) & 1ull) << dab;
-  tm[b] ^= (uint32_t)((Q >> LE) & 1ull) << dba;
-}
-template <int... LE>
-__device__ __forceinline__ void link_targets(uint64_t P, uint64_t Q, uint32_t (&tm)[14],
-                                             std::integer_sequence<int, LE...>) {
-  (link_edge_target<LE>(P, Q, tm), ...);
-}
-template <int X>
-__device__ __forceinline__ void closure_of(const D1Tab& t, uint32_t m, uint64_t& path, uint32_t& em) {
-  if ((m >> X) & 1u) {
-    path ^= tab_closure<X>(t);
-    em ^= 1u << tab_end(t, X);
+// Link edge (a, b) left by a visit goes to the lower star of whichever
+// endpoint ranks higher, as the direction towards the other one.  le: a, b,
+// direction a -> b, direction b -> a, four bits each; at[x][0] / at[x][1]: the
+// edges that have x as their a / their b.  Copied to shared
+// memory: the index differs from lane to lane (constant memory would
+// serialise), and read from global memory they did not stay in L1 (21 % hits).
+struct D1Links {
+  unsigned long long at[14][2];
+  uint16_t le[36];
+};
+constexpr D1Links make_links() {
+  D1Links t{};
+  for (int e = 0; e < 36; ++e) {
+    const int a = geo_edge(e, 0), b = geo_edge(e, 1);
+    t.le[e] = (uint16_t)(a | b << 4 | geo_dir(a, b) << 8 | geo_dir(b, a) << 12);
+    t.at[a][0] |= 1ull << e;
+    t.at[b][1] |= 1ull << e;
   }
+  return t;
 }
-template <int... X>
-__device__ __forceinline__ void closures(const D1Tab& t, uint32_t m, uint64_t& path, uint32_t& em,
-                                         std::integer_sequence<int, X...>) {
-  (closure_of<X>(t, m, path, em), ...);
-}
+__device__ const D1Links g_links = make_links();
 
 // One lower-star visit: apply the closures of the star's pending edges
 // (linear over Z/2), keep the positive critical edges left as (v << 4 | x),
 // and append the link edges left to the stage as updates of the target
-// stars.  One dependent global load: the star's table row.  With `chain`
-// set, a visit whose link edges all go to one target star hands that update
-// back in *next instead of staging it, and the caller visits it at once (a
-// star reached again later by another part of its mask is simply visited
-// again: the projection is linear).
+// stars.  One dependent global access: the star's table row, of which only
+// the closures asked for are read.  The loops run over the bits that are set:
+// a visit has little more than one pending edge and 1.1 targets on average.
+// With `chain` set, a visit whose link edges all go to one target star hands
+// that update back in *next instead of staging it, and the caller visits it at
+// once (a star reached again later by another part of its mask is simply
+// visited again: the projection is linear).
+// Unrolling all 14 closures and 36 link edges at compile time needed the whole
+// row in registers (64 are what 32 warps per SM leave: it spilled) and issued a
+// fifth more instructions; the loops are worth it only where the groups of a
+// warp share them (tsf_group.cuh): Morse boundaries of a 256^3 field 13.0 ms
+// unrolled, 25.5 with loops and a barrier per group, 10.9 in lockstep.
 template <int SCAP>
-__device__ __forceinline__ bool d1_visit(const D1Ctx& c, FEnt fe, const int32_t* snd, FEnt* stage, int* s_ntot,
-                                         int* s_flag, unsigned long long* myouts, int& myout, int& updates, bool chain,
-                                         FEnt* next, uint32_t* status) {
-  uint32_t v = (uint32_t)fe.key;
-  uint32_t m = fe.mask;
+__device__ __forceinline__ bool d1_visit(const D1Ctx& c, FEnt fe, const int32_t* snd, const D1Links& links,
+                                         FEnt* stage, int* s_ntot, int* s_flag, unsigned long long* myouts, int& myout,
+                                         int& updates, bool chain, FEnt* next, uint32_t* status) {
+  const uint32_t v = (uint32_t)fe.key;
   if ((int64_t)v >= c.d.nv) {  // never for a valid entry: report and let the column be recomputed
     atomicOr(status, kErrInconsistent);
     atomicOr(s_flag, 1);
     return false;
   }
-  D1Tab t;
-  {
-    const uint4* s4 = reinterpret_cast<const uint4*>(c.tab + v);
-    uint4* d4 = reinterpret_cast<uint4*>(&t);
+  const uint32_t* row = reinterpret_cast<const uint32_t*>(c.tab + v);
+  const uint4 q89 = __ldg(reinterpret_cast<const uint4*>(row + 16));
+  uint4 nk[4];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) d4[k] = __ldg(s4 + k);
-  }
-  uint64_t path = 0;
+  for (int k = 0; k < 4; ++k) nk[k] = __ldg(reinterpret_cast<const uint4*>(row + 20) + k);
+  const uint64_t ends = (uint64_t)q89.y << 32 | q89.x, above = (uint64_t)q89.w << 32 | q89.z;
+  uint64_t path = fe.pad ? 1ull << (fe.pad - 1) : 0ull;  // a column's first entry brings a link edge
   uint32_t em = 0;
-  closures(t, m, path, em, std::make_integer_sequence<int, 14>{});
+  for (uint32_t mm = fe.mask & 0x3FFFu; mm; mm &= mm - 1) {
+    const int x = __ffs((int)mm) - 1, off = 36 * x;  // off <= 468: words 14 and 15 of the closures' 16
+    const uint32_t* p = row + (off >> 5);
+    path ^= ((uint64_t)__ldg(p + 1) << 32 | __ldg(p)) >> (off & 31);  // 36 bits from a multiple of 4 <= 28
+    em ^= 1u << ((uint32_t)(ends >> (4 * x)) & 15u);
+  }
+  path &= (1ull << 36) - 1;
   em &= 0x3FFFu;
   if (em) {
     em &= ~__ldg(c.d0mask + v);  // negative critical edges are not rows
-    for (; em; em &= em - 1) myouts[myout++] = ((unsigned long long)v << 4) | (unsigned)(__ffs(em) - 1);
-  }
-  uint32_t tmask[14];
-#pragma unroll
-  for (int k = 0; k < 14; ++k) tmask[k] = 0;
-  link_targets(path & t.q[9], path & ~t.q[9], tmask, std::make_integer_sequence<int, 36>{});
-  int cnt = 0, only = 0;
-#pragma unroll
-  for (int hn = 0; hn < 14; ++hn)
-    if (tmask[hn]) {
-      ++cnt;
-      only = hn;
+    if (em) {  // their indices are looked up at the column's end: bring them to L2
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(c.rec + v));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(c.c1base + v));
     }
-  if (!cnt) return false;
-  updates += cnt;
-  if (chain && cnt == 1) {
-    uint32_t hv = (uint32_t)((int32_t)v + snd[only]);
-    next->key = star_key(t.nkey[only], hv);
-    next->mask = tmask[only];
-    next->pad = 0;
-    return true;
+    for (; em; em &= em - 1) myouts[myout++] = ((unsigned long long)v << 4) | (unsigned)(__ffs((int)em) - 1);
   }
-  int off = atomicAdd(s_ntot, cnt);
-  if (off + cnt > SCAP) {
-    atomicOr(s_flag, 1);
-    return false;
-  }
-#pragma unroll
-  for (int hn = 0; hn < 14; ++hn) {
-    if (tmask[hn]) {
-      uint32_t hv = (uint32_t)((int32_t)v + snd[hn]);
-      FEnt e;
-      e.key = star_key(t.nkey[hn], hv);
-      e.mask = tmask[hn];
-      e.pad = 0;
-      stage[off++] = e;
-      // the star is likely visited in a later round: bring its row to L2
-      const char* row = reinterpret_cast<const char*>(c.tab + hv);
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(row + 128));
+  while (path) {
+    const int e0 = __ffsll((long long)path) - 1;
+    const uint32_t l0 = (uint32_t)links.le[e0];
+    const int hn = (int)((above >> e0) & 1ull ? l0 & 15u : (l0 >> 4) & 15u);
+    // all of them that go to the same star
+    uint64_t same = path & ((above & links.at[hn][0]) | (~above & links.at[hn][1]));
+    path ^= same;
+    uint32_t mask = 0;
+    for (; same; same &= same - 1) {
+      const int e = __ffsll((long long)same) - 1;
+      const uint32_t l = (uint32_t)links.le[e];
+      mask |= 1u << ((above >> e) & 1ull ? (l >> 8) & 15u : l >> 12);
     }
+    const uint32_t hv = (uint32_t)((int32_t)v + snd[hn]);
+    FEnt t;
+    t.mask = mask;
+    t.pad = 0;
+    ++updates;
+    const uint4 k4 = hn < 8 ? (hn < 4 ? nk[0] : nk[1]) : (hn < 12 ? nk[2] : nk[3]);
+    t.key = star_key(hn & 2 ? (hn & 1 ? k4.w : k4.z) : (hn & 1 ? k4.y : k4.x), hv);
+    if (chain && !path) {  // the only one
+      *next = t;
+      return true;
+    }
+    chain = false;
+    const int off = atomicAdd(s_ntot, 1);
+    if (off >= SCAP) {
+      atomicOr(s_flag, 1);
+      return false;
+    }
+    stage[off] = t;
+    // the star is likely visited in a later round: bring its row to L2
+    const char* trow = reinterpret_cast<const char*>(c.tab + hv);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(trow));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(trow + 128));
   }
   return false;
 }
@@ -850,8 +869,9 @@ __device__ __forceinline__ bool d1_visit(const D1Ctx& c, FEnt fe, const int32_t*
 template <int GS, int SCAP>
 __device__ void group_sort_stage(FEnt* a, int n) {
   static_assert(SCAP % GS == 0 && (SCAP & (SCAP - 1)) == 0, "a stage is a power of two");
-  if (n <= GS) group_sort_reg<GS, 1>(a, n);
-  else if (n <= 2 * GS && SCAP >= 2 * GS) group_sort_reg<GS, (SCAP >= 2 * GS ? 2 : 1)>(a, n);
+  const int most = gmax<GS>(n);
+  if (most <= GS) group_sort_reg<GS, 1>(a, n);
+  else if (most <= 2 * GS && SCAP >= 2 * GS) group_sort_reg<GS, (SCAP >= 2 * GS ? 2 : 1)>(a, n);
   else group_sort_smem<GS>(a, n);
 }
 
@@ -876,7 +896,8 @@ __device__ int group_combine(FEnt* front, int nb, int nf, FEnt* other, FEnt* sta
   }
   gsync<GS>();
   int kept = 0;
-  for (int base = 0; base < total; base += GS) {
+  const int most = gmax<GS>(total);
+  for (int base = 0; base < most; base += GS) {
     int k = base + tid;
     int keep = 0;
     FEnt e;
@@ -904,103 +925,84 @@ __device__ int group_combine(FEnt* front, int nb, int nf, FEnt* other, FEnt* sta
 // column moves to a block.  The defaults depend on the diagram's size.  A
 // large diagram (at least kLargeD1 critical triangles) keeps enough columns
 // in flight in phase A to fill the GPU, so its columns stay there (no
-// chaining, 128 rounds, 64 + 128 entries per column).  A small one gains
-// from moving its long columns to 128-thread blocks early (chains of 2, 16
-// rounds, 32 + 64 entries).  Measured, ms per iteration on the 256^3
-// headline field (1.8 M critical triangles) / the 128^3 filament field
-// (~0.25 M): large settings 64.7 / 2.89, small settings 67.8 / 1.89;
-// 32 rounds with either tile lay in between on both (65.1-65.5 / 2.07-2.15).
+// chaining, 128 rounds); a smaller one gains from moving its long columns to
+// 128-thread blocks early (chains of 2, 16 rounds).  Stage time, ms: 256^3
+// field (2.6e6 triangles) at 16 / 24 / 64 / 128 rounds 11.3 / 8.5 / 8.1 / 8.1;
+// 97 x 61 x 130 field (8e4) at 6 / 12 / 16 / 24: 0.68 / 0.48 / 0.50 / 0.52.
 constexpr int kOutCap = 28;
 constexpr int kLargeD1 = 1 << 19;
 constexpr int kChainLarge = 1, kRoundsLarge = 128;  // defaults of knobs 10 and 11, large diagrams
 constexpr int kChainSmall = 2, kRoundsSmall = 16;   // ... small diagrams
 // Below 2^13 critical triangles every column can have its block at once, so
-// phase A only keeps the columns that end after a few rounds.  Stage time at
-// 4 / 16 rounds: 0.101 / 0.155 ms for a 32^3 field (3.5e3 triangles),
-// 0.46 / 0.53 for the 128^3 filament field (2e3), but 1.22 / 0.77 for the
-// 97 x 61 x 130 field (8e4).
+// phase A only keeps the columns that end after a few rounds.  At 2 / 4 / 6 /
+// 12 rounds: 32^3 field (3e3 triangles) 0.136 / 0.105 / 0.107 / 0.138 ms, 128^3
+// filament field (2e3) 0.38 / 0.39 / 0.43 / 0.44, but 1.8 / 1.2 / 0.68 / 0.48
+// for the 97 x 61 x 130 field.
 constexpr int kTinyD1 = 1 << 13, kRoundsTiny = 4;
 
-// Round loop of one column.  Phase A (max_rounds > 0): every column, one
-// group of GS threads (a half or a whole warp; NT / GS columns per block);
-// a column still open after max_rounds, or whose frontier outgrows the
-// group's buffers, saves its entries and is listed for phase B (NT = GS =
-// 128, one block per listed column).  Groups of one block share nothing
-// but the neighbour offsets and synchronise only among themselves.
-template <int NT, int FCAP, int SCAP, int MINB = (NT == 32 ? 12 : 4), int GS = NT>
-__global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, int max_rounds, uint32_t* status) {
-  static_assert(GS == NT || (NT == 32 && GS < 32), "several groups only within one warp");
+// One column.  Phase A (max_rounds > 0): every column, one group of GS threads
+// (a quarter, a half or a whole warp); a column still open after max_rounds,
+// or whose frontier outgrows the group's buffers, saves its entries and is
+// listed for phase B (NT = GS = 128, one block per listed column).  Groups of
+// a warp run in lockstep: a group without a column (not `live`), or whose
+// column has stopped, goes along without changing anything.  Groups of one
+// block otherwise share only the tables.
+template <int NT, int FCAP, int SCAP, int GS>
+__device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool live, bool phase_b, int max_rounds,
+                                          FEnt* front, const int32_t* snd, const D1Links& links, int* scan_sm,
+                                          unsigned long long* acc, uint32_t* status) {
   constexpr int G = NT / GS;
-  const int ncols = W.flags[1];
   const int gi = (int)threadIdx.x / GS;
-  extern __shared__ __align__(16) unsigned char smem[];
-  FEnt* front = reinterpret_cast<FEnt*>(smem) + (size_t)gi * (2 * FCAP + SCAP);
   FEnt* other = front + FCAP;
   FEnt* stage = other + FCAP;
-  __shared__ int32_t snd[16];
-  __shared__ int scan_sm[16];  // GS/32 + 1 <= 16 (blocks only)
   __shared__ int sg_nf[G], sg_flag[G], sg_ntot[G], sg_otot[G];
-  __shared__ Vec sg_out[G], sg_grow[G], sg_fr[G], sg_fr2[G];
+  __shared__ Vec sg_out[G], sg_grow[G], sg_fr[G];
   int& s_nf = sg_nf[gi];
   int& s_flag = sg_flag[gi];
   int& s_ntot = sg_ntot[gi];
   int& s_otot = sg_otot[gi];
   Vec& s_out = sg_out[gi];
   Vec& s_grow = sg_grow[gi];
-  if (threadIdx.x < 14) snd[threadIdx.x] = c.nd.d[threadIdx.x];
-  if (NT > 32) __syncthreads();
-  else __syncwarp();  // snd is read by every group
-  const bool phase_b = max_rounds <= 0;
-  int j;
-  if (phase_b) {
-    if ((int)blockIdx.x >= *W.nbig) return;
-    j = W.big[blockIdx.x];
-  } else {
-    j = (int)blockIdx.x * G + gi;
-    if (j >= ncols) return;
-  }
+  Vec& s_fr = sg_fr[gi];
   const int tid = gtid<GS>();
   if (tid == 0) {
     s_flag = 0;
     s_nf = 0;
     s_ntot = 0;
     s_otot = 0;
-    if (phase_b) {
+    if (live && phase_b) {
       uint4 cs = W.cont[j];
       s_ntot = (int)cs.y;  // saved entries, combined below like a stage
       s_out.off = cs.z;
       s_out.size = cs.w;
       s_out.cap = W.cont_cap[j];
       s_out.h = W.pool + s_out.off;
-    } else {
-      if (!vec_alloc(W, s_out, 64, status)) s_flag = 1;
-      // seed: the boundary of the critical triangle, each edge an entry of
-      // the lower star of its higher endpoint
-      uint32_t ve = c.L.c2_ve[W.cols[j]];
-      uint32_t v0 = ve >> 6;
-      int e0 = (int)(ve & 63u);
-      uint32_t ea = (uint32_t)((int32_t)v0 + c.nd.d[c_geo.edge[e0][0]]);
-      uint32_t eb = (uint32_t)((int32_t)v0 + c.nd.d[c_geo.edge[e0][1]]);
-      uint32_t ends[3][2] = {{v0, ea}, {v0, eb}, {ea, eb}};
-      for (int k = 0; k < 3; ++k) {
-        uint32_t p = ends[k][0], q = ends[k][1];
-        uint32_t rp = c.rank[p], rq = c.rank[q];
-        uint32_t hi = rp > rq ? p : q, lo = rp > rq ? q : p;
-        FEnt e;
-        e.key = star_key(value_key(c.f[hi]), hi);
-        e.mask = 1u << nbr_of_pair(c.d, hi, lo);
-        e.pad = 0u;
-        stage[s_ntot++] = e;
+    } else if (live) {
+      s_out.off = kOut0 * (uint32_t)j;
+      s_out.size = 0;
+      s_out.cap = kOut0;
+      s_out.h = W.pool + s_out.off;
+      if ((unsigned long long)kOut0 * (unsigned)j + kOut0 > W.pool_cap) {
+        atomicOr(status, kErrPool);
+        s_flag = 1;
       }
+      // seed: the boundary of the critical triangle.  Its highest vertex is v0;
+      // the edge opposite goes to its lower star as a link edge of v0.
+      const uint32_t ve = c.L.c2_ve[W.cols[j]];
+      const int e0 = (int)(ve & 63u);
+      FEnt e;
+      e.key = ve >> 6;  // alone in the frontier: not compared
+      e.mask = 1u << (links.le[e0] & 15) | 1u << (links.le[e0] >> 4 & 15);
+      e.pad = (uint32_t)e0 + 1;
+      front[0] = e;
+      s_nf = 1;
     }
   }
   gsync<GS>();
   if (phase_b) {
     uint4 cs = W.cont[j];
     for (int i = tid; i < (int)cs.y; i += GS) stage[i] = fent_restore(W.pool + cs.x + 2 * (size_t)i);
-  }
-  gsync<GS>();
-  {
+    gsync<GS>();
     int n0 = group_combine<GS, SCAP>(front, 0, 0, other, stage, s_ntot, scan_sm);
     if (tid == 0) {
       s_nf = n0;
@@ -1011,19 +1013,20 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
   int visits = 0, updates = 0, rounds = 0;
   bool failed = s_flag != 0;
   bool handoff = false;
-  while (!failed) {
-    int nf = s_nf;
-    if (nf == 0) break;
-    if (!phase_b && rounds >= max_rounds) break;
+  bool run = live && !failed;
+  for (;;) {
+    const int nf = run ? s_nf : 0;
+    if (nf == 0 || (!phase_b && rounds >= max_rounds)) run = false;
     // every target is a lower neighbour of the visited vertex, so the
     // frontier's highest key drops each round: at most nv rounds
-    if (rounds > c.d.nv) {
+    if (run && rounds > c.d.nv) {
       if (tid == 0) atomicOr(status, kErrRounds);
       failed = true;
-      break;
+      run = false;
     }
-    ++rounds;
-    int nb = min(GS, nf);
+    if (!gany<GS>(run)) break;
+    rounds += run ? 1 : 0;
+    const int nb = run ? min(GS, nf) : 0;
     int myout = 0;
     unsigned long long myouts[kOutCap];
     if (tid < nb) {
@@ -1032,21 +1035,21 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
         ++visits;
         FEnt nxt;
         bool more = k + 1 < c.chain && myout + 14 <= kOutCap;
-        if (!d1_visit<SCAP>(c, cur, snd, stage, &s_ntot, &s_flag, myouts, myout, updates, more, &nxt, status))
+        if (!d1_visit<SCAP>(c, cur, snd, links, stage, &s_ntot, &s_flag, myouts, myout, updates, more, &nxt, status))
           break;
         cur = nxt;
       }
     }
-    int ooff = myout ? atomicAdd(&s_otot, myout) : 0;
+    const int ooff = myout ? atomicAdd(&s_otot, myout) : 0;
     gsync<GS>();
-    if (s_flag) {  // stage overflow: updates were dropped, recompute the column
+    if (run && s_flag) {  // stage overflow: updates were dropped, recompute the column
       failed = true;
-      break;
+      run = false;
     }
     // outputs: append to the column's list in the pool (grown by the group)
-    int otot = s_otot;
-    if (otot > 0) {
-      if (tid == 0) {
+    const int otot = run ? s_otot : 0;
+    if (gany<GS>(otot > 0)) {
+      if (tid == 0 && otot > 0) {
         s_grow.h = nullptr;
         if (s_out.size + otot > s_out.cap) {
           uint32_t cap = s_out.cap;
@@ -1058,57 +1061,60 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
         }
       }
       gsync<GS>();
-      if (s_flag) {
+      if (run && s_flag) {
         failed = true;
-        break;
+        run = false;
       }
-      if (s_grow.h) {
-        for (uint32_t i = tid; i < s_out.size; i += GS) s_grow.h[i] = s_out.h[i];
+      const bool grow = run && otot > 0 && s_grow.h;
+      if (gany<GS>(grow)) {
+        if (grow)
+          for (uint32_t i = tid; i < s_out.size; i += GS) s_grow.h[i] = s_out.h[i];
         gsync<GS>();
-        if (tid == 0) {
+        if (grow && tid == 0) {
           s_grow.size = s_out.size;
           s_out = s_grow;
         }
         gsync<GS>();
       }
-      for (int k = 0; k < myout; ++k) s_out.h[s_out.size + ooff + k] = myouts[k];
+      if (run)
+        for (int k = 0; k < myout; ++k) s_out.h[s_out.size + ooff + k] = myouts[k];
       gsync<GS>();
-      if (tid == 0) {
+      if (tid == 0 && run) {
         s_out.size += otot;
         s_otot = 0;
       }
     }
-    int ntot = s_ntot;
-    if (nf - nb + ntot > FCAP) {  // the new frontier would not fit
-      handoff = !phase_b;
-      failed = true;
-      if (handoff) {  // phase A: the rest and the stage go to phase B as they are
-        Vec& s_fr = sg_fr[gi];
-        int rest = nf - nb;
-        if (tid == 0 && !vec_alloc(W, s_fr, 2u * (uint32_t)(rest + ntot), status)) s_flag = 1;
-        gsync<GS>();
-        if (!s_flag) {
-          for (int i = tid; i < rest; i += GS) fent_save(s_fr.h + 2 * i, front[nb + i]);
-          for (int i = tid; i < ntot; i += GS) fent_save(s_fr.h + 2 * (rest + i), stage[i]);
-          gsync<GS>();
-          if (tid == 0) {
-            W.cont[j] = make_uint4(s_fr.off, (uint32_t)(rest + ntot), s_out.off, s_out.size);
-            W.cont_cap[j] = s_out.cap;
-            W.big[atomicAdd(W.nbig, 1)] = j;
-          }
-        } else {
-          handoff = false;
-        }
+    const int ntot = run ? s_ntot : 0;
+    const int rest = nf - nb;
+    const bool over = run && rest + ntot > FCAP;  // the new frontier would not fit
+    if (gany<GS>(over)) {
+      const bool save = over && !phase_b;  // phase A: the rest and the stage go to phase B as they are
+      if (over) {
+        failed = true;
+        run = false;
       }
-      break;
+      if (save && tid == 0 && !vec_alloc(W, s_fr, 2u * (uint32_t)(rest + ntot), status)) s_flag = 1;
+      gsync<GS>();
+      if (save && !s_flag) {
+        handoff = true;
+        for (int i = tid; i < rest; i += GS) fent_save(s_fr.h + 2 * i, front[nb + i]);
+        for (int i = tid; i < ntot; i += GS) fent_save(s_fr.h + 2 * (rest + i), stage[i]);
+      }
+      gsync<GS>();
+      if (handoff && save && tid == 0) {
+        W.cont[j] = make_uint4(s_fr.off, (uint32_t)(rest + ntot), s_out.off, s_out.size);
+        W.cont_cap[j] = s_out.cap;
+        W.big[atomicAdd(W.nbig, 1)] = j;
+      }
     }
-    if (nf == nb && ntot <= GS) {
+    if (!gany<GS>(run && !(rest == 0 && ntot <= GS))) {
       // every entry is taken next round, so neither their order nor
       // combining equal keys matters (a star listed twice is visited twice
       // with parts of its mask: the projection is linear)
-      for (int i = tid; i < ntot; i += GS) front[i] = stage[i];
+      if (run)
+        for (int i = tid; i < ntot; i += GS) front[i] = stage[i];
       gsync<GS>();  // every thread has read s_ntot before it is reset
-      if (tid == 0) {
+      if (tid == 0 && run) {
         s_nf = ntot;
         s_ntot = 0;
       }
@@ -1116,8 +1122,9 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
       continue;
     }
     gsync<GS>();
-    int nn = group_combine<GS, SCAP>(front, nb, nf, other, stage, ntot, scan_sm);
-    if (tid == 0) {
+    // a group that has stopped keeps its frontier: it combines nothing
+    const int nn = group_combine<GS, SCAP>(front, run ? nb : 0, run ? nf : 0, other, stage, run ? ntot : 0, scan_sm);
+    if (tid == 0 && run) {
       s_nf = nn;
       s_ntot = 0;
     }
@@ -1127,63 +1134,55 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
   int vtot, utot;
   gscan<GS>(visits, vtot, scan_sm);
   gscan<GS>(updates, utot, scan_sm);
-  if (handoff || (!failed && !phase_b && s_nf > 0)) {
-    if (!handoff) {  // still open after max_rounds: save the frontier for phase B
-      Vec& s_fr2 = sg_fr2[gi];
-      if (tid == 0 && !vec_alloc(W, s_fr2, 2u * (uint32_t)s_nf, status)) s_flag = 1;
-      gsync<GS>();
-      if (s_flag) {
-        if (tid == 0) {
-          W.redo[j] = 1;
-          W.hsize[j] = 0;
-        }
-        return;
-      }
-      for (int i = tid; i < s_nf; i += GS) fent_save(s_fr2.h + 2 * i, front[i]);
-      gsync<GS>();
-      if (tid == 0) {
-        W.cont[j] = make_uint4(s_fr2.off, (uint32_t)s_nf, s_out.off, s_out.size);
-        W.cont_cap[j] = s_out.cap;
-        W.big[atomicAdd(W.nbig, 1)] = j;
-      }
+  bool redo = live && failed && !handoff;
+  const bool open = live && !failed && !phase_b && s_nf > 0;  // still open after max_rounds: save the frontier for phase B
+  if (gany<GS>(open)) {
+    if (open && tid == 0 && !vec_alloc(W, s_fr, 2u * (uint32_t)s_nf, status)) s_flag = 1;
+    gsync<GS>();
+    redo = redo || (open && s_flag);
+    if (open && !redo)
+      for (int i = tid; i < s_nf; i += GS) fent_save(s_fr.h + 2 * i, front[i]);
+    gsync<GS>();
+    if (open && !redo && tid == 0) {
+      W.cont[j] = make_uint4(s_fr.off, (uint32_t)s_nf, s_out.off, s_out.size);
+      W.cont_cap[j] = s_out.cap;
+      W.big[atomicAdd(W.nbig, 1)] = j;
     }
-    if (tid == 0) {
-      W.redo[j] = 0;
-      W.hsize[j] = 0;
-      atomicAdd(&W.stats[0], (unsigned long long)vtot);
-      atomicAdd(&W.stats[2], (unsigned long long)rounds);
-      atomicAdd(&W.stats[4], (unsigned long long)utot);
-    }
-    return;
   }
-  if (failed) {
-    if (tid == 0) {
-      W.redo[j] = 1;
-      W.hsize[j] = 0;
-    }
-    return;
+  const bool goes_on = live && !redo && (handoff || open);
+  if (goes_on && tid == 0) {
+    W.redo[j] = 0;
+    W.hsize[j] = 0;
+    acc[0] += (unsigned long long)vtot;
+    acc[2] += (unsigned long long)rounds;
+    acc[4] += (unsigned long long)utot;
   }
   // finished: (v, x) -> C1 index, sort descending, keep the entries present
   // an odd number of times (Z/2)
-  uint32_t nout = s_out.size;
+  bool fin = live && !redo && !goes_on;
+  int nout = fin ? (int)s_out.size : 0;
   int n2 = 1;
-  while (n2 < (int)nout) n2 <<= 1;
+  while (n2 < nout) n2 <<= 1;
+  n2 = gmax<GS>(n2);
   unsigned long long* a = reinterpret_cast<unsigned long long*>(stage);
   if (n2 > 2 * SCAP) {  // too long for shared memory: sort in the pool
-    if (tid == 0 && !vec_alloc(W, s_grow, (uint32_t)n2, status)) s_flag = 1;
+    if (fin && tid == 0 && !vec_alloc(W, s_grow, (uint32_t)n2, status)) s_flag = 1;
     gsync<GS>();
-    if (s_flag) {
-      if (tid == 0) {
-        W.redo[j] = 1;
-        W.hsize[j] = 0;
-      }
-      return;
+    if (fin && s_flag) {
+      redo = true;
+      fin = false;
+      nout = 0;
     }
-    a = s_grow.h;
+    if (fin) a = s_grow.h;
   }
-  for (int i = tid; i < n2; i += GS) {
+  if (redo && tid == 0) {
+    W.redo[j] = 1;
+    W.hsize[j] = 0;
+  }
+  if (!gany<GS>(fin)) return;
+  for (int i = tid; fin && i < n2; i += GS) {
     unsigned long long ci = 0;
-    if (i < (int)nout) {
+    if (i < nout) {
       uint32_t v = (uint32_t)(s_out.h[i] >> 4);
       int x = (int)(s_out.h[i] & 15ull);
       int cnt = __popc(rec_crit_edges(ld_rec(c.rec, v)));
@@ -1197,17 +1196,18 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
     a[i] = ci;
   }
   gsync<GS>();
-  group_sort_desc<GS>(a, n2);
+  group_sort_desc<GS>(a, n2, fin);
   int kept = 0;
-  for (int base = 0; base < (int)nout; base += GS) {
+  const int most = gmax<GS>(nout);
+  for (int base = 0; base < most; base += GS) {
     int k = base + tid;
     int keep = 0;
     unsigned long long x = 0;
-    if (k < (int)nout) {
+    if (k < nout) {
       x = a[k];
       if (k == 0 || a[k - 1] != x) {
         int e = k + 1;
-        while (e < (int)nout && a[e] == x) ++e;
+        while (e < nout && a[e] == x) ++e;
         keep = (e - k) & 1;
       }
     }
@@ -1217,23 +1217,89 @@ __global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, 
     kept += t;
   }
   gsync<GS>();
-  if (tid == 0) {
+  if (fin && tid == 0) {
     W.hoff[j] = s_out.off;
     W.hsize[j] = (uint32_t)kept;
     W.redo[j] = 0;
-    atomicAdd(&W.stats[0], (unsigned long long)vtot);
-    atomicMax(&W.stats[1], (unsigned long long)vtot);
-    atomicAdd(&W.stats[2], (unsigned long long)rounds);
-    atomicMax(&W.stats[3], (unsigned long long)rounds);
-    atomicAdd(&W.stats[4], (unsigned long long)utot);
+    acc[0] += (unsigned long long)vtot;
+    acc[1] = max(acc[1], (unsigned long long)vtot);
+    acc[2] += (unsigned long long)rounds;
+    acc[3] = max(acc[3], (unsigned long long)rounds);
+    acc[4] += (unsigned long long)utot;
   }
 }
 
-// Phase A runs two columns per warp (half a warp each: a round visits ~9
-// lower stars on average, so a whole warp left most lanes idle), keeps its
-// shared memory small (4 KB per column) and its registers at 63 so that 28
-// one-warp blocks, 56 columns, share an SM: the rounds are latency-bound.  A visit appends 1.1 updates on average, 14 at most; a
-// column that outgrows the buffers continues in phase B.
+// Groups take columns by ticket (W.flags[2] in phase A, [3] in phase B), so a
+// launch is as large as the GPU and not as the diagram: phase B's blocks with
+// nothing to do took 0.29 ms for 4.9e5 triangles.
+template <int NT, int FCAP, int SCAP, int MINB = (NT == 32 ? 12 : 4), int GS = NT>
+__global__ void __launch_bounds__(NT, MINB) k_d1_morse_group(D1Ctx c, D1Work W, int max_rounds, uint32_t* status) {
+  static_assert(GS == NT || GS < 32, "several groups only within one warp");
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ D1Links links;
+  __shared__ int32_t snd[16];
+  __shared__ int scan_sm[16];  // GS/32 + 1 <= 16 (blocks only)
+  __shared__ int s_ticket;
+  const bool phase_b = max_rounds <= 0;
+  const int total = phase_b ? *W.nbig : W.flags[1];
+  FEnt* front = reinterpret_cast<FEnt*>(smem) + (size_t)(threadIdx.x / GS) * (2 * FCAP + SCAP);
+  if (threadIdx.x < 14) snd[threadIdx.x] = c.nd.d[threadIdx.x];
+  for (int i = threadIdx.x; i < (int)(sizeof(D1Links) / 4); i += NT)
+    reinterpret_cast<uint32_t*>(&links)[i] = __ldg(reinterpret_cast<const uint32_t*>(&g_links) + i);
+  if (NT > 32) __syncthreads();
+  else __syncwarp();  // read by every group
+  // the group's share of W.stats (added once: per column the atomics on one
+  // line took as long as a round)
+  __shared__ unsigned long long s_acc[NT / GS][kD1Stats];
+  unsigned long long* acc = s_acc[threadIdx.x / GS];
+  if (gtid<GS>() == 0)
+    for (int k = 0; k < kD1Stats; ++k) acc[k] = 0;
+  int* const tickets = W.flags + (phase_b ? 3 : 2);
+  // With many columns to come the next ticket is drawn before the column, else
+  // after it (a ticket drawn early waits behind a long column).
+  const bool early = !phase_b && total > 8 * (int)gridDim.x * (NT / GS);
+  int next = gtid<GS>() == 0 ? atomicAdd(tickets, 1) : 0;
+  for (;;) {
+    int t;
+    if (GS > 32) {
+      if (threadIdx.x == 0) s_ticket = next;
+      __syncthreads();
+      t = s_ticket;
+    } else {
+      t = __shfl_sync(0xFFFFFFFFu, next, 0, GS);
+    }
+    const bool live = t < total;
+    if (!gany<GS>(live)) break;
+    if (early && gtid<GS>() == 0) next = atomicAdd(tickets, 1);
+    gsync<GS>();  // the group is done with the last column's shared words and ticket
+    d1_column<NT, FCAP, SCAP, GS>(c, W, !live ? 0 : phase_b ? W.big[t] : t, live, phase_b, max_rounds, front, snd,
+                                  links, scan_sm, acc, status);
+    if (!early && gtid<GS>() == 0) next = atomicAdd(tickets, 1);
+  }
+  if (gtid<GS>() == 0 && acc[0]) {
+    atomicAdd(&W.stats[0], acc[0]);
+    atomicMax(&W.stats[1], acc[1]);
+    atomicAdd(&W.stats[2], acc[2]);
+    atomicMax(&W.stats[3], acc[3]);
+    atomicAdd(&W.stats[4], acc[4]);
+  }
+}
+
+// Phase A is bound by the latency of its rounds (a table row from L2 or memory,
+// then a few hundred instructions; ncu: 43 % of issue slots, 60 % of the stalls
+// on loads), so what counts is columns in flight and lanes in use: a round
+// visits 4 lower stars on average on noise, 30 on long filaments.  Registers
+// are held to 64 so that 32 one-warp blocks share an SM; a column that outgrows
+// its tile continues in phase B.  Stage time, ms, with a quarter warp and
+// 32 + 64 entries (8) / a quarter and 16 + 32 (6) / half a warp and 32 + 64 (5) /
+// a whole warp and 64 + 128 (4):
+//   256^3 field, 2.6e6 triangles        8.1 / 9.5 / 8.7 / 10.4   -> 8
+//   96^3 field, 7e4 triangles           0.78 / 0.71 / 0.83 / 0.93 -> 6
+//   97 x 61 x 130 field, 8e4 triangles  0.54 / 0.50 / 0.61 / 0.71 -> 6
+//   32^3 field, 3e3 triangles           0.116 / 0.112 / 0.103 / 0.105
+//   128^3 filament field, 2e3           0.42 / 0.40 / 0.44 / 0.39 -> 4
+// Before (half-warp groups on their own, whole rows in local memory, a launch
+// block per column): 15.2, 1.03, 0.77, 0.103 and 0.50 ms.
 constexpr int kThreadsB = 128;
 constexpr int kFrontA = 64, kStageA = 128;
 constexpr int kFrontH = 32, kStageH = 64;
@@ -1251,7 +1317,7 @@ void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st) {
     return;
   }
   if (n2 <= kSelectOne) {
-    k_d1_select_one<<<1, kSelectT, 0, st>>>(n2, P.d2_max, W.cols, P.d1_edge, W.flags + 1); note_launch();
+    k_d1_select_one<<<1, kSelectT, 0, st>>>(n2, P.d2_max, W.cols, P.d1_edge, W.flags + 1, W.pool_head); note_launch();
     return;
   }
   uint32_t* flag = reinterpret_cast<uint32_t*>(W.lowc);  // scratch (n2 entries available)
@@ -1259,7 +1325,7 @@ void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st) {
   uint32_t* sums = reinterpret_cast<uint32_t*>(W.hcap);
   k_d1_select<<<(n2 + 255) / 256, 256, 0, st>>>(n2, P.d2_max, flag); note_launch();
   exclusive_scan_u32(flag, pos, n2, sums, st);
-  k_d1_gather<<<(n2 + 255) / 256, 256, 0, st>>>(n2, flag, pos, W.cols, P.d1_edge, W.flags + 1); note_launch();
+  k_d1_gather<<<(n2 + 255) / 256, 256, 0, st>>>(n2, flag, pos, W.cols, P.d1_edge, W.flags + 1, W.pool_head); note_launch();
 }
 
 void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1, int n2, const uint32_t* rank,
@@ -1285,9 +1351,9 @@ void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int 
   const int64_t mr = g_morse_rounds.load();
   const int roundsA =
       mr > 0 ? (int)std::min<int64_t>(mr, 1 << 20) : (n2 >= kLargeD1 ? kRoundsLarge : n2 >= kTinyD1 ? kRoundsSmall : kRoundsTiny);
-  cudaMemsetAsync(W.pool_head, 0, 4, st);
   cudaMemsetAsync(W.stats, 0, kD1Stats * sizeof(unsigned long long), st);
   cudaMemsetAsync(W.nbig, 0, sizeof(int32_t), st);
+  cudaMemsetAsync(W.flags + 2, 0, 2 * sizeof(int32_t), st);  // the tickets
   size_t sb = d1_group_smem(kFrontB, kStageB);
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1305,52 +1371,55 @@ void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int 
                          (int)(2 * d1_group_smem(kFrontA, kStageA)));
     cudaFuncSetAttribute(k_d1_morse_group<32, kFrontH, kStageH, 32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(2 * d1_group_smem(kFrontH, kStageH)));
+    cudaFuncSetAttribute(k_d1_morse_group<32, kFrontH, kStageH, 32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(4 * d1_group_smem(kFrontH, kStageH)));
     cudaFuncSetAttribute(k_d1_morse_group<32, kFrontQ, kStageQ, 32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(4 * d1_group_smem(kFrontQ, kStageQ)));
     cudaFuncSetAttribute(k_d1_morse_group<kThreadsB, kFrontB, kStageB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sb);
     attr[dev].store(true, std::memory_order_release);
   }
-  // phase A buffers: the default, or 2x / 4x larger (more shared memory per
-  // warp, fewer warps per SM; a column that outgrows them continues in
-  // phase B)
-  // knob 7 = 0: the larger tile for large diagrams, the smaller one otherwise
+  // blocks of g columns, at most what an SM holds of them
+  const auto blocks = [&](int g, int per_sm) { return std::min((n2 + g - 1) / g, d1_sms() * per_sm); };
+  // knob 7 = 0: by size, see the figures at kThreadsB
   int64_t phase_a = g_d1_phase_a.load();
-  if (phase_a == 0 && n2 < kLargeD1) phase_a = 5;
+  if (phase_a == 0) phase_a = n2 >= kLargeD1 ? 8 : n2 >= kTinyD1 ? 6 : 4;
   switch (phase_a) {
     case 1:
-      k_d1_morse_group<32, kFrontA * 2, kStageA * 2><<<n2, 32, d1_group_smem(kFrontA * 2, kStageA * 2), st>>>(
+      k_d1_morse_group<32, kFrontA * 2, kStageA * 2><<<blocks(1, 12), 32, d1_group_smem(kFrontA * 2, kStageA * 2), st>>>(
           c, W, roundsA, status);
       break;
     case 2:
-      k_d1_morse_group<32, kFrontA * 4, kStageA * 4><<<n2, 32, d1_group_smem(kFrontA * 4, kStageA * 4), st>>>(
+      k_d1_morse_group<32, kFrontA * 4, kStageA * 4><<<blocks(1, 12), 32, d1_group_smem(kFrontA * 4, kStageA * 4), st>>>(
           c, W, roundsA, status);
       break;
     case 3:  // one warp per column without the register cap
-      k_d1_morse_group<32, kFrontA, kStageA><<<n2, 32, d1_group_smem(kFrontA, kStageA), st>>>(c, W, roundsA,
+      k_d1_morse_group<32, kFrontA, kStageA><<<blocks(1, 12), 32, d1_group_smem(kFrontA, kStageA), st>>>(c, W, roundsA,
                                                                                              status);
       break;
     case 4:  // one warp per column, registers capped (63) so that 32 warps fit an SM
-      k_d1_morse_group<32, kFrontA, kStageA, 32><<<n2, 32, d1_group_smem(kFrontA, kStageA), st>>>(c, W, roundsA,
+      k_d1_morse_group<32, kFrontA, kStageA, 32><<<blocks(1, 32), 32, d1_group_smem(kFrontA, kStageA), st>>>(c, W, roundsA,
                                                                                                   status);
       break;
     case 5:  // half a warp per column with the smaller tile
-      k_d1_morse_group<32, kFrontH, kStageH, 32, 16><<<(n2 + 1) / 2, 32, 2 * d1_group_smem(kFrontH, kStageH), st>>>(
+      k_d1_morse_group<32, kFrontH, kStageH, 32, 16><<<blocks(2, 32), 32, 2 * d1_group_smem(kFrontH, kStageH), st>>>(
           c, W, roundsA, status);
       break;
     case 6:  // a quarter of a warp per column with the smallest tile
-      k_d1_morse_group<32, kFrontQ, kStageQ, 32, 8><<<(n2 + 3) / 4, 32, 4 * d1_group_smem(kFrontQ, kStageQ), st>>>(
+      k_d1_morse_group<32, kFrontQ, kStageQ, 32, 8><<<blocks(4, 32), 32, 4 * d1_group_smem(kFrontQ, kStageQ), st>>>(
           c, W, roundsA, status);
       break;
-    default:  // (0, 7) half a warp per column (two columns per warp), registers capped for 32 warps per SM
-      k_d1_morse_group<32, kFrontA, kStageA, 32, 16><<<(n2 + 1) / 2, 32, 2 * d1_group_smem(kFrontA, kStageA), st>>>(
+    case 8:  // a quarter of a warp per column with half a warp's tile
+      k_d1_morse_group<32, kFrontH, kStageH, 32, 8><<<blocks(4, 32), 32, 4 * d1_group_smem(kFrontH, kStageH), st>>>(
+          c, W, roundsA, status);
+      break;
+    default:  // (7) half a warp per column (two columns per warp), registers capped for 32 warps per SM
+      k_d1_morse_group<32, kFrontA, kStageA, 32, 16><<<blocks(2, 32), 32, 2 * d1_group_smem(kFrontA, kStageA), st>>>(
           c, W, roundsA, status);
   }
   note_launch();
-  k_d1_morse_group<kThreadsB, kFrontB, kStageB><<<n2, kThreadsB, sb, st>>>(c, W, 0, status); note_launch();
+  k_d1_morse_group<kThreadsB, kFrontB, kStageB><<<blocks(1, 4), kThreadsB, sb, st>>>(c, W, 0, status); note_launch();
   k_d1_morse<<<(n2 + 63) / 64, 64, 0, st>>>(c, W, status); note_launch();
 }
-
-static_assert(sizeof(D1Ctl) <= 64, "the control block is PairScratch::counter (64 bytes)");
 
 }  // namespace tsf

@@ -18,29 +18,34 @@ struct __align__(16) FEnt {
 
 // A group is GS threads: an aligned part of a warp (GS = 8 or 16, lanes
 // [GS*k, GS*(k+1))), one warp (GS = 32) or the whole block (GS = blockDim.x
-// > 32).  Helpers for the group of the calling thread.
+// > 32).  The groups of one warp run in lockstep: they call every helper
+// together, so one instruction serves them all (with a barrier per group each
+// would run on its own from the first barrier on).  A helper takes each
+// group's own counts; loops with barriers run to the warp's largest (gmax),
+// branches with barriers are taken when any group needs them (gany).
 template <int GS>
 __device__ __forceinline__ int gtid() {
   return GS > 32 ? (int)threadIdx.x : (int)(threadIdx.x & (GS - 1));
 }
 template <int GS>
-__device__ __forceinline__ unsigned gmask() {
-  static_assert(GS > 32 || (GS >= 1 && (GS & (GS - 1)) == 0), "a part of a warp is a power of two");
-  if (GS >= 32) return 0xFFFFFFFFu;
-  // GS < 32 here; the guard keeps the shift in range when GS = 32 instantiates this line
-  constexpr unsigned low = GS >= 32 ? 0xFFFFFFFFu : ((1u << (GS & 31)) - 1u);
-  return low << ((threadIdx.x & 31u) & ~(unsigned)(GS - 1));
-}
-template <int GS>
 __device__ __forceinline__ void gsync() {
   if (GS > 32) __syncthreads();
-  else __syncwarp(gmask<GS>());
+  else __syncwarp();
+}
+// x is the same in all threads of a group.
+template <int GS>
+__device__ __forceinline__ int gmax(int x) {  // x >= 0
+  return GS < 32 ? (int)__reduce_max_sync(0xFFFFFFFFu, (unsigned)x) : x;
+}
+template <int GS>
+__device__ __forceinline__ bool gany(bool x) {
+  return GS < 32 ? __any_sync(0xFFFFFFFFu, x) != 0 : x;
 }
 
 template <int GS>
 __device__ __forceinline__ int gscan(int v, int& total, int* sm) {  // exclusive; sm: >= GS/32 + 1 ints (GS > 32)
   if (GS <= 32) {
-    const unsigned m = gmask<GS>();
+    const unsigned m = 0xFFFFFFFFu;
     const int lane = gtid<GS>();
     int inc = v;
 #pragma unroll
@@ -76,13 +81,15 @@ __device__ __forceinline__ int gscan(int v, int& total, int* sm) {  // exclusive
   return res;
 }
 
-// Descending bitonic sort of a[0..n2) (n2 a power of two) by key, 64-bit
-// values (shared or global memory of the group; its barrier orders both).
+// Descending bitonic sort of a[0..n2) (n2 a power of two, the same for the
+// groups of a warp) by key, 64-bit values (shared or global memory of the
+// group; its barrier orders both); nothing for a group that is not `on`.
 template <int GS>
-__device__ void group_sort_desc(unsigned long long* a, int n2) {
+__device__ void group_sort_desc(unsigned long long* a, int n2, bool on) {
+  const int m2 = on ? n2 : 0;
   for (int size = 2; size <= n2; size <<= 1)
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = gtid<GS>(); i < n2; i += GS) {
+      for (int i = gtid<GS>(); i < m2; i += GS) {
         int jx = i ^ stride;
         if (jx > i) {
           bool desc = (i & size) == 0;
@@ -101,7 +108,7 @@ __device__ void group_sort_desc(unsigned long long* a, int n2) {
 template <int GS>
 __device__ void group_sort_smem(FEnt* a, int n) {
   int n2 = 1;
-  while (n2 < n) n2 <<= 1;
+  while (n2 < gmax<GS>(n)) n2 <<= 1;
   for (int i = n + gtid<GS>(); i < n2; i += GS) {
     a[i].key = 0ull;
     a[i].mask = 0u;
@@ -135,7 +142,7 @@ __device__ void group_sort_reg(FEnt* a, int n) {
   constexpr int N = GS * E;
   constexpr int W = GS < 32 ? GS : 32;  // threads that exchange by shuffles
   const int tid = gtid<GS>(), lane = tid & 31;
-  const unsigned gm = gmask<GS>();
+  const unsigned gm = 0xFFFFFFFFu;
   unsigned long long k[E];
   uint32_t m[E];
 #pragma unroll

@@ -145,7 +145,7 @@ struct D1Work {
   unsigned long long* pool;
   uint32_t pool_cap;
   uint32_t* pool_head;
-  int32_t* flags;         // [0] changed, [1] number of candidate columns
+  int32_t* flags;         // [1] number of candidate columns, [2], [3] tickets of the Morse boundaries
   unsigned long long* stats;  // [0] lower stars visited, [1] max per column
   int32_t* redo;          // columns whose warp frontier overflowed
   uint4* cont;            // open columns after phase A: frontier off/size, output off/size
@@ -153,6 +153,8 @@ struct D1Work {
   int32_t* big;           // list of open columns
   int32_t* nbig;
 };
+int d1_sms();  // of the current device
+
 // D1: candidate columns (their number in W.flags[1]), Morse boundaries,
 // reduction; grids are sized by n2, the kernels read the column count.
 void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st);
