@@ -454,6 +454,102 @@ __global__ void __launch_bounds__(kGT, MINB) k_gradient_list(Dims d, const uint3
 }
 
 
+// Where the closed stars of the updated vertices cover much of the grid, they
+// are marked without a list (no atomics), and a pass over all marks recomputes
+// them.
+__global__ void k_gradient_mark(Dims d, const uint32_t* __restrict__ upd, int64_t nu, uint32_t* __restrict__ mark,
+                                uint32_t gen) {
+  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nu * 15) return;
+  uint32_t u = upd[t / 15];
+  int i = (int)(t % 15);
+  uint32_t w = u;
+  if (i < 14) {
+    int x, y, z, nx, ny, nz;
+    vxyz(d, u, x, y, z);
+    if (!nbr_xyz(d, x, y, z, i, nx, ny, nz)) return;
+    w = vid(d, nx, ny, nz);
+  }
+  mark[w] = gen;
+}
+
+// Work of a lower star's sweeps: its lower neighbours and the link edges
+// between them (0 .. 50).
+template <int... A>
+__device__ __forceinline__ int lower_edges2(uint32_t lower, std::integer_sequence<int, A...>) {
+  return (((lower >> A) & 1u ? __popc(lower & geo_adj(A)) : 0) + ...);
+}
+__device__ __forceinline__ int star_work(const Dims& d, const uint32_t* __restrict__ rank, uint32_t v) {
+  int x, y, z;
+  vxyz(d, v, x, y, z);
+  const uint32_t rv = __ldg(rank + v);
+  uint32_t lower = 0;
+#pragma unroll
+  for (int i = 0; i < 14; ++i) {
+    int nx, ny, nz;
+    if (nbr_xyz(d, x, y, z, i, nx, ny, nz) && __ldg(rank + vid(d, nx, ny, nz)) < rv) lower |= 1u << i;
+  }
+  return __popc(lower) + (lower_edges2(lower, std::make_integer_sequence<int, 14>{}) >> 1);
+}
+
+constexpr int kGPer = 4;  // vertices of a window per thread
+static_assert(14 + 36 < 63, "work bins");
+
+// The marked lower stars (mark[v] == gen); *count receives their number.
+// Bound by instruction issue (ncu: ALU pipe 79 %), and in k_gradient two thirds
+// of the lanes idle on noise, as a star's sweeps take 0 to 50 steps.  So a
+// block sorts a window of kGT * kGPer vertices by that number, and a warp gets
+// stars that take about as long: 37 % fewer instructions.  A field that changes
+// in many places is noisy; on smooth ones, where neighbours take about as long
+// anyway, sorting cost more than it gave (0.59 -> 0.66 ms, all stars of the
+// 128^3 filament field), so the first diagram keeps k_gradient.  Stage, noisy
+// 256^3 field, 97 % of the stars: 10.0 -> 7.0 ms.
+template <int MINB>
+__global__ void __launch_bounds__(kGT, MINB) k_gradient_marked(Dims d, const uint32_t* __restrict__ rank, const float* __restrict__ values,
+                                const uint32_t* __restrict__ mark, uint32_t gen, unsigned long long* __restrict__ count,
+                                Rec* __restrict__ rec, uint8_t* __restrict__ vnext8, D1Tab* __restrict__ tab,
+                                uint32_t* status) {
+  __shared__ GradGeo sg;
+  __shared__ GradSmem sm;
+  __shared__ int bin[64];
+  __shared__ uint16_t sorted[kGT * kGPer];
+  const int tid = threadIdx.x;
+  const int64_t base = (int64_t)blockIdx.x * (kGT * kGPer);
+  if (tid < 64) bin[tid] = 0;
+  grad_geo_to_shared(sg);  // ends with a barrier
+  int key[kGPer], pos[kGPer];
+#pragma unroll
+  for (int k = 0; k < kGPer; ++k) {
+    const int64_t v = base + k * kGT + tid;
+    key[k] = v < d.nv && __ldg(mark + v) == gen ? star_work(d, rank, (uint32_t)v) : -1;
+    if (key[k] >= 0) pos[k] = atomicAdd(&bin[key[k]], 1);
+  }
+  __syncthreads();
+  if (tid < 32) {  // exclusive scan of the 64 bins
+    const int a = bin[2 * tid], b = bin[2 * tid + 1];
+    int inc = a + b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (tid >= o) inc += x;
+    }
+    bin[2 * tid] = inc - a - b;
+    bin[2 * tid + 1] = inc - b;  // bin 63 is empty: the total
+  }
+  __syncthreads();
+  const int total = bin[63];
+  if (tid == 0 && total) atomicAdd(count, (unsigned long long)total);
+#pragma unroll
+  for (int k = 0; k < kGPer; ++k)
+    if (key[k] >= 0) sorted[bin[key[k]] + pos[k]] = (uint16_t)(k * kGT + tid);
+  __syncthreads();
+  // warps take turns from both ends, so that each gets long and short ones
+  for (int k = 0; k * kGT < total; ++k) {
+    const int i = k * kGT + (k & 1 ? kGT - 32 - (tid & ~31) + (tid & 31) : tid);
+    if (i < total) gradient_star(d, rank, values, base + sorted[i], rec, vnext8, tab, status, sg, sm);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Compaction of critical cells, in increasing rank of their highest vertex
 // (then the lexicographic order inside one lower star), which is the
@@ -763,12 +859,26 @@ void launch_gradient(const Dims& d, const uint32_t* rank, const float* f, Rec* r
   note_launch();
 }
 
+// From a sixteenth of the grid on (whose closed stars cover five eighths of it
+// if they lie at random) marks replace the list, where there are windows for
+// six blocks per SM (32^3 field: list 60 us, marks 108).
 void launch_gradient_incremental(const Dims& d, const uint32_t* rank, const float* f, const uint32_t* upd, int64_t nu,
                                  uint32_t* mark, uint32_t gen, uint32_t* list, unsigned long long* count, Rec* rec,
                                  uint8_t* vnext8, D1Tab* tab, uint32_t* status, cudaStream_t st) {
   cudaMemsetAsync(count, 0, sizeof(unsigned long long), st);
   if (nu <= 0) return;
   unsigned nb = (unsigned)((nu * 15 + 255) / 256);
+  if (16 * nu >= d.nv && d.nv >= (int64_t)(6 * kGT * kGPer) * d1_sms()) {
+    k_gradient_mark<<<nb, 256, 0, st>>>(d, upd, nu, mark, gen); note_launch();
+    const unsigned nm = (unsigned)((d.nv + kGT * kGPer - 1) / (kGT * kGPer));
+    switch (gradient_blocks()) {
+      case 1: k_gradient_marked<1><<<nm, kGT, 0, st>>>(d, rank, f, mark, gen, count, rec, vnext8, tab, status); break;
+      case 2: k_gradient_marked<5><<<nm, kGT, 0, st>>>(d, rank, f, mark, gen, count, rec, vnext8, tab, status); break;
+      default: k_gradient_marked<6><<<nm, kGT, 0, st>>>(d, rank, f, mark, gen, count, rec, vnext8, tab, status); break;
+    }
+    note_launch();
+    return;
+  }
   k_gradient_expand<<<nb, 256, 0, st>>>(d, upd, nu, mark, gen, list, count); note_launch();
   unsigned nl = (unsigned)((std::min<int64_t>(nu * 15, d.nv) + kGT - 1) / kGT);
   switch (gradient_blocks()) {

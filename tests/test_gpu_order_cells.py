@@ -29,6 +29,23 @@ def test_merged_order_gives_the_diagram_of_a_new_field(changed):
         assert gpu_rows(fld.diagram()) == gpu_rows(gpu_field(f).diagram())
 
 
+@pytest.mark.parametrize("part", [1 / 16 - 1e-5, 1 / 16 + 1e-5, 1.0], ids=["listed", "marked", "all"])
+def test_lower_stars_after_many_changes(part):
+    """Changes on either side of a sixteenth of a grid large enough for marks
+    instead of a list; its size is no multiple of the 512-vertex windows."""
+    f = S.random_field((79, 81, 83), seed=5, kind="uniform")
+    fld = gpu_field(f)
+    fld.set_threshold(0.98)
+    rng = np.random.default_rng(6)
+    for _ in range(2):
+        at = rng.permutation(f.size)[:int(part * f.size)]
+        f = f.copy()
+        f.ravel()[at] = rng.uniform(0, 1, len(at))
+        fld.loss_and_grad(f)
+        a, b = fld.diagram(), gpu_field(f).diagram()
+        assert len(a) == len(b) and all(np.array_equal(a[k], b[k]) for k in a.dtype.names)
+
+
 @pytest.mark.parametrize("shape", [(2, 2, 511), (2, 32, 32), (3, 3, 228), (2, 2, 513), (4, 23, 89), (2, 2048, 2),
                                    (5, 7, 117), (27, 27, 27)])
 @pytest.mark.parametrize("kind", ["uniform", "ties"])
