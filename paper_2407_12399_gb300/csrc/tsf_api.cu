@@ -105,6 +105,8 @@ struct tsf_field {
   int64_t n_updated = 0, n_gradient = 0;
   unsigned long long d1_stats[15] = {};
   int d1_cols = 0;
+  tsf_pair* out_pairs = nullptr;  // a diagram in the caller's layout
+  int cap_out = 0;
   int32_t* h_flags = nullptr;  // pinned
   double ms_diag = 0, ms_assign = 0, ms_step = 0;
   int64_t assign_rounds = 0, assign_phases = 0, assign_checks = 0;
@@ -781,6 +783,7 @@ int tsf_destroy_field(tsf_field* F) {
     dev_free(S->skip);
   }
   dev_free(F->d1ctl);
+  dev_free(F->out_pairs);
   dev_free(F->PO.d0_min);
   dev_free(F->PO.d0_killed);
   dev_free(F->PO.d0mask);
@@ -957,23 +960,19 @@ int tsf_compute_diagram(tsf_field* F, tsf_pair* out, int64_t cap, int64_t* n_out
     }
     *n_out = F->np;
     if (F->np > cap) return TSF_ECAPACITY;
-    std::vector<Pt> h(F->np);
-    ck(cudaMemcpyAsync(h.data(), F->pts, sizeof(Pt) * F->np, cudaMemcpyDeviceToHost, F->st));
-    ck(cudaStreamSynchronize(F->st));
-    std::vector<tsf_pair> o(F->np);
-    for (int i = 0; i < F->np; ++i) {
-      o[i].dim = h[i].dim;
-      o[i].essential = h[i].ess;
-      o[i].v_birth = h[i].vb;
-      o[i].v_death = h[i].vd;
-      o[i].cell_birth = h[i].cb;
-      o[i].cell_death = h[i].cd;
-      o[i].birth = h[i].b;
-      o[i].death = h[i].d;
+    // into the caller's layout on the device, then one copy
+    if (F->np > F->cap_out) {
+      dev_free(F->out_pairs);
+      F->cap_out = 0;
+      const int c = F->np + F->np / 2 + 64;
+      ck(dev_alloc(&F->out_pairs, c));
+      F->cap_out = c;
     }
-    if (F->np)
-      ck(cudaMemcpyAsync(out, o.data(), sizeof(tsf_pair) * F->np,
-                         out_on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost, F->st));
+    if (F->np) {
+      pairs_out(F->np, F->pts, F->out_pairs, F->st);
+      ck(cudaMemcpyAsync(out, F->out_pairs, sizeof(tsf_pair) * F->np,
+                         out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, F->st));
+    }
     ck(cudaStreamSynchronize(F->st));
     return TSF_OK;
   });

@@ -1,5 +1,6 @@
 // tsf_solver.cuh -- diagram points, targets and the solver's scratch buffers.
 #pragma once
+#include "../../include/tsf.h"
 #include "tsf_kernels.cuh"
 
 namespace tsf {
@@ -118,6 +119,8 @@ struct AssignStats {
   int32_t phases;     // auction eps phases (all groups)
   int32_t checks;     // auction release passes (all groups)
 };
+
+void pairs_out(int np, const Pt* pts, tsf_pair* out, cudaStream_t st);
 
 int build_diagram(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1, int n2, int n3, const PairOut& P,
                   const uint32_t* order, const float* f, SolverBufs& B, Pt* out, int cap, cudaStream_t st);
