@@ -89,21 +89,7 @@ struct __align__(16) D1Tab {
   uint32_t nkey[14];
   uint32_t pad[2];
 };
-static_assert(sizeof(D1Tab) == 144, "nine 16-byte loads per row");
-
-template <int X>
-__host__ __device__ __forceinline__ uint64_t tab_closure(const D1Tab& t) {
-  constexpr int off = 36 * X, wi = off >> 6, bi = off & 63;
-  uint64_t lo = t.q[wi] >> bi;
-  if constexpr (bi > 28) lo |= t.q[wi + 1] << (64 - bi);
-  return lo & ((1ull << 36) - 1);
-}
-__host__ __device__ inline void tab_set_closure(D1Tab& t, int x, uint64_t path) {
-  int off = 36 * x, wi = off >> 6, bi = off & 63;
-  t.q[wi] |= path << bi;
-  if (bi > 28) t.q[wi + 1] |= path >> (64 - bi);
-}
-__host__ __device__ __forceinline__ int tab_end(const D1Tab& t, int x) { return (int)((t.q[8] >> (4 * x)) & 15ull); }
+static_assert(sizeof(D1Tab) == 144, "rows start on 16-byte boundaries");
 
 // Grid helpers -------------------------------------------------------------
 struct Dims {
