@@ -30,6 +30,20 @@ constexpr uint32_t kNoOwner = 0x7FFFFFFFu;
 constexpr uint32_t kLongAdd = 64;  // whole-GPU rounds: column additions at least this long run on a warp
 constexpr int kLongCap = 1024;     // ... at most this many per block and round (the rest on one thread)
 
+// Stage failures after which nothing is reduced (results are discarded).
+__device__ __forceinline__ bool d1_failed(const uint32_t* status) {
+  return (*reinterpret_cast<const volatile uint32_t*>(status) & (kErrSpin | kErrRounds | kErrPool | kErrTrace)) != 0u;
+}
+
+// Nobody owns a row yet: a launch of its own, ahead of kernels that return
+// early after a failed stage, so that every record is one of this diagram's.
+__global__ void k_d1_init(int n1, D1Work W) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n1) return;
+  W.owner[i] = kNoOwner;
+  W.orec[i] = make_uint4(kNoOwner, 0u, 0u, 0u);
+}
+
 // Number of entries of a strictly decreasing column greater than v (loads
 // from L2: other SMs may have written the column in this kernel).
 __device__ __forceinline__ uint32_t d1_count_greater(unsigned long long v, const unsigned long long* arr,
@@ -107,11 +121,7 @@ __global__ void __launch_bounds__(kUFT) k_d1_reduce_grid(D1Work W, int n1, D1Ctl
   const long long c_start = clock64();
   // an earlier stage failed (its results are discarded): every block returns
   // before the first barrier, and the later kernels see the same bits
-  if (*reinterpret_cast<const volatile uint32_t*>(status) & (kErrSpin | kErrRounds | kErrPool | kErrTrace)) return;
-  for (int k = gt; k < n1; k += gn) {
-    W.owner[k] = kNoOwner;
-    W.orec[k] = make_uint4(kNoOwner, 0u, 0u, 0u);
-  }
+  if (d1_failed(status)) return;
   for (int j = gt; j < ncols; j += gn) {
     mark[j] = -1;
     if (W.hsize[j] > 0) listA[atomicAdd(&ctl->n[0], 1)] = j;
@@ -330,16 +340,6 @@ __device__ __forceinline__ bool rec_same(const uint4& a, const uint4& b) {
 // A record's column lies in the pool (an absent owner has none).
 __device__ __forceinline__ bool rec_ok(const uint4& r, uint32_t pool_cap) {
   return r.x == kNoOwner || (r.z > 0u && (unsigned long long)r.y + r.z <= pool_cap);
-}
-
-// Stage failures after which nothing is reduced (results are discarded).
-__device__ __forceinline__ bool d1_failed(const uint32_t* status) {
-  return (*reinterpret_cast<const volatile uint32_t*>(status) & (kErrSpin | kErrRounds | kErrPool | kErrTrace)) != 0u;
-}
-
-__global__ void k_d1_init(int n1, D1Work W) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n1) W.orec[i] = make_uint4(kNoOwner, 0u, 0u, 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -863,12 +863,14 @@ __global__ void __launch_bounds__(kLT, 1) k_d1_long(D1Work W, int n1, D1Ctl* ctl
 }
 
 // Every row's owner is paired with it.
-__global__ void k_d1_edges(int n1, D1Work W, int32_t* d1_edge) {
+__global__ void k_d1_edges(int n1, D1Work W, int32_t* d1_edge, uint32_t* status) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) W.stats[10] += W.stats[14] + W.stats[15];
-  if (i >= n1) return;
+  if (i >= n1 || d1_failed(status)) return;
   const uint32_t j = W.orec[i].x;
-  if (j != kNoOwner) d1_edge[W.cols[j]] = i;
+  if (j == kNoOwner) return;
+  if (j < (uint32_t)W.flags[1]) d1_edge[W.cols[j]] = i;
+  else atomicOr(status, kErrInconsistent);
 }
 
 // ---------------------------------------------------------------------------
@@ -908,6 +910,7 @@ void launch_d1_reduce(int n1, int n2, D1Work& W, PairOut& P, uint32_t* status, D
   const size_t words = d1_long_words(n1);
   cudaMemsetAsync(ctl, 0, sizeof(D1Ctl), st);
   if (words) cudaMemsetAsync(W.hbits, 0, words * sizeof(uint32_t), st);
+  k_d1_init<<<(n1 + 255) / 256, 256, 0, st>>>(n1, W); note_launch();
   bool listed = false;
   const int nb = n2 >= get_knob(5) ? cooperative_blocks((const void*)k_d1_reduce_grid, kUFT) : 0;
   if (nb > 0) {
@@ -917,15 +920,12 @@ void launch_d1_reduce(int n1, int n2, D1Work& W, PairOut& P, uint32_t* status, D
     listed = cooperative_launch((const void*)k_d1_reduce_grid, dim3(nb), dim3(kUFT), args, st) == cudaSuccess;
     if (!listed) cudaGetLastError();  // not launched: the warps take every column
   }
-  if (!listed) {
-    k_d1_init<<<(n1 + 255) / 256, 256, 0, st>>>(n1, W); note_launch();
-  }
   const int sms = d1_sms();
   const int warps = std::min((n2 + kColWarps - 1) / kColWarps, sms * 4);
   k_d1_columns<<<warps, kColWarps * 32, 0, st>>>(W, n1, ctl, listed, cap, max_adds, status); note_launch();
   const size_t lsm = (size_t)window * 128 + 4 * (size_t)((long_groups(n1) + 31) / 32);
   k_d1_long<<<sms, kLT, lsm, st>>>(W, n1, ctl, window, status); note_launch();
-  k_d1_edges<<<(n1 + 255) / 256, 256, 0, st>>>(n1, W, P.d1_edge); note_launch();
+  k_d1_edges<<<(n1 + 255) / 256, 256, 0, st>>>(n1, W, P.d1_edge, status); note_launch();
 }
 
 }  // namespace tsf
