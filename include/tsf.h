@@ -320,7 +320,10 @@ int64_t tsf_kernel_launches(void);
  *  12: additions a D1 column makes on a warp before it goes to a block (0:
  *      the default, 24);
  *  13: groups of 1024 rows that such a block keeps in shared memory (0: all
- *      that fit; the rest in global memory).
+ *      that fit; the rest in global memory);
+ *  14: 64-bit words of a new field's D1 column pool per critical triangle (0:
+ *      the default, 64 and at least 2^20 in all).  A diagram that runs out of
+ *      it doubles the pool and starts D1 again, at most six times.
  * Returns the previous value, or -1 for an unknown knob.  Set them only
  * while no call of this library is running. */
 int64_t tsf_debug_set(int what, int64_t value);

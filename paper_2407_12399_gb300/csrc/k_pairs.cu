@@ -63,6 +63,9 @@ std::atomic<int64_t> g_morse_rounds{0};
 // (0: all that fit)
 std::atomic<int64_t> g_chain_max{0};
 std::atomic<int64_t> g_long_window{0};
+// words of the D1 column pool per critical triangle in the first attempt (0:
+// the default, see compute_diagram)
+std::atomic<int64_t> g_pool_words{0};
 
 static std::atomic<int64_t>* knob(int what) {
   return what == 1   ? &g_uf_grid_min
@@ -78,6 +81,7 @@ static std::atomic<int64_t>* knob(int what) {
          : what == 11 ? &g_morse_rounds
          : what == 12 ? &g_chain_max
          : what == 13 ? &g_long_window
+         : what == 14 ? &g_pool_words
                      : nullptr;
 }
 
@@ -955,10 +959,16 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
   const int gi = (int)threadIdx.x / GS;
   FEnt* other = front + FCAP;
   FEnt* stage = other + FCAP;
-  __shared__ int sg_nf[G], sg_flag[G], sg_ntot[G], sg_otot[G];
+  __shared__ int sg_nf[G], sg_flag[G], sg_full[G], sg_ntot[G], sg_otot[G];
   __shared__ Vec sg_out[G], sg_grow[G], sg_fr[G];
   int& s_nf = sg_nf[gi];
+  // s_flag: a visit's updates were dropped (set by any thread between two
+  // barriers, read after the second).  s_full: the pool had no room (set by
+  // thread 0 right before a barrier at each allocation, read right after it): a
+  // word of its own, as slower warps may still be reading s_flag when thread 0
+  // allocates.  Every branch with barriers depends on such settled words only.
   int& s_flag = sg_flag[gi];
+  int& s_full = sg_full[gi];
   int& s_ntot = sg_ntot[gi];
   int& s_otot = sg_otot[gi];
   Vec& s_out = sg_out[gi];
@@ -1012,6 +1022,7 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
   }
   int visits = 0, updates = 0, rounds = 0;
   bool failed = s_flag != 0;
+  gsync<GS>();  // before the first visits, which may set it
   bool handoff = false;
   bool run = live && !failed;
   for (;;) {
@@ -1049,19 +1060,20 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
     // outputs: append to the column's list in the pool (grown by the group)
     const int otot = run ? s_otot : 0;
     if (gany<GS>(otot > 0)) {
-      if (tid == 0 && otot > 0) {
+      if (tid == 0) {
         s_grow.h = nullptr;
-        if (s_out.size + otot > s_out.cap) {
+        s_full = 0;
+        if (otot > 0 && s_out.size + otot > s_out.cap) {
           uint32_t cap = s_out.cap;
           while (cap < s_out.size + otot) cap *= 2;
           if (!vec_alloc(W, s_grow, cap, status)) {
             s_grow.h = nullptr;
-            s_flag = 1;
+            s_full = 1;
           }
         }
       }
       gsync<GS>();
-      if (run && s_flag) {
+      if (run && s_full) {
         failed = true;
         run = false;
       }
@@ -1093,9 +1105,9 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
         failed = true;
         run = false;
       }
-      if (save && tid == 0 && !vec_alloc(W, s_fr, 2u * (uint32_t)(rest + ntot), status)) s_flag = 1;
+      if (save && tid == 0) s_full = vec_alloc(W, s_fr, 2u * (uint32_t)(rest + ntot), status) ? 0 : 1;
       gsync<GS>();
-      if (save && !s_flag) {
+      if (save && !s_full) {
         handoff = true;
         for (int i = tid; i < rest; i += GS) fent_save(s_fr.h + 2 * i, front[nb + i]);
         for (int i = tid; i < ntot; i += GS) fent_save(s_fr.h + 2 * (rest + i), stage[i]);
@@ -1137,9 +1149,9 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
   bool redo = live && failed && !handoff;
   const bool open = live && !failed && !phase_b && s_nf > 0;  // still open after max_rounds: save the frontier for phase B
   if (gany<GS>(open)) {
-    if (open && tid == 0 && !vec_alloc(W, s_fr, 2u * (uint32_t)s_nf, status)) s_flag = 1;
+    if (open && tid == 0) s_full = vec_alloc(W, s_fr, 2u * (uint32_t)s_nf, status) ? 0 : 1;
     gsync<GS>();
-    redo = redo || (open && s_flag);
+    redo = redo || (open && s_full);
     if (open && !redo)
       for (int i = tid; i < s_nf; i += GS) fent_save(s_fr.h + 2 * i, front[i]);
     gsync<GS>();
@@ -1166,9 +1178,9 @@ __device__ __forceinline__ void d1_column(const D1Ctx& c, D1Work& W, int j, bool
   n2 = gmax<GS>(n2);
   unsigned long long* a = reinterpret_cast<unsigned long long*>(stage);
   if (n2 > 2 * SCAP) {  // too long for shared memory: sort in the pool
-    if (fin && tid == 0 && !vec_alloc(W, s_grow, (uint32_t)n2, status)) s_flag = 1;
+    if (fin && tid == 0) s_full = vec_alloc(W, s_grow, (uint32_t)n2, status) ? 0 : 1;
     gsync<GS>();
-    if (fin && s_flag) {
+    if (fin && s_full) {
       redo = true;
       fin = false;
       nout = 0;

@@ -497,9 +497,11 @@ int compute_diagram(tsf_field* F, bool incremental) {
   stage_end(F, kD2);
   // D1, growing the column pool until it suffices (D0 and D2 report through
   // the same status word, read after the first attempt)
+  const int64_t pool_knob = get_knob(14), pool0 = pool_knob > 0
+                                                      ? std::min<int64_t>(pool_knob, 1 << 20) * std::max(F->n2, 1)
+                                                      : std::max<int64_t>((int64_t)64 * std::max(F->n2, 1), 1 << 20);
   for (int attempt = 0;; ++attempt) {
-    uint32_t want = (uint32_t)std::min<int64_t>(std::max<int64_t>((int64_t)64 * std::max(F->n2, 1), 1 << 20) << attempt,
-                                                 (int64_t)1 << 31);
+    uint32_t want = (uint32_t)std::min<int64_t>(pool0 << attempt, (int64_t)1 << 31);
     if (want > F->pool_cap) {
       dev_free(F->W.pool);
       ck(dev_alloc(&F->W.pool, want));
