@@ -323,7 +323,9 @@ int64_t tsf_kernel_launches(void);
  *      that fit; the rest in global memory);
  *  14: 64-bit words of a new field's D1 column pool per critical triangle (0:
  *      the default, 64 and at least 2^20 in all).  A diagram that runs out of
- *      it doubles the pool and starts D1 again, at most six times.
+ *      it doubles the pool and starts D1 again, at most six times;
+ *  15: polls of a sort's look-back before it gives up and makes the call fail
+ *      with TSF_ETIMEOUT (0: the default, 2^24; negative: gives up at once).
  * Returns the previous value, or -1 for an unknown knob.  Set them only
  * while no call of this library is running. */
 int64_t tsf_debug_set(int what, int64_t value);

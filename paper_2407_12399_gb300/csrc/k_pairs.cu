@@ -66,6 +66,9 @@ std::atomic<int64_t> g_long_window{0};
 // words of the D1 column pool per critical triangle in the first attempt (0:
 // the default, see compute_diagram)
 std::atomic<int64_t> g_pool_words{0};
+// polls of a sort's look-back before it gives up (k_sort.cu; 0: the default,
+// negative: none at all)
+std::atomic<int64_t> g_sort_polls{0};
 
 static std::atomic<int64_t>* knob(int what) {
   return what == 1   ? &g_uf_grid_min
@@ -82,6 +85,7 @@ static std::atomic<int64_t>* knob(int what) {
          : what == 12 ? &g_chain_max
          : what == 13 ? &g_long_window
          : what == 14 ? &g_pool_words
+         : what == 15 ? &g_sort_polls
                      : nullptr;
 }
 

@@ -2651,9 +2651,9 @@ __global__ void k_grad_keys(int n, const Grad64* __restrict__ G, uint32_t* __res
 }
 
 __global__ void k_loss_grad_apply(int n, const int32_t* __restrict__ idx, const Grad64* __restrict__ G,
-                                  double* __restrict__ grad) {
+                                  double* __restrict__ grad, const uint32_t* __restrict__ status) {
   int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
+  if (r >= n || (*status & kErrSpin)) return;  // a sort that gave up leaves no usable indices
   uint32_t v = G[idx[r]].v;
   if (r > 0 && G[idx[r - 1]].v == v) return;
   double acc = 0.0;
@@ -2676,7 +2676,7 @@ void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* gr
     k_grad_keys<<<(n + 255) / 256, 256, 0, st>>>(n, G, key, iota); note_launch();
     sort_u32_pairs(key, iota, n, nullptr, reinterpret_cast<uint32_t*>(idx), iota + n, status, st);
   }
-  k_loss_grad_apply<<<(2 * np + 255) / 256, 256, 0, st>>>(2 * np, idx, G, grad); note_launch();
+  k_loss_grad_apply<<<(2 * np + 255) / 256, 256, 0, st>>>(2 * np, idx, G, grad, status); note_launch();
 }
 
 // New field values: copies the changed ones and lists their vertices, so

@@ -122,6 +122,14 @@ void exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* 
 constexpr uint32_t kLbAgg = 1u << 30, kLbInc = 2u << 30, kLbVal = (1u << 30) - 1;
 constexpr int kSpinLimit = 1 << 24;
 
+// Polls a tile's look-back makes at most (every earlier tile takes one).  A
+// look-back that gives up sets kErrSpin, and its sort leaves places of the
+// output unwritten: whoever uses them as indices checks the word first.
+static int os_polls() {
+  const int64_t k = get_knob(15);
+  return k == 0 ? kSpinLimit : (int)std::min<int64_t>(std::max<int64_t>(k, 0), kSpinLimit);
+}
+
 // Counts one key's four digits: the low two vary from key to key, the high two
 // often agree across a warp and are added once per value.
 __device__ __forceinline__ void os_count(uint32_t (*h)[256], uint32_t k, bool in, int lane) {
@@ -193,7 +201,8 @@ __global__ void __launch_bounds__(kRT) k_os_pass(int64_t n, int shift, bool firs
                                                  const uint32_t* __restrict__ keys_in,
                                                  const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
                                                  uint32_t* __restrict__ vals_out, const uint32_t* __restrict__ hist,
-                                                 uint32_t* lookback, uint32_t* tile_counter, uint32_t* status) {
+                                                 uint32_t* lookback, uint32_t* tile_counter, int polls,
+                                                 uint32_t* status) {
   __shared__ uint32_t whist[kRW][256];
   __shared__ uint32_t s_off[256];   // output position of a digit's run minus its place in the tile
   __shared__ uint32_t s_sw[kRW];
@@ -261,15 +270,13 @@ __global__ void __launch_bounds__(kRT) k_os_pass(int64_t n, int shift, bool firs
     int64_t t = (int64_t)tile - 1;
     int spins = 0;
     while (t >= 0) {
+      if (spins++ >= polls) {
+        atomicOr(status, kErrSpin);
+        break;
+      }
       uint32_t word = lb[t * 256 + d];
       uint32_t flag = word & ~kLbVal;
-      if (flag == 0) {
-        if (++spins > kSpinLimit) {
-          atomicOr(status, kErrSpin);
-          break;
-        }
-        continue;
-      }
+      if (flag == 0) continue;
       excl += word & kLbVal;
       if (flag == kLbInc) break;
       --t;
@@ -322,6 +329,7 @@ void sort_u32_pairs(const uint32_t* keys, const uint32_t* vals, int64_t n, uint3
   uint32_t* lookback = counters + 64;
   cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (1024 + 64 + 4 * 256 * (size_t)ntiles), st);
   k_os_hist_u32<<<os_hist_blocks(n), 256, 0, st>>>(n, keys, hist); note_launch();
+  const int polls = os_polls();
   const uint32_t* kin = keys;
   const uint32_t* vin = vals;
   for (int pass = 0; pass < 4; ++pass) {
@@ -330,7 +338,7 @@ void sort_u32_pairs(const uint32_t* keys, const uint32_t* vals, int64_t n, uint3
     uint32_t* vout = last ? vals_out : ((pass & 1) ? vB : vA);
     if (!last && !kout) kout = (pass & 1) ? kB : kA;
     k_os_pass<<<ntiles, kRT, 0, st>>>(n, 8 * pass, false, nullptr, kin, vin, kout, vout, hist + 256 * pass,
-                                      lookback + (size_t)pass * 256 * ntiles, counters + pass, status); note_launch();
+                                      lookback + (size_t)pass * 256 * ntiles, counters + pass, polls, status); note_launch();
     kin = kout;
     vin = vout;
   }
@@ -355,6 +363,7 @@ void vertex_order(const float* f, int64_t n, uint32_t* order, uint32_t* rank, ui
   uint32_t* lookback = counters + 64;
   cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (1024 + 64 + 4 * 256 * (size_t)ntiles), st);
   k_os_hist<<<os_hist_blocks(n), 256, 0, st>>>(n, f, hist, status); note_launch();
+  const int polls = os_polls();
   const uint32_t* kin = nullptr;
   const uint32_t* vin = nullptr;
   for (int pass = 0; pass < 4; ++pass) {
@@ -362,7 +371,7 @@ void vertex_order(const float* f, int64_t n, uint32_t* order, uint32_t* rank, ui
     uint32_t* kout = last ? skey : ((pass & 1) ? kB : kA);
     uint32_t* vout = last ? order : ((pass & 1) ? vB : vA);
     k_os_pass<<<ntiles, kRT, 0, st>>>(n, 8 * pass, first, f, kin, vin, kout, vout, hist + 256 * pass,
-                                      lookback + (size_t)pass * 256 * ntiles, counters + pass, status); note_launch();
+                                      lookback + (size_t)pass * 256 * ntiles, counters + pass, polls, status); note_launch();
     kin = kout;
     vin = vout;
   }

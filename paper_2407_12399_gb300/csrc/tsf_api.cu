@@ -1105,15 +1105,17 @@ int tsf_loss_and_gradient(tsf_field* F, const float* values, int values_on_devic
     if (r) return r;
     eval(F, 0.0f);
     *loss = F->loss;
+    F->h_flags[0] = 0;
     if (grad) {
       if (!F->lgrad) ck(dev_alloc(&F->lgrad, (size_t)F->d.nv));
       loss_gradient(F->np, F->pts, F->T, F->B, F->lgrad, F->d.nv, F->status, F->st);
       ck(cudaMemcpyAsync(grad, F->lgrad, sizeof(double) * F->d.nv,
                          grad_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, F->st));
+      ck(cudaMemcpyAsync(F->h_flags, F->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, F->st));
     }
     ck(cudaStreamSynchronize(F->st));
     ck(cudaGetLastError());
-    return TSF_OK;
+    return status_code((uint32_t)F->h_flags[0]);
   });
 }
 

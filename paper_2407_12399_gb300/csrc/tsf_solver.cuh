@@ -132,7 +132,7 @@ void targets_as_points(int nt, const Tg* T, Pt* R, cudaStream_t st);
 void replace_values(int64_t nv, const float* in, float* f, uint32_t* upd, unsigned long long* count,
                     cudaStream_t st);
 // dL/df (fp64, nv entries) of the topological loss for the current points
-// and their matching.
+// and their matching.  Sorts: the caller reads the status word afterwards.
 void loss_gradient(int np, const Pt* pts, const Tg* T, SolverBufs& B, double* grad, int64_t nv, uint32_t* status,
                    cudaStream_t st);
 int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double prec, SolverBufs& B, uint32_t* status,
