@@ -186,9 +186,9 @@ __global__ void k_key64(int n, const int* __restrict__ n_dev, KeyFn kf, uint32_t
 }
 
 __global__ void k_gather_u32(int n, const uint32_t* __restrict__ src, const uint32_t* __restrict__ perm,
-                             uint32_t* __restrict__ dst) {
+                             uint32_t* __restrict__ dst, const uint32_t* __restrict__ status) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[perm[i]];
+  if (i < n) dst[i] = *status & kErrSpin ? 0u : src[perm[i]];
 }
 
 // A key function as a comparator: equal keys in index order.
@@ -213,7 +213,7 @@ static int32_t* radix_sort64(int n, const int* n_dev, KeyFn kf, uint32_t* rs, in
   k_key64<<<nb, 256, 0, st>>>(n, n_dev, kf, lo, hi, iota); note_launch();
   uint32_t* p1 = reinterpret_cast<uint32_t*>(tmp);
   sort_u32_pairs(lo, iota, n, nullptr, p1, scratch, status, st);
-  k_gather_u32<<<nb, 256, 0, st>>>(n, hi, p1, hi2); note_launch();
+  k_gather_u32<<<nb, 256, 0, st>>>(n, hi, p1, hi2, status); note_launch();
   sort_u32_pairs(hi2, p1, n, nullptr, reinterpret_cast<uint32_t*>(out), scratch, status, st);
   return out;
 }
@@ -505,8 +505,19 @@ __device__ __forceinline__ int key_cmp(const Pt& x, const Pt& y) {
 // the whole list: 1.3 ms for 3e6 points, 0.38 ms now).
 __global__ void __launch_bounds__(256) k_still(int np, const Pt* __restrict__ cur, const int32_t* __restrict__ ck,
                                                int nr, const Pt* __restrict__ ref, const int32_t* __restrict__ rk,
-                                               Pt* __restrict__ out, uint8_t* __restrict__ taken) {
+                                               Pt* __restrict__ out, uint8_t* __restrict__ taken,
+                                               const uint32_t* __restrict__ status) {
   __shared__ int range[2];
+  if (*status & kErrSpin) {  // a sort gave up, no usable orders: every point unmatched
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < np) {
+      Pt p = cur[i];
+      p.tgt = -1;
+      p.still = 0;
+      out[i] = p;
+    }
+    return;
+  }
   const int r = blockIdx.x * 256 + threadIdx.x, last = min((int)blockIdx.x * 256 + 255, np - 1);
   // first reference index in [a, b) with a key not below x's (`past`: above it)
   auto bound = [&](const Pt& x, int a, int b, bool past) {
@@ -2307,7 +2318,8 @@ int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double p
     else if (radix) rk = radix_sort64(nr, nullptr, KeyBits{ref}, B.rsort, B.idxD, B.idxC, status, st);
     else rk = merge_sort(nr, B.idxC, B.idxD, KeyLess{ref}, st);
   }
-  k_still<<<(np + 255) / 256, 256, 0, st>>>(np, pts, ck, nr, ref, rk, B.tmp_pts, B.taken); note_launch();
+  k_still<<<(np + 255) / 256, 256, 0, st>>>(np, pts, ck, nr, ref, rk, B.tmp_pts, B.taken, status);
+  note_launch();
   cudaMemcpyAsync(pts, B.tmp_pts, sizeof(Pt) * (size_t)np, cudaMemcpyDeviceToDevice, st);
   cudaMemcpyAsync(B.keyord, ck, sizeof(int32_t) * (size_t)np, cudaMemcpyDeviceToDevice, st);
   B.keyord_for = pts;
@@ -2564,8 +2576,11 @@ struct ContribBits {  // ContribLess as one 64-bit key
 // one thread per vertex segment: acc = +0, acc += c in increasing value order
 __global__ void k_apply_step(int nc, const int* __restrict__ nc_dev, const int32_t* __restrict__ idx,
                              const Contrib* __restrict__ C, float* __restrict__ f, uint32_t* __restrict__ upd,
-                             unsigned long long* __restrict__ nupd) {
+                             unsigned long long* __restrict__ nupd, const uint32_t* __restrict__ status) {
   int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t s = *status;
+  if (r == 0) nupd[1] = s;
+  if (s & kErrSpin) return;  // a sort that gave up leaves no usable indices
   if (nc_dev) nc = min(*nc_dev, nc);
   if (r >= nc) return;
   uint32_t v = C[idx[r]].v;
@@ -2582,7 +2597,9 @@ __global__ void k_apply_step(int nc, const int* __restrict__ nc_dev, const int32
 }
 
 int64_t gradient_step(int np, const Pt* pts, const Tg* T, float alpha_b, float alpha_d, float* f, uint32_t* upd,
-                      SolverBufs& B, uint32_t* status, cudaStream_t st) {
+                      SolverBufs& B, uint32_t* status, uint32_t* h_status, cudaStream_t st) {
+  *h_status = 0;
+  cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
   cudaMemsetAsync(B.count, 0, sizeof(int), st);
   cudaMemsetAsync(B.counters, 0, sizeof(unsigned long long), st);
   if (np == 0) return 0;
@@ -2591,12 +2608,14 @@ int64_t gradient_step(int np, const Pt* pts, const Tg* T, float alpha_b, float a
   int32_t* idx = 2 * np <= B.cap_rsort
                      ? radix_sort64(2 * np, B.count, ContribBits{B.contrib}, B.rsort, B.idxB, B.idxA, status, st)
                      : merge_sort(2 * np, B.idxA, B.idxB, ContribLess{B.contrib}, st, B.count);
-  k_apply_step<<<(2 * np + 255) / 256, 256, 0, st>>>(2 * np, B.count, idx, B.contrib, f, upd, B.counters);
+  k_apply_step<<<(2 * np + 255) / 256, 256, 0, st>>>(2 * np, B.count, idx, B.contrib, f, upd, B.counters,
+                                                           status);
   note_launch();
-  unsigned long long nupd = 0;
-  cudaMemcpyAsync(&nupd, B.counters, sizeof(nupd), cudaMemcpyDeviceToHost, st);
+  unsigned long long nupd[2] = {0, 0};  // vertices updated, status word
+  cudaMemcpyAsync(nupd, B.counters, sizeof(nupd), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
-  return (int64_t)nupd;
+  *h_status = (uint32_t)nupd[1];
+  return (int64_t)nupd[0];
 }
 
 // ---------------------------------------------------------------------------

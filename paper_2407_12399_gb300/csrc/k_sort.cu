@@ -19,9 +19,14 @@ __device__ __forceinline__ uint32_t rs_key(bool first, const float* __restrict__
   return first ? value_key(__ldg(f + i)) : __ldg(keys + i);
 }
 
-__global__ void k_rank_scatter(int64_t n, const uint32_t* __restrict__ order, uint32_t* __restrict__ rank) {
+// After a sort that gave up the order is no permutation; any permutation keeps
+// the kernels that follow in bounds until the status word is read.
+__global__ void k_rank_scatter(int64_t n, uint32_t* __restrict__ order, uint32_t* __restrict__ rank,
+                               const uint32_t* __restrict__ status) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) rank[__ldg(order + i)] = (uint32_t)i;
+  if (i >= n) return;
+  if (*status & kErrSpin) order[i] = (uint32_t)i;
+  rank[order[i]] = (uint32_t)i;
 }
 
 // ---- exclusive scan of uint32 (block sums, one-block scan, apply) ---------
@@ -375,7 +380,7 @@ void vertex_order(const float* f, int64_t n, uint32_t* order, uint32_t* rank, ui
     kin = kout;
     vin = vout;
   }
-  k_rank_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, order, rank); note_launch();
+  k_rank_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, order, rank, status); note_launch();
 }
 
 }  // namespace tsf

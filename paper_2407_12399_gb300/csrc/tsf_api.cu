@@ -474,12 +474,11 @@ int compute_diagram(tsf_field* F, bool incremental) {
   ck(cudaMemcpyAsync(&tot, F->totals, sizeof(int4), cudaMemcpyDeviceToHost, st));
   ck(cudaMemcpyAsync(&s, F->status, sizeof(s), cudaMemcpyDeviceToHost, st));
   ck(cudaStreamSynchronize(st));
-  if (s & kErrNaN) {
+  if (status_code(s) != TSF_OK) {  // no order, or one of values that have none
     F->order_valid = false;
     F->records_valid = false;
-    return TSF_ENAN;
+    return status_code(s);
   }
-  if (status_code(s) != TSF_OK) return status_code(s);
   F->n_gradient = (int64_t)ngrad;
   F->n0 = tot.x;
   F->n1 = tot.y;
@@ -572,7 +571,10 @@ int run_assign(tsf_field* F, const Pt* ref, int nr, double prec = 0.0) {
     // the failed pass may have written partial assignments: restart from the still step
   }
   uint32_t s = as.status_valid ? as.status : read_status(F);
-  if (status_code(s) != TSF_OK) return status_code(s);
+  if (status_code(s) != TSF_OK) {
+    F->B.keyord_for = nullptr;  // the points' key order may be incomplete
+    return status_code(s);
+  }
   F->ms_assign = now_ms() - t0;
   F->assign_rounds = as.rounds;
   F->assign_phases = as.phases;
@@ -666,9 +668,12 @@ int step(tsf_field* F, const tsf_params* p, tsf_stats* stats) {
   double t0 = now_ms();
   bool fast = p->fast_gradient_update != 0;
   stage_begin(F, kStep);
-  F->n_updated =
-      gradient_step(F->np, F->pts, F->T, p->alpha_b, p->alpha_d, F->f, fast ? F->upd : nullptr, F->B, F->status, st);
+  uint32_t s = 0;
+  const int64_t nupd = gradient_step(F->np, F->pts, F->T, p->alpha_b, p->alpha_d, F->f, fast ? F->upd : nullptr, F->B,
+                                     F->status, &s, st);
   stage_end(F, kStep);
+  if (status_code(s) != TSF_OK) return status_code(s);  // nothing has changed
+  F->n_updated = nupd;
   F->upd_valid = fast;
   F->ms_step = now_ms() - t0;
   // previous diagram (with its assignment) becomes the still-pair reference
@@ -1221,8 +1226,11 @@ int tsf_zero_pairs(tsf_field* F, uint64_t* out, int64_t cap_pairs, int64_t* n_ou
     ck(cudaMemsetAsync(F->status, 0, 4, F->st));
     vertex_order(F->f, F->d.nv, F->order, F->rank, F->skey, F->sort_scratch, F->status, F->st);
     uint32_t s = read_status(F);
-    F->order_valid = !(s & kErrNaN);
-    if (s & kErrNaN) return TSF_ENAN;
+    F->order_valid = status_code(s) == TSF_OK;
+    if (!F->order_valid) {
+      F->records_valid = false;
+      return status_code(s);
+    }
     unsigned long long* dout = nullptr;
     int64_t cap = std::max<int64_t>(cap_pairs, 1);
     ck(dev_alloc(&dout, 2 * (size_t)cap));

@@ -140,8 +140,9 @@ int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double p
 void loss_and_counts(int np, const Pt* pts, int nt, const Tg* T, float cancel_eps, SolverBufs& B, double* h_loss,
                      unsigned long long* h_counts, cudaStream_t st);
 // One gradient step (Eq. 3); returns the number of vertices whose value
-// changed and, with upd non-null, lists them there.
+// changed and, with upd non-null, lists them there.  *h_status receives the
+// status word, cleared before; no value changes when a sort gave up.
 int64_t gradient_step(int np, const Pt* pts, const Tg* T, float alpha_b, float alpha_d, float* f, uint32_t* upd,
-                      SolverBufs& B, uint32_t* status, cudaStream_t st);
+                      SolverBufs& B, uint32_t* status, uint32_t* h_status, cudaStream_t st);
 
 }  // namespace tsf
