@@ -604,6 +604,20 @@ __global__ void k_cand_count(int npg, const int32_t* __restrict__ plist, const P
   if (threadIdx.x == 0) cnt[t] = s;
 }
 
+// *total = sum of the k counts, in 64 bits (k targets x npg points can exceed 32).
+__global__ void __launch_bounds__(1024) k_cand_total(int k, const uint32_t* __restrict__ cnt,
+                                                     unsigned long long* __restrict__ total) {
+  __shared__ unsigned long long s;
+  if (threadIdx.x == 0) s = 0ull;
+  __syncthreads();
+  unsigned long long c = 0ull;
+  for (int t = threadIdx.x; t < k; t += 1024) c += cnt[t];
+  for (int o = 16; o; o >>= 1) c += __shfl_down_sync(0xFFFFFFFFu, c, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&s, c);
+  __syncthreads();
+  if (threadIdx.x == 0) *total = s;
+}
+
 __global__ void k_cand_fill(int npg, const int32_t* __restrict__ plist, const Pt* __restrict__ pts, int k,
                             const int32_t* __restrict__ tlist, const Tg* __restrict__ T,
                             const uint32_t* __restrict__ off, Cand* __restrict__ cands) {
@@ -2301,8 +2315,10 @@ int assign_groups(int np, Pt* pts, int nt, const Tg* T, double prec, SolverBufs&
 constexpr int kParts = 16, kPartPoints = 1 << 14;  // parts per target, points from which they are used
 
 // Assignment phi*_j.  `ref` is the previous diagram (or the targets at j = 0,
-// each assigned to itself).  Returns 0, or a negative value when a scratch
-// buffer is too small (the caller grows it and retries).
+// each assigned to itself).  Returns 0, or a negative value: -2 and -3 when a
+// scratch buffer (candidates, columns) is too small for as->need entries (the
+// caller grows it and retries), -4 when a cooperative launch was refused, -5
+// for more than kMaxCand candidates.
 int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double prec, SolverBufs& B,
            uint32_t* status, AssignStats* as, cudaStream_t st) {
   // 1) still pairs
@@ -2374,6 +2390,8 @@ int assign(int np, Pt* pts, int nr, const Pt* ref, int nt, const Tg* T, double p
   return assign_groups(np, pts, nt, T, prec, B, status, as, st);
 }
 
+constexpr int kMaxCand = 1 << 30;  // candidates of a group (32-bit positions; 40 GB of buffers)
+
 // General path: group by group with host-sized buffers.
 int assign_groups(int np, Pt* pts, int nt, const Tg* T, double prec, SolverBufs& B, uint32_t* status,
                   AssignStats* as, cudaStream_t st) {
@@ -2399,9 +2417,17 @@ int assign_groups(int np, Pt* pts, int nt, const Tg* T, double prec, SolverBufs&
     }
     if (k > B.cap_k) return -1;
     k_cand_count<<<k, 256, 0, st>>>(npg, B.plist, pts, k, B.tlist, T, B.u32a); note_launch();
+    k_cand_total<<<1, 1024, 0, st>>>(k, B.u32a, B.counters); note_launch();
     exclusive_scan_u32(B.u32a, B.u32b, k, B.u32c, st);
-    int nc = (int)read_tail(B.u32a, B.u32b, k, st);
-    if (nc > B.cap_cand) return -2;
+    unsigned long long total = 0;
+    cudaMemcpyAsync(&total, B.counters, sizeof(total), cudaMemcpyDeviceToHost, st);
+    cudaStreamSynchronize(st);
+    if (total > (unsigned long long)kMaxCand) return -5;
+    const int nc = (int)total;
+    if (nc > B.cap_cand) {
+      as->need = nc;
+      return -2;
+    }
     if (nc == 0) continue;
     k_cand_fill<<<k, 256, 0, st>>>(npg, B.plist, pts, k, B.tlist, T, B.u32b, B.cands); note_launch();
     int32_t* ci = merge_sort(nc, B.idxC, B.idxD, CandLess{B.cands}, st);
@@ -2410,7 +2436,10 @@ int assign_groups(int np, Pt* pts, int nt, const Tg* T, double prec, SolverBufs&
     k_cand_keep<<<(nc + 255) / 256, 256, 0, st>>>(nc, ci, B.cands, B.u32b, k, B.is_col, B.kept, B.nkept); note_launch();
     exclusive_scan_u32(B.is_col, B.colpos, npg, B.u32c, st);
     int mc = (int)read_tail(B.is_col, B.colpos, npg, st);
-    if (mc + k + 1 > B.cap_cols) return -3;
+    if (mc + k + 1 > B.cap_cols) {
+      as->need = mc + k + 1;
+      return -3;
+    }
     k_colpos<<<(npg + 255) / 256, 256, 0, st>>>(npg, B.is_col, B.colpos, B.colpos, B.col_point); note_launch();
     k_diag_t<<<(k + 255) / 256, 256, 0, st>>>(k, B.tlist, T, B.diag_t); note_launch();
     if (prec > 0.0 && k >= kGridMin) {

@@ -371,20 +371,29 @@ void grow_solver(tsf_field* F, int np, int nt) {
 void grow_assign(tsf_field* F, int cand, int cols) {
   SolverBufs& B = F->B;
   if (cand > B.cap_cand) {
-    int c = cand + cand / 2 + 1024;
+    int c = cand + std::min(cand / 2, 1 << 26) + 1024;
+    if (c + 64 > F->cap_idxcd) {  // candidate sorts use idxC/idxD
+      int ci = c + 64;
+      int32_t *ic = nullptr, *id = nullptr;  // others use them too: kept if there is no room
+      cudaError_t e = dev_alloc(&ic, ci);
+      if (e == cudaSuccess) e = dev_alloc(&id, ci);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        dev_free(ic);
+        ck(e);
+      }
+      dev_free(B.idxC);
+      dev_free(B.idxD);
+      B.idxC = ic;
+      B.idxD = id;
+      F->cap_idxcd = ci;
+    }
     dev_free(B.cands);
     dev_free(B.kept);
+    B.cap_cand = 0;
     ck(dev_alloc(&B.cands, c));
     ck(dev_alloc(&B.kept, c));
     B.cap_cand = c;
-    if (c + 64 > F->cap_idxcd) {  // candidate sorts use idxC/idxD
-      int ci = c + 64;
-      dev_free(B.idxC);
-      dev_free(B.idxD);
-      ck(dev_alloc(&B.idxC, ci));
-      ck(dev_alloc(&B.idxD, ci));
-      F->cap_idxcd = ci;
-    }
   }
   if (cols > B.cap_cols) {
     int c = cols + cols / 2 + 1024;
@@ -401,6 +410,7 @@ void grow_assign(tsf_field* F, int cand, int cols) {
     dev_free(H.bw);
     dev_free(B.aux);
     dev_free(B.col_to_row);
+    B.cap_cols = 0;
     ck(dev_alloc(&H.u, c + 1));
     ck(dev_alloc(&H.v, c + 1));
     ck(dev_alloc(&H.minv, c + 1));
@@ -557,17 +567,19 @@ int compute_diagram(tsf_field* F, bool incremental) {
 int run_assign(tsf_field* F, const Pt* ref, int nr, double prec = 0.0) {
   double t0 = now_ms();
   AssignStats as{};
-  for (int attempt = 0; attempt < 8; ++attempt) {
+  for (int attempt = 0;; ++attempt) {
     as.status_valid = false;
     ck(cudaMemsetAsync(F->status, 0, 4, F->st));
     stage_begin(F, kAssign);
     int r = assign(F->np, F->pts, nr, ref, F->nt, F->T, prec, F->B, F->status, &as, F->st);
     stage_end(F, kAssign);
     if (r == 0) break;
-    if (r == -2) grow_assign(F, std::max(2 * F->B.cap_cand, 4096), 0);
-    else if (r == -3) grow_assign(F, 0, std::max(2 * F->B.cap_cols, 4096));
-    else if (r == -4) return TSF_ECUDA;  // a cooperative launch was refused
-    else return TSF_EINTERNAL;
+    if (r == -4) return TSF_ECUDA;  // a cooperative launch was refused
+    if (r == -5) return TSF_ENOMEM;
+    // each of the three groups may find each of the two buffers too small once
+    if ((r != -2 && r != -3) || attempt >= 6) return TSF_EINTERNAL;
+    if (r == -2) grow_assign(F, std::max(as.need, 4096), 0);
+    else grow_assign(F, 0, std::max(as.need, 4096));
     // the failed pass may have written partial assignments: restart from the still step
   }
   uint32_t s = as.status_valid ? as.status : read_status(F);

@@ -113,6 +113,7 @@ int64_t radix_sort64_words(int64_t n);
 
 struct AssignStats {
   int k[4];
+  int need;           // entries that a buffer found too small has to have
   uint32_t status;    // the status word, read with the group counts (fast path)
   bool status_valid;
   int32_t rounds;     // auction rounds (all groups)
