@@ -98,7 +98,9 @@ struct tsf_field {
   int np = 0, nprev = 0;
   Tg* T = nullptr;
   int nt = 0;
-  bool have_targets = false, diagram_current = false, records_valid = false, upd_valid = false;
+  bool have_targets = false, records_valid = false, upd_valid = false;
+  // pts is the current values' diagram; ... and carries their assignment
+  bool diagram_current = false, matched = false;
   int iter = 0;
   double loss = 0, loss0 = 0;
   unsigned long long counts[4] = {0, 0, 0, 0};
@@ -441,6 +443,11 @@ static_assert(TSF_ENAN == -2 && TSF_ETIMEOUT == -5 && TSF_EINTERNAL == -8, "stat
 int compute_diagram(tsf_field* F, bool incremental) {
   cudaStream_t st = F->st;
   double t0 = now_ms();
+  // until this one is complete there is no current diagram (its points replace
+  // F->pts, whose key order is kept for it only as long as they stay)
+  F->diagram_current = F->matched = false;
+  F->np = 0;
+  if (F->B.keyord_for == F->pts) F->B.keyord_for = nullptr;
   ck(cudaMemsetAsync(F->status, 0, 4, st));
   stage_begin(F, kSort);
   if (incremental && F->order_valid && F->upd_valid && F->n_updated <= kIncOrderMax) {
@@ -587,6 +594,7 @@ int run_assign(tsf_field* F, const Pt* ref, int nr, double prec = 0.0) {
     F->B.keyord_for = nullptr;  // the points' key order may be incomplete
     return status_code(s);
   }
+  F->matched = true;
   F->ms_assign = now_ms() - t0;
   F->assign_rounds = as.rounds;
   F->assign_phases = as.phases;
@@ -675,8 +683,20 @@ int check_params(const tsf_params* p) {
   return TSF_OK;
 }
 
+// The current values' diagram and assignment, where an earlier call failed
+// before it had them: from nothing, every point matched by the exact solver.
+int ensure_matched(tsf_field* F) {
+  if (F->matched) return TSF_OK;
+  if (!F->diagram_current) {
+    int r = compute_diagram(F, false);
+    if (r) return r;
+  }
+  return run_assign(F, F->prev, 0);
+}
+
 int step(tsf_field* F, const tsf_params* p, tsf_stats* stats) {
   cudaStream_t st = F->st;
+  if (int r = ensure_matched(F)) return r;
   double t0 = now_ms();
   bool fast = p->fast_gradient_update != 0;
   stage_begin(F, kStep);
@@ -1078,6 +1098,7 @@ int tsf_simplify(tsf_field* F, const tsf_params* p, float* out_values, int out_o
   if (check_params(p)) return TSF_EINVAL;
   if (!F->have_targets) return TSF_ENOTARGET;
   return guarded_f(F, [&]() {
+    if (int r = ensure_matched(F)) return r;
     eval(F, p->cancel_eps);
     int done = is_done(F, p);
     fill_stats(F, p, stats, done);
@@ -1156,11 +1177,12 @@ int tsf_set_start_field(tsf_field* F, const float* values, int values_on_device)
     F->upd_valid = true;
     // the current diagram (with its assignment) is the still-pair reference
     // of the start field's diagram, as after a solver step (Section 4.3)
+    const bool reuse = F->matched;
     std::swap(F->pts, F->prev);
     F->nprev = F->np;
     int r = compute_diagram(F, true);
     if (r) return r;
-    r = run_assign(F, F->prev, F->nprev);
+    r = run_assign(F, F->prev, reuse ? F->nprev : 0);
     if (r) return r;
     F->iter = 0;
     eval(F, 0.0f);

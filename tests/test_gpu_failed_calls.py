@@ -1,0 +1,60 @@
+"""Calls that fail, and the calls after them: no diagram or assignment of earlier
+values is taken for the current one."""
+import numpy as np
+import pytest
+
+import oracle
+
+from .test_gpu_parity import NAMED, bits, gpu_field, gpu_rows, oracle_rows
+
+pytestmark = pytest.mark.gpu
+
+ROUND_CAP = 3
+
+
+def test_nothing_of_earlier_values_is_returned_for_a_nan_field():
+    import paper_2407_12399_gb300 as tsf
+    f = NAMED["plain_32"]()
+    fld = gpu_field(f)
+    fld.set_threshold(0.1)
+    bad = f.copy()
+    bad[3, 4, 5] = np.nan
+    for call in (lambda: fld.loss_and_grad(bad), fld.diagram, lambda: fld.step(stop_s=0.0), fld.simplify):
+        with pytest.raises(tsf.TsfError) as e:
+            call()
+        assert e.value.code == tsf.TSF_ENAN
+    rng = np.random.default_rng(5)
+    g = (f + rng.uniform(-0.01, 0.01, f.shape)).astype(np.float32)
+    loss, grad = fld.loss_and_grad(g)
+    other = gpu_field(f)
+    other.set_threshold(0.1)
+    want_loss, want = other.loss_and_grad(g)
+    assert loss == want_loss and np.array_equal(grad.view(np.uint64), want.view(np.uint64))
+    assert gpu_rows(fld.diagram()) == oracle_rows(g, oracle.diagram(g)["pairs"])
+
+
+@pytest.mark.parametrize("name,tau", [("plain_32", 0.1), ("filament_64", 0.05)])
+def test_a_step_after_a_failed_one_matches_the_current_diagram(name, tau):
+    """The failed step has moved the values; the next one starts from their
+    diagram, matched as without the reuse of the previous assignment."""
+    import paper_2407_12399_gb300 as tsf
+    f = NAMED[name]()
+    fld = gpu_field(f)
+    fld.set_threshold(tau)
+    old = tsf.tsf_debug_set(ROUND_CAP, 1)
+    try:
+        with pytest.raises(tsf.TsfError) as e:
+            fld.step(stop_s=0.0)
+    finally:
+        tsf.tsf_debug_set(ROUND_CAP, old)
+    assert e.value.code == tsf.TSF_ETIMEOUT
+    want = gpu_field(f)
+    want.set_threshold(tau)
+    want.step(stop_s=0.0, fast_assignment_update=0)
+    assert np.array_equal(bits(fld.values()), bits(want.values()))
+    assert gpu_rows(fld.diagram()) == gpu_rows(want.diagram())
+    for _ in range(2):
+        fld.step(stop_s=0.0)
+        want.step(stop_s=0.0)
+        assert np.array_equal(bits(fld.values()), bits(want.values()))
+        assert [x.tolist() for x in fld.assignment()] == [x.tolist() for x in want.assignment()]
