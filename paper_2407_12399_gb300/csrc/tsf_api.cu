@@ -1281,7 +1281,6 @@ int tsf_zero_pairs(tsf_field* F, uint64_t* out, int64_t cap_pairs, int64_t* n_ou
     dev_free(dout);
     s = read_status(F);
     if (status_code(s) != TSF_OK) return status_code(s);
-    F->diagram_current = false;
     return rc;
   });
 }

@@ -1,5 +1,5 @@
 """Calls that fail, and the calls after them: no diagram or assignment of earlier
-values is taken for the current one."""
+values is taken for the current one.  A call that only looks leaves both."""
 import numpy as np
 import pytest
 
@@ -58,3 +58,17 @@ def test_a_step_after_a_failed_one_matches_the_current_diagram(name, tau):
         want.step(stop_s=0.0)
         assert np.array_equal(bits(fld.values()), bits(want.values()))
         assert [x.tolist() for x in fld.assignment()] == [x.tolist() for x in want.assignment()]
+
+
+def test_zero_pairs_leave_the_diagram_and_its_assignment():
+    f = NAMED["plain_32"]()
+    fld, want = gpu_field(f), gpu_field(f)
+    for x in (fld, want):
+        x.set_threshold(0.1)
+    for _ in range(2):
+        for x in (fld, want):
+            x.step(stop_s=0.0)
+        assert len(fld.zero_pairs()) > 0
+        assert gpu_rows(fld.diagram()) == gpu_rows(want.diagram())
+        assert [x.tolist() for x in fld.assignment()] == [x.tolist() for x in want.assignment()]
+    assert np.array_equal(bits(fld.values()), bits(want.values()))
