@@ -229,10 +229,10 @@ int tsf_batch_simplify(tsf_batch* batch, const tsf_params* params, tsf_stats* st
 /* Autotuner of the batch (not in the paper): times the full persistence
  * diagram of every field (all fields concurrently, each candidate twice,
  * the second pass counted) for each candidate schedule of the D1 Morse
- * boundaries' first phase — 0: half a warp per column with 64 + 128
- * frontier and stage entries, 1: half a warp with 32 + 64, 2: a quarter of
- * a warp with 16 + 32, 3: one warp with 64 + 128 (tsf_debug_set knob 7
- * values 7, 5, 6, 4) — and keeps the fastest.  The choice applies
+ * boundaries' first phase — 0: the default, by each diagram's size, 1: a
+ * quarter of a warp per column with 32 + 64 frontier and stage entries, 2: a
+ * quarter of a warp with 16 + 32, 3: one warp with 64 + 128 (tsf_debug_set
+ * knob 7 values 0, 8, 6, 4) — and keeps the fastest.  The choice applies
  * process-wide; results never depend on it.  *choice receives it (0..3),
  * ms[c] (cap entries, may be NULL when cap is 0) the time of candidate c in
  * milliseconds.  Call it before the signal thresholds are set (it replaces

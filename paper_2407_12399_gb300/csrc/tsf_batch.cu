@@ -159,11 +159,12 @@ int tsf_batch_step(tsf_batch* b, const tsf_params* params, tsf_stats* stats) {
 
 int tsf_batch_autotune(tsf_batch* b, int* choice, double* ms, int cap) {
   if (!b || !choice || cap < 0 || (cap > 0 && !ms)) return TSF_EINVAL;
-  // candidates: the D1 Morse boundaries' first phase (knob 7): half a warp
-  // per column with 64 + 128 frontier and stage entries, half a warp with
-  // 32 + 64, a quarter of a warp with 16 + 32, one warp with 64 + 128
+  // candidates: the D1 Morse boundaries' first phase (knob 7): by each
+  // diagram's size, so that tuning a batch of small fields does not pin a
+  // schedule on large ones unless it is faster, and each of the three
+  // schedules that the sizes choose from
   constexpr int kCand = 4;
-  constexpr int64_t kKnob[kCand] = {7, 5, 6, 4};
+  constexpr int64_t kKnob[kCand] = {0, 8, 6, 4};
   const int64_t keep = tsf::get_knob(7);
   double best = -1.0;
   int arg = 0;
