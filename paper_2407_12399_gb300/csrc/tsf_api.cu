@@ -504,13 +504,22 @@ int compute_diagram(tsf_field* F, bool incremental) {
   grow_crit(F, F->n0, F->n1, F->n2, F->n3);
   launch_crit_write(F->d, F->order, F->rank, F->rec, pack, F->tile_counts, F->L, F->cidx, F->c1base, F->c2base, st);
   stage_end(F, kCrit);
-  stage_begin(F, kD0);
-  launch_traces(F->d, F->nd, F->L, F->n0, F->n1, F->n2, F->n3, F->rank, F->rec, F->vnext8, F->cidx, F->S0, F->S2,
-                F->PO, F->status, st);
-  stage_end(F, kD0);
-  stage_begin(F, kD2);
-  launch_union_find(F->L, F->n0, F->n1, F->n2, F->n3, F->S0, F->S2, F->PO, F->status, st);
-  stage_end(F, kD2);
+  // D0 and D2 pairs, in shared launches unless each is timed on its own
+  auto pairs = [&](int n0, int n1, int n2, int n3) {
+    launch_traces(F->d, F->nd, F->L, n0, n1, n2, n3, F->rank, F->rec, F->vnext8, F->cidx, F->S0, F->S2, F->PO,
+                  F->status, st);
+    launch_union_find(F->L, n0, n1, n2, n3, F->S0, F->S2, F->PO, F->status, st);
+  };
+  if (F->prof) {
+    stage_begin(F, kD0);
+    pairs(F->n0, F->n1, 0, 0);
+    stage_end(F, kD0);
+    stage_begin(F, kD2);
+    pairs(0, 0, F->n2, F->n3);
+    stage_end(F, kD2);
+  } else {
+    pairs(F->n0, F->n1, F->n2, F->n3);
+  }
   // D1, growing the column pool until it suffices (D0 and D2 report through
   // the same status word, read after the first attempt)
   const int64_t pool_knob = get_knob(14), pool0 = pool_knob > 0
