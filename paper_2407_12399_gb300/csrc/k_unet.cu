@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "tsf_unet.cuh"
@@ -1042,8 +1043,8 @@ namespace {
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
-bool g_attr_set[64] = {};
+std::atomic<EncodeTiledFn> g_encode{nullptr};  // networks may run in several host threads
+std::atomic<bool> g_attr_set[64] = {};
 }  // namespace
 
 // Planes as (2 * lx, ly, lz, chunks) 8-byte elements, two per voxel, so that a
@@ -1053,13 +1054,15 @@ bool g_attr_set[64] = {};
 // multiples of two elements, 16 bytes.
 int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz, int chunks, int bx, int by, int bz,
                       int bchunks) {
-  if (!g_encode) {
+  EncodeTiledFn encode = g_encode.load(std::memory_order_acquire);
+  if (!encode) {
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess || !fn)
       return -1;
-    g_encode = reinterpret_cast<EncodeTiledFn>(fn);
+    encode = reinterpret_cast<EncodeTiledFn>(fn);
+    g_encode.store(encode, std::memory_order_release);
   }
   const uint64_t nv = static_cast<uint64_t>(lx) * ly * lz;
   cuuint64_t dims[4] = {2 * static_cast<cuuint64_t>(lx), static_cast<cuuint64_t>(ly), static_cast<cuuint64_t>(lz),
@@ -1068,7 +1071,7 @@ int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz
   cuuint32_t box[4] = {2 * static_cast<cuuint32_t>(bx), static_cast<cuuint32_t>(by), static_cast<cuuint32_t>(bz),
                        static_cast<cuuint32_t>(bchunks)};
   cuuint32_t es[4] = {1, 1, 1, 1};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(base), dims, strides, box, es,
+  CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(base), dims, strides, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
@@ -1163,11 +1166,11 @@ int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaSt
   if (encode_planes_map(&map, in_planes, a.lx, a.ly, a.lz, in_chunks, p.pitch, p.ty + 2, 1, in_chunks) != 0) return -2;
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !g_attr_set[dev]) {
+  if (dev >= 0 && dev < 64 && !g_attr_set[dev].load(std::memory_order_acquire)) {
     for (const Kernel k : {k_conv_tc<0>, k_conv_tc<1>, k_conv_tc<2>, k_conv_tc<2, true>, k_conv_tc<3>, k_conv_tc<4>,
                            k_conv_tc<6>})
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kConvSmem));
-    g_attr_set[dev] = true;
+    g_attr_set[dev].store(true, std::memory_order_release);
   }
   const size_t smem = static_cast<size_t>(kConvSmemFixed) + static_cast<size_t>(p.stages) * p.a_bytes +
                       static_cast<size_t>(p.b_slots) * p.b_bytes;
@@ -1259,12 +1262,12 @@ int launch_wgrad(const void* x, int cin, int cin_real, const void* gz, int cout,
   if (encode_planes_map(&xm, x, lx, ly, lz, cin / 8, p.pitch, p.ty, 3, p.cin_chunks) != 0 ||
       encode_planes_map(&gm, gz, lx, ly, lz, p.cout_chunks, p.tx, p.ty, 1, p.cout_chunks) != 0)
     return -2;
-  static bool attr[64] = {};
+  static std::atomic<bool> attr[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !attr[dev]) {
+  if (dev >= 0 && dev < 64 && !attr[dev].load(std::memory_order_acquire)) {
     cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kWgSmem) + 1024);
-    attr[dev] = true;
+    attr[dev].store(true, std::memory_order_release);
   }
   k_wgrad_tc<<<dim3(p.blocks, p.groups), kWgThreads, static_cast<size_t>(p.stages) * p.stage_bytes + 1024, st>>>(
       xm, gm, p, partial, bpartial, status);
