@@ -23,6 +23,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "tsf_kernels.cuh"
 #include "tsf_unet.cuh"
 
 namespace tsf {
@@ -1089,7 +1090,7 @@ ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
   const int ksteps = chunks / 2, taps = single ? 14 : 9;
   const int b_bytes = single ? 2 * cout * 16 : ksteps * 2 * 3 * cout * 16;  // weights of a tap (of a pair of taps)
   const int room = static_cast<int>(kConvSmem) - kConvSmemFixed;
-  const int min_x = (lx + kConvTx - 1) / kConvTx;
+  const int min_x = (lx + kConvTx - 1) / kConvTx, sms = tsf::d1_sms();
   for (int tiles_x = min_x; tiles_x <= min_x + 3; ++tiles_x) {
     const int tx = (lx + tiles_x - 1) / tiles_x, pitch = tx + 2;
     for (int tz = 1; tz <= 16; ++tz) {
@@ -1135,7 +1136,7 @@ ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
         const double loads = (tz + 2) * (p.a_tx + (p.b_resident ? 0.0 : static_cast<double>(taps) * b_bytes)) / 30.0;
         const double epilogue = 120.0 * p.mtiles * tz * (cout / 16);
         const int64_t tiles = static_cast<int64_t>(tiles_x) * tiles_y * p.tiles_z;
-        const double time = static_cast<double>((tiles + kConvSms - 1) / kConvSms) *
+        const double time = static_cast<double>((tiles + sms - 1) / sms) *
                                 std::max(std::max(mma + 1200.0, loads), epilogue) + std::min(mma, loads) / 2 + epilogue;
         if (best.tx == 0 || time < best_time) {
           best = p;
@@ -1174,7 +1175,7 @@ int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaSt
   }
   const size_t smem = static_cast<size_t>(kConvSmemFixed) + static_cast<size_t>(p.stages) * p.a_bytes +
                       static_cast<size_t>(p.b_slots) * p.b_bytes;
-  kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, kConvSms), kConvThreads, smem, st>>>(map, a);
+  kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, tsf::d1_sms()), kConvThreads, smem, st>>>(map, a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
 
@@ -1204,7 +1205,7 @@ void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void*
       planes, lx, ly, lz, static_cast<uint4*>(out));
 }
 
-int head_blocks(int64_t nv) { return static_cast<int>(std::min<int64_t>((nv + 255) / 256, kConvSms)); }
+int head_blocks(int64_t nv) { return static_cast<int>(std::min<int64_t>((nv + 255) / 256, tsf::d1_sms())); }
 
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
                           double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st) {
@@ -1230,7 +1231,7 @@ WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout) {
   // rows per step: four stages in shared memory, and four steps for every
   // block (each block's partial is written and read once more)
   const int row_bytes = 16 * (3 * p.cin_chunks * p.pitch + p.copies * p.cout_chunks * p.tx);
-  int blocks = std::max(kConvSms / p.groups, 1);
+  int blocks = std::max(tsf::d1_sms() / p.groups, 1);
   const int by_smem = std::max(static_cast<int>(kWgSmem / kWgStagesMax) / row_bytes, 1);
   const int by_steps = std::max(static_cast<int>(static_cast<int64_t>(ly) * lz * p.tiles_x / (4 * blocks)), 1);
   p.ty = std::min(std::min(by_smem, by_steps), std::min(ly, 256));

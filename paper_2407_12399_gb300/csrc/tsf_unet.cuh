@@ -16,7 +16,6 @@ constexpr int kConvBSlotsMax = 14;             // taps' weights in shared memory
 constexpr size_t kConvSmem = 220 * 1024;       // dynamic shared memory, one block per SM
 constexpr int kConvSmemFixed = 1024;           // ... of which alignment
 constexpr int kConvTx = 126;                   // voxels of a tile along x: a row with its halo is one TMA run
-constexpr int kConvSms = 152;
 constexpr uint32_t kUnetErrSpin = 1u << 5;     // a bounded wait gave up (same bit as the solver's)
 
 enum ConvMode { kConvForward = 0, kConvDgrad = 1, kConvHead = 2 };
