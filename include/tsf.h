@@ -325,7 +325,9 @@ int64_t tsf_kernel_launches(void);
  *      the default, 64 and at least 2^20 in all).  A diagram that runs out of
  *      it doubles the pool and starts D1 again, at most six times;
  *  15: polls of a sort's look-back before it gives up and makes the call fail
- *      with TSF_ETIMEOUT (0: the default, 2^24; negative: gives up at once).
+ *      with TSF_ETIMEOUT (0: the default, 2^24; negative: gives up at once);
+ *  16: device allocations of the fields until one is refused, as if the
+ *      device were full (counts down; 0: none is).
  * Returns the previous value, or -1 for an unknown knob.  Set them only
  * while no call of this library is running. */
 int64_t tsf_debug_set(int what, int64_t value);

@@ -69,6 +69,8 @@ std::atomic<int64_t> g_pool_words{0};
 // polls of a sort's look-back before it gives up (k_sort.cu; 0: the default,
 // negative: none at all)
 std::atomic<int64_t> g_sort_polls{0};
+// device allocations of the fields until one is refused (0: none is)
+std::atomic<int64_t> g_alloc_fail{0};
 
 static std::atomic<int64_t>* knob(int what) {
   return what == 1   ? &g_uf_grid_min
@@ -86,12 +88,20 @@ static std::atomic<int64_t>* knob(int what) {
          : what == 13 ? &g_long_window
          : what == 14 ? &g_pool_words
          : what == 15 ? &g_sort_polls
+         : what == 16 ? &g_alloc_fail
                      : nullptr;
 }
 
 int64_t get_knob(int what) {
   std::atomic<int64_t>* k = knob(what);
   return k ? k->load() : -1;
+}
+
+bool refuse_allocation() {
+  int64_t k = g_alloc_fail.load(std::memory_order_relaxed);
+  while (k > 0)
+    if (g_alloc_fail.compare_exchange_weak(k, k - 1)) return k == 1;
+  return false;
 }
 
 int64_t set_knob(int what, int64_t value) {

@@ -30,7 +30,10 @@ template <class T>
 cudaError_t dev_alloc(T** p, size_t n) {
   *p = nullptr;
   if (n == 0) n = 1;
-  return cudaMalloc((void**)p, n * sizeof(T));
+  if (refuse_allocation()) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
+  if (e != cudaSuccess) cudaGetLastError();  // returned here: not the next call's error too
+  return e;
 }
 template <class T>
 void dev_free(T*& p) {
@@ -172,15 +175,20 @@ void grow_pairs(PairScratch& S, int& cap_items, int items, int& cap_nodes, int n
   }
 }
 
+// Buffers that grow: a capacity counts only while all of its buffers exist (it
+// is zero from the first one freed to the last one allocated), so that a call
+// after one that ran out of memory allocates them again.
 void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
   auto need = [](int have, int want) { return want > have ? std::max(want + want / 2, 1024) : have; };
   int c0 = need(F->cap_c0, n0), c1 = need(F->cap_c1, n1), c2 = need(F->cap_c2, n2), c3 = need(F->cap_c3, n3);
   if (c0 != F->cap_c0) {
+    F->cap_c0 = 0;
     dev_free(F->L.c0);
     ck(dev_alloc(&F->L.c0, c0));
     F->cap_c0 = c0;
   }
   if (c1 != F->cap_c1) {
+    F->cap_c1 = 0;
     dev_free(F->L.c1_key);
     dev_free(F->L.c1_vn);
     dev_free(F->PO.d0_min);
@@ -196,6 +204,7 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
     F->cap_c1 = c1;
   }
   if (c2 != F->cap_c2) {
+    F->cap_c2 = 0;
     dev_free(F->L.c2_ve);
     dev_free(F->PO.d2_max);
     dev_free(F->PO.d1_edge);
@@ -206,10 +215,6 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
     dev_free(F->W.hsize);
     dev_free(F->W.lowc);
     dev_free(F->W.redo);
-  dev_free(F->W.cont);
-  dev_free(F->W.cont_cap);
-  dev_free(F->W.big);
-  dev_free(F->W.nbig);
     dev_free(F->W.cont);
     dev_free(F->W.cont_cap);
     dev_free(F->W.big);
@@ -230,6 +235,7 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
     F->cap_c2 = c2;
   }
   if (c3 != F->cap_c3) {
+    F->cap_c3 = 0;
     dev_free(F->L.c3);
     ck(dev_alloc(&F->L.c3, c3));
     F->cap_c3 = c3;
@@ -245,14 +251,22 @@ void grow_crit(tsf_field* F, int n0, int n1, int n2, int n3) {
 void grow_solver(tsf_field* F, int np, int nt) {
   bool again = np > F->cap_pts || nt > F->cap_t;
   if (!again) return;
-  int cp = std::max(np + np / 2 + 64, F->cap_pts);
-  int ctt = std::max(nt + nt / 2 + 64, F->cap_t);
+  int cp = std::max(std::max(np + np / 2 + 64, F->cap_pts), std::max(F->np, F->nprev));
+  int ctt = std::max(std::max(nt + nt / 2 + 64, F->cap_t), F->nt);
   int ci = std::max(2 * cp, ctt) + 64;
   SolverBufs& B = F->B;
   // points (current/previous) keep their contents across a resize
   Pt *np_ = nullptr, *pp_ = nullptr;
-  ck(dev_alloc(&np_, cp));
-  ck(dev_alloc(&pp_, cp));
+  Tg* nt_ = nullptr;
+  cudaError_t e = dev_alloc(&np_, cp);
+  if (e == cudaSuccess) e = dev_alloc(&pp_, cp);
+  if (e == cudaSuccess) e = dev_alloc(&nt_, ctt);
+  if (e != cudaSuccess) {  // as it was
+    dev_free(np_);
+    dev_free(pp_);
+    ck(e);
+  }
+  F->cap_pts = F->cap_t = 0;
   if (F->pts && F->np) ck(cudaMemcpyAsync(np_, F->pts, sizeof(Pt) * F->np, cudaMemcpyDeviceToDevice, F->st));
   if (F->prev && F->nprev) ck(cudaMemcpyAsync(pp_, F->prev, sizeof(Pt) * F->nprev, cudaMemcpyDeviceToDevice, F->st));
   ck(cudaStreamSynchronize(F->st));
@@ -260,8 +274,6 @@ void grow_solver(tsf_field* F, int np, int nt) {
   dev_free(F->prev);
   F->pts = np_;
   F->prev = pp_;
-  Tg* nt_ = nullptr;
-  ck(dev_alloc(&nt_, ctt));
   if (F->T && F->nt) ck(cudaMemcpyAsync(nt_, F->T, sizeof(Tg) * F->nt, cudaMemcpyDeviceToDevice, F->st));
   ck(cudaStreamSynchronize(F->st));
   dev_free(F->T);
@@ -380,7 +392,6 @@ void grow_assign(tsf_field* F, int cand, int cols) {
       cudaError_t e = dev_alloc(&ic, ci);
       if (e == cudaSuccess) e = dev_alloc(&id, ci);
       if (e != cudaSuccess) {
-        cudaGetLastError();
         dev_free(ic);
         ck(e);
       }
@@ -529,6 +540,7 @@ int compute_diagram(tsf_field* F, bool incremental) {
     uint32_t want = (uint32_t)std::min<int64_t>(pool0 << attempt, (int64_t)1 << 31);
     if (want > F->pool_cap) {
       dev_free(F->W.pool);
+      F->pool_cap = 0;
       ck(dev_alloc(&F->W.pool, want));
       F->pool_cap = want;
     }
@@ -700,6 +712,7 @@ int ensure_matched(tsf_field* F) {
     int r = compute_diagram(F, false);
     if (r) return r;
   }
+  grow_solver(F, F->np, F->nt);
   return run_assign(F, F->prev, 0);
 }
 

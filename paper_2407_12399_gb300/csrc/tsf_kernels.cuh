@@ -30,6 +30,8 @@ void sort_u32_pairs(const uint32_t* keys, const uint32_t* vals, int64_t n, uint3
 // previous value, -1 for an unknown knob.
 int64_t set_knob(int what, int64_t value);
 int64_t get_knob(int what);
+// Counts down knob 16; true for the allocation it asks to refuse.
+bool refuse_allocation();
 
 // Number of kernels this library has launched (process-wide).
 void note_launch();

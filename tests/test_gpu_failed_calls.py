@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2407_12399_gb300 import synthetic as S
 
 from .test_gpu_parity import NAMED, bits, gpu_field, gpu_rows, oracle_rows
 
@@ -72,3 +73,56 @@ def test_zero_pairs_leave_the_diagram_and_its_assignment():
         assert gpu_rows(fld.diagram()) == gpu_rows(want.diagram())
         assert [x.tolist() for x in fld.assignment()] == [x.tolist() for x in want.assignment()]
     assert np.array_equal(bits(fld.values()), bits(want.values()))
+
+
+ALLOC = 16
+
+
+def _solve(fld, f):
+    fld.set_threshold(0.1)
+    fld.step(stop_s=0.0)
+    v = fld.values()
+    loss, grad = fld.loss_and_grad(f)
+    return bits(v).tobytes(), gpu_rows(fld.diagram()), loss, grad.tobytes()
+
+
+def test_every_refused_allocation_is_reported_and_the_field_goes_on():
+    """Refuses the n-th device allocation for every n that a field needs: of a new
+    field, and of a field whose buffers have to grow.  The call fails with
+    TSF_ENOMEM; a diagram small enough for the old buffers and the solve that
+    failed then both work."""
+    import torch
+
+    import paper_2407_12399_gb300 as tsf
+    f = NAMED["plain_32"]()
+    small = S.linear_field(f.shape)
+    dev, small_dev = torch.from_numpy(f).cuda(), torch.from_numpy(small).cuda()
+    want = _solve(gpu_field(f), f)
+    want_small = gpu_rows(gpu_field(small).diagram())
+
+    for grown in (False, True):
+        refused = 0
+        for n in range(1, 1000):
+            fld = None
+            if grown:
+                fld = tsf.Field(small_dev)
+                fld.set_threshold(0.1)
+                tsf.tsf_set_field(fld._h, dev.data_ptr(), 1)
+            tsf.tsf_debug_set(ALLOC, n)
+            try:
+                fld = fld or tsf.Field(dev)
+                _solve(fld, f)
+            except tsf.TsfError as e:
+                assert e.code == tsf.TSF_ENOMEM
+                refused += 1
+            finally:
+                left = tsf.tsf_debug_set(ALLOC, 0)
+            if fld is not None:
+                tsf.tsf_set_field(fld._h, small_dev.data_ptr(), 1)
+                assert gpu_rows(fld.diagram()) == want_small
+                tsf.tsf_set_field(fld._h, dev.data_ptr(), 1)
+                assert _solve(fld, f) == want
+                fld.close()
+            if left > 0:  # fewer than n allocations in all
+                break
+        assert refused > (40 if grown else 80) and left > 0
