@@ -14,11 +14,6 @@ constexpr int kRI = 16;             // items per thread
 constexpr int kRTile = kRT * kRI;   // 4096 items per tile
 constexpr int kRWarpItems = kRTile / kRW;  // 512 items per warp, contiguous
 
-__device__ __forceinline__ uint32_t rs_key(bool first, const float* __restrict__ f, const uint32_t* __restrict__ keys,
-                                           int64_t i) {
-  return first ? value_key(__ldg(f + i)) : __ldg(keys + i);
-}
-
 // After a sort that gave up the order is no permutation; any permutation keeps
 // the kernels that follow in bounds until the status word is read.
 __global__ void k_rank_scatter(int64_t n, uint32_t* __restrict__ order, uint32_t* __restrict__ rank,
@@ -127,12 +122,13 @@ void exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* 
 constexpr uint32_t kLbAgg = 1u << 30, kLbInc = 2u << 30, kLbVal = (1u << 30) - 1;
 constexpr int kSpinLimit = 1 << 24;
 
-// Polls a tile's look-back makes at most (every earlier tile takes one).  A
-// look-back that gives up sets kErrSpin, and its sort leaves places of the
-// output unwritten: whoever uses them as indices checks the word first.
+// Polls in vain that a tile's look-back makes at most; negative: it looks at
+// nothing and gives up.  A look-back that gives up sets kErrSpin, and its sort
+// leaves places of the output unwritten: whoever uses them as indices checks the
+// word first.
 static int os_polls() {
   const int64_t k = get_knob(15);
-  return k == 0 ? kSpinLimit : (int)std::min<int64_t>(std::max<int64_t>(k, 0), kSpinLimit);
+  return k == 0 ? kSpinLimit : (int)std::min<int64_t>(std::max<int64_t>(k, -1), kSpinLimit);
 }
 
 // Counts one key's four digits: the low two vary from key to key, the high two
@@ -201,8 +197,9 @@ __device__ __forceinline__ uint32_t exscan256(uint32_t v, uint32_t* sw) {
 // One digit: a tile's keys are ranked, moved to their places in the tile's
 // digit order in shared memory, and written from there, so that the keys of a
 // digit leave as one run (written from the registers, 16.8 M pairs took 364 us
-// a pass, 272 us now).
-__global__ void __launch_bounds__(kRT) k_os_pass(int64_t n, int shift, bool first, const float* __restrict__ f,
+// a pass, 272 us now).  Two blocks fit an SM (128 registers a thread; with 142
+// one does, and a pass takes 0.1 ms longer).
+__global__ void __launch_bounds__(kRT, 2) k_os_pass(int64_t n, int shift, bool first, const float* __restrict__ f,
                                                  const uint32_t* __restrict__ keys_in,
                                                  const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
                                                  uint32_t* __restrict__ vals_out, const uint32_t* __restrict__ hist,
@@ -275,13 +272,15 @@ __global__ void __launch_bounds__(kRT) k_os_pass(int64_t n, int shift, bool firs
     int64_t t = (int64_t)tile - 1;
     int spins = 0;
     while (t >= 0) {
-      if (spins++ >= polls) {
-        atomicOr(status, kErrSpin);
-        break;
-      }
-      uint32_t word = lb[t * 256 + d];
+      uint32_t word = polls < 0 ? 0u : lb[t * 256 + d];
       uint32_t flag = word & ~kLbVal;
-      if (flag == 0) continue;
+      if (flag == 0) {
+        if (++spins > polls) {
+          atomicOr(status, kErrSpin);
+          break;
+        }
+        continue;
+      }
       excl += word & kLbVal;
       if (flag == kLbInc) break;
       --t;
