@@ -227,7 +227,6 @@ __global__ void __launch_bounds__(kUFT) k_d1_reduce_grid(D1Work W, int n1, D1Ctl
     if (gt == 0) {
       ctl->n[which ^ 1] = 0;  // the list the next round fills
       ctl->which = which;
-      ctl->rounds = round + 1;
       W.stats[5] = (unsigned long long)(round + 1);
       W.stats[8] += 1;
       W.stats[9] += (unsigned long long)(clock64() - c_round);

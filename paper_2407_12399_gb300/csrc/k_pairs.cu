@@ -40,19 +40,19 @@ std::atomic<int64_t> g_barrier_limit{1 << 24};
 // rounds down to 2^12, 0.33 ms without
 std::atomic<int64_t> g_d1_grid_min{1 << 18};
 std::atomic<int64_t> g_d1_handoff{1 << 17};
-// schedule of the D1 Morse boundaries' phase A: 0 the default (half a warp
-// per column, 64 frontier + 128 stage entries for diagrams of at least 2^19
-// critical triangles, else as 5), 1 and 2 one warp with 128 +
-// 256 and 256 + 512, 3 one warp with 64 + 128 uncapped, 4 capped, 5 half a
-// warp with 32 + 64, 6 a quarter of a warp with 16 + 32, 7 half a warp
-// with 64 + 128 at any size
+// schedule of the D1 Morse boundaries' phase A, as threads per column and its
+// frontier + stage entries: 0 the default (8 for diagrams of at least 2^19
+// critical triangles, 4 below 2^13, else 6), 1 and 2 one warp with 128 + 256 and
+// 256 + 512, 3 one warp with 64 + 128 uncapped, 4 capped, 5 half a warp with 32 +
+// 64, 6 a quarter of a warp with 16 + 32, 7 half a warp with 64 + 128, 8 a
+// quarter of a warp with 32 + 64
 std::atomic<int64_t> g_d1_phase_a{0};
 // blocks per SM the lower-star gradient kernels are compiled for: 0 the
 // default (six), 1 no register cap, 2 five
 std::atomic<int64_t> g_gradient_blocks{0};
 // entries of a column that a warp of the D1 reduction keeps in shared memory
 // (at most 256; longer columns go to a block)
-std::atomic<int64_t> g_chain_cap{512};
+std::atomic<int64_t> g_chain_cap{256};
 // D1 Morse boundaries: visits a thread chains per round along single-target
 // updates (0: the default), rounds of the first phase before a column moves
 // to a block (0: the default); both defaults depend on the diagram's size
@@ -425,7 +425,6 @@ struct D1Ctx {
   CritLists L;
   const uint8_t* d0_killed;
   const uint32_t* d0mask;
-  const float* f;
   int chain;  // visits one thread makes per round along single-target updates
 };
 
@@ -1355,8 +1354,8 @@ void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st) {
 }
 
 void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1, int n2, const uint32_t* rank,
-                     const uint32_t* order, const float* f, const Rec* rec, const D1Tab* tab, const uint32_t* c1base,
-                     D1Work& W, PairOut& P, uint32_t* status, cudaStream_t st) {
+                     const uint32_t* order, const Rec* rec, const D1Tab* tab, const uint32_t* c1base, D1Work& W,
+                     PairOut& P, uint32_t* status, cudaStream_t st) {
   if (n2 == 0) return;
   D1Ctx c;
   c.d = d;
@@ -1369,7 +1368,6 @@ void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int 
   c.L = L;
   c.d0_killed = P.d0_killed;
   c.d0mask = P.d0mask;
-  c.f = f;
   {
     const int64_t ch = g_morse_chain.load();
     c.chain = ch > 0 ? (int)std::min<int64_t>(ch, 8) : (n2 >= kLargeD1 ? kChainLarge : kChainSmall);

@@ -559,8 +559,8 @@ int compute_diagram(tsf_field* F, bool incremental) {
     launch_d1_prepare(F->n2, F->W, F->PO, st);
     stage_end(F, kD1);
     stage_begin(F, kD1Morse);
-    launch_d1_morse(F->d, F->nd, F->L, F->n1, F->n2, F->rank, F->order, F->f, F->rec, F->tab, F->c1base, F->W,
-                    F->PO, F->status, st);
+    launch_d1_morse(F->d, F->nd, F->L, F->n1, F->n2, F->rank, F->order, F->rec, F->tab, F->c1base, F->W, F->PO,
+                    F->status, st);
     stage_end(F, kD1Morse);
     stage_begin(F, kD1Reduce);
     launch_d1_reduce(F->n1, F->n2, F->W, F->PO, F->status, F->d1ctl, st);

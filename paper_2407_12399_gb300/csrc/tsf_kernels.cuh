@@ -118,11 +118,10 @@ struct D1Ctl {
   unsigned bar[2];  // grid barrier: arrivals, generation
   int n[2];         // lengths of the two column lists
   int which;        // list holding the active columns
-  int rounds;       // rounds done
   int next;         // columns that warps have taken
   int nheavy;       // columns moved to blocks (D1Work::heavy)
   int next_heavy;   // ... taken by blocks
-  int pad[7];
+  int pad[8];
 };
 
 // Counters of the D1 stages (D1Work::stats): [0] lower stars visited, [1]
@@ -161,8 +160,8 @@ int d1_sms();  // of the current device
 // reduction; grids are sized by n2, the kernels read the column count.
 void launch_d1_prepare(int n2, D1Work& W, PairOut& P, cudaStream_t st);
 void launch_d1_morse(const Dims& d, const NbrDelta& nd, const CritLists& L, int n1, int n2, const uint32_t* rank,
-                     const uint32_t* order, const float* f, const Rec* rec, const D1Tab* tab, const uint32_t* c1base,
-                     D1Work& W, PairOut& P, uint32_t* status, cudaStream_t st);
+                     const uint32_t* order, const Rec* rec, const D1Tab* tab, const uint32_t* c1base, D1Work& W,
+                     PairOut& P, uint32_t* status, cudaStream_t st);
 // Words of D1Work::hbits that a reduction over n1 rows uses.
 size_t d1_long_words(int n1);
 void launch_d1_reduce(int n1, int n2, D1Work& W, PairOut& P, uint32_t* status, D1Ctl* ctl, cudaStream_t st);
