@@ -865,10 +865,10 @@ __global__ void __launch_bounds__(kLT, 1) k_d1_long(D1Work W, int n1, D1Ctl* ctl
 __global__ void k_d1_edges(int n1, D1Work W, int32_t* d1_edge, uint32_t* status) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) W.stats[10] += W.stats[14] + W.stats[15];
-  if (i >= n1 || d1_failed(status)) return;
-  const uint32_t j = W.orec[i].x;
-  if (j == kNoOwner) return;
-  if (j < (uint32_t)W.flags[1]) d1_edge[W.cols[j]] = i;
+  if (i >= n1) return;
+  const uint32_t j = W.orec[i].x, ncols = (uint32_t)W.flags[1];
+  if (j == kNoOwner || d1_failed(status)) return;
+  if (j < ncols) d1_edge[W.cols[j]] = i;
   else atomicOr(status, kErrInconsistent);
 }
 

@@ -2558,9 +2558,10 @@ void loss_and_counts(int np, const Pt* pts, int nt, const Tg* T, float cancel_ep
 // gradient step (Section 4.1)
 // ---------------------------------------------------------------------------
 __global__ void k_contrib(int np, const Pt* __restrict__ pts, const Tg* __restrict__ T, float alpha_b, float alpha_d,
-                          Contrib* __restrict__ C, int* __restrict__ count) {
+                          Contrib* __restrict__ C, int* __restrict__ count, uint32_t* __restrict__ status) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
+  if (i == 0) *status = 0u;  // the step's own from here on
   const Pt& p = pts[i];
   float tb, td;
   if (p.tgt >= 0) {
@@ -2608,9 +2609,9 @@ __global__ void k_apply_step(int nc, const int* __restrict__ nc_dev, const int32
                              unsigned long long* __restrict__ nupd, const uint32_t* __restrict__ status) {
   int r = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t s = *status;
+  if (nc_dev) nc = min(*nc_dev, nc);
   if (r == 0) nupd[1] = s;
   if (s & kErrSpin) return;  // a sort that gave up leaves no usable indices
-  if (nc_dev) nc = min(*nc_dev, nc);
   if (r >= nc) return;
   uint32_t v = C[idx[r]].v;
   if (r > 0 && C[idx[r - 1]].v == v) return;
@@ -2628,11 +2629,11 @@ __global__ void k_apply_step(int nc, const int* __restrict__ nc_dev, const int32
 int64_t gradient_step(int np, const Pt* pts, const Tg* T, float alpha_b, float alpha_d, float* f, uint32_t* upd,
                       SolverBufs& B, uint32_t* status, uint32_t* h_status, cudaStream_t st) {
   *h_status = 0;
-  cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
   cudaMemsetAsync(B.count, 0, sizeof(int), st);
   cudaMemsetAsync(B.counters, 0, sizeof(unsigned long long), st);
   if (np == 0) return 0;
-  k_contrib<<<(np + 255) / 256, 256, 0, st>>>(np, pts, T, alpha_b, alpha_d, B.contrib, B.count); note_launch();
+  k_contrib<<<(np + 255) / 256, 256, 0, st>>>(np, pts, T, alpha_b, alpha_d, B.contrib, B.count, status);
+  note_launch();
   // at most two contributions per point: sized by 2 np, counted on the device
   int32_t* idx = 2 * np <= B.cap_rsort
                      ? radix_sort64(2 * np, B.count, ContribBits{B.contrib}, B.rsort, B.idxB, B.idxA, status, st)
