@@ -32,3 +32,21 @@ def test_first_crowded_matching_is_complete():
         assert np.array_equal(d[key][own], t[key][matched])
     moved = np.unique(np.concatenate([d["v_birth"][tgt < 0], d["v_death"][tgt < 0]]))
     assert np.count_nonzero(grad) <= len(moved)
+
+
+def test_crowded_auction_is_within_its_precision_of_the_exact_matching():
+    """The same step from the same values, every point matched anew: the auction's
+    distance (the square root of the loss) within 1 % of the exact one, and on its
+    first call, before any buffer has grown."""
+    f = S.random_field((28, 28, 28), seed=2, kind="uniform")
+    loss = {}
+    for precision in (0.01, 0.0):
+        fld = gpu_field(f)
+        fld.set_threshold(0.3)
+        loss[precision] = fld.step(stop_s=0.0, fast_assignment_update=0, assignment_precision=precision)["loss"]
+        tgt, still = fld.assignment()
+        assert not still.any()
+        matched = tgt[tgt >= 0]
+        assert len(np.unique(matched)) == len(matched) > 1024
+    assert loss[0.0] <= loss[0.01] * (1 + 1e-12)
+    assert np.sqrt(loss[0.01]) <= 1.01 * np.sqrt(loss[0.0])
