@@ -23,7 +23,6 @@
 #include <atomic>
 #include <cstdint>
 
-#include "tsf_kernels.cuh"
 #include "tsf_unet.cuh"
 
 namespace tsf {
@@ -1083,14 +1082,15 @@ int encode_planes_map(CUtensorMap* map, const void* base, int lx, int ly, int lz
 // tile's tz + 2 planes feed one, two or three output planes each; loads and
 // epilogue run beside the MMAs, and a change of tiles costs about 1200.  Small
 // grids take smaller tiles so that every SM has one.
-ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
+ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout, int sms) {
   ConvPlan best{};
   double best_time = 0.0;
   const bool single = chunks == 1;
   const int ksteps = chunks / 2, taps = single ? 14 : 9;
   const int b_bytes = single ? 2 * cout * 16 : ksteps * 2 * 3 * cout * 16;  // weights of a tap (of a pair of taps)
   const int room = static_cast<int>(kConvSmem) - kConvSmemFixed;
-  const int min_x = (lx + kConvTx - 1) / kConvTx, sms = tsf::d1_sms();
+  const int min_x = (lx + kConvTx - 1) / kConvTx;
+  const unsigned usms = static_cast<unsigned>(sms);
   for (int tiles_x = min_x; tiles_x <= min_x + 3; ++tiles_x) {
     const int tx = (lx + tiles_x - 1) / tiles_x, pitch = tx + 2;
     for (int tz = 1; tz <= 16; ++tz) {
@@ -1135,8 +1135,8 @@ ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout) {
         mma = std::max(mma * p.mtiles, groups * (72.0 + 49.0 * ((p.mtiles + 1) / 2)));
         const double loads = (tz + 2) * (p.a_tx + (p.b_resident ? 0.0 : static_cast<double>(taps) * b_bytes)) / 30.0;
         const double epilogue = 120.0 * p.mtiles * tz * (cout / 16);
-        const int64_t tiles = static_cast<int64_t>(tiles_x) * tiles_y * p.tiles_z;
-        const double time = static_cast<double>((tiles + sms - 1) / sms) *
+        const unsigned tiles = static_cast<unsigned>(tiles_x * tiles_y * p.tiles_z);  // a 32-bit division each
+        const double time = static_cast<double>((tiles + usms - 1) / usms) *
                                 std::max(std::max(mma + 1200.0, loads), epilogue) + std::min(mma, loads) / 2 + epilogue;
         if (best.tx == 0 || time < best_time) {
           best = p;
@@ -1160,7 +1160,7 @@ int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaSt
                         : in_chunks == 12 ? k_conv_tc<6>
                                           : nullptr;
   if (!kernel || a.cout % 16 != 0 || a.cout > 96 || (a.cout > 85 && in_chunks != 4)) return -1;
-  a.plan = plan_conv(a.lx, a.ly, a.lz, in_chunks, a.cout);
+  a.plan = plan_conv(a.lx, a.ly, a.lz, in_chunks, a.cout, a.sms);
   const ConvPlan& p = a.plan;
   if (p.tx == 0) return -3;
   CUtensorMap map;
@@ -1175,7 +1175,7 @@ int launch_conv(const ConvArgs& a0, const void* in_planes, int in_chunks, cudaSt
   }
   const size_t smem = static_cast<size_t>(kConvSmemFixed) + static_cast<size_t>(p.stages) * p.a_bytes +
                       static_cast<size_t>(p.b_slots) * p.b_bytes;
-  kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, tsf::d1_sms()), kConvThreads, smem, st>>>(map, a);
+  kernel<<<std::min(p.tiles_x * p.tiles_y * p.tiles_z, a.sms), kConvThreads, smem, st>>>(map, a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
 
@@ -1205,16 +1205,17 @@ void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void*
       planes, lx, ly, lz, static_cast<uint4*>(out));
 }
 
-int head_blocks(int64_t nv) { return static_cast<int>(std::min<int64_t>((nv + 255) / 256, tsf::d1_sms())); }
+int head_blocks(int64_t nv, int sms) { return static_cast<int>(std::min<int64_t>((nv + 255) / 256, sms)); }
 
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
-                          double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st) {
-  const int nb = head_blocks(nv);
+                          double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, int sms,
+                          cudaStream_t st) {
+  const int nb = head_blocks(nv, sms);
   k_head_backward<<<nb, 256, 0, st>>>(static_cast<const uint4*>(u1), hw, nv, f, g, static_cast<uint4*>(gz), partial);
   k_head_reduce<<<1, 18 * 32, 0, st>>>(partial, nb, nv, loss, grad, hw_off, hb_off);
 }
 
-WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout) {
+WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout, int sms) {
   WgradPlan p{};
   p.lz = lz;
   p.cout_chunks = cout / 8;
@@ -1231,7 +1232,7 @@ WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout) {
   // rows per step: four stages in shared memory, and four steps for every
   // block (each block's partial is written and read once more)
   const int row_bytes = 16 * (3 * p.cin_chunks * p.pitch + p.copies * p.cout_chunks * p.tx);
-  int blocks = std::max(tsf::d1_sms() / p.groups, 1);
+  int blocks = std::max(sms / p.groups, 1);
   const int by_smem = std::max(static_cast<int>(kWgSmem / kWgStagesMax) / row_bytes, 1);
   const int by_steps = std::max(static_cast<int>(static_cast<int64_t>(ly) * lz * p.tiles_x / (4 * blocks)), 1);
   p.ty = std::min(std::min(by_smem, by_steps), std::min(ly, 256));
@@ -1247,17 +1248,18 @@ WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout) {
   return p;
 }
 
-int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout) {
-  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout).blocks) * 27 * cin * cout;
+int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout, int sms) {
+  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout, sms).blocks) * 27 * cin * cout;
 }
 
-int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout) {
-  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout).blocks) * cout;
+int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout, int sms) {
+  return static_cast<int64_t>(plan_wgrad(lx, ly, lz, cin, cout, sms).blocks) * cout;
 }
 
 int launch_wgrad(const void* x, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
-                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, cudaStream_t st) {
-  const WgradPlan p = plan_wgrad(lx, ly, lz, cin, cout);
+                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, int sms,
+                 cudaStream_t st) {
+  const WgradPlan p = plan_wgrad(lx, ly, lz, cin, cout, sms);
   if (p.stages < 1 || cout % 16 != 0 || cout > 64 || cin > 96) return -1;
   CUtensorMap xm, gm;
   if (encode_planes_map(&xm, x, lx, ly, lz, cin / 8, p.pitch, p.ty, 3, p.cin_chunks) != 0 ||

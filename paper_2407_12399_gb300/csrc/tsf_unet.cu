@@ -62,7 +62,7 @@ void dfree(T*& p) {
 }  // namespace
 
 struct tsf_unet {
-  int device = 0;
+  int device = 0, sms = 0;
   cudaStream_t st = nullptr;
   uint32_t* status = nullptr;
   float *params = nullptr, *rounded = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
@@ -149,12 +149,12 @@ int ensure_grid(tsf_unet* U, int lx, int ly, int lz, bool train) {
     const int level[NCONV] = {1, 1, 2, 2, 4, 4, 2, 2, 1, 1};
     for (int i = 0; i < NCONV; ++i) {
       const int k = level[i], cin = kNet.L[i].cin_pad, cout = kNet.L[i].cout;
-      wp = std::max(wp, wgrad_partial_floats(lx / k, ly / k, lz / k, cin, cout));
-      bp = std::max(bp, bias_partial_floats(lx / k, ly / k, lz / k, cin, cout));
+      wp = std::max(wp, wgrad_partial_floats(lx / k, ly / k, lz / k, cin, cout, U->sms));
+      bp = std::max(bp, bias_partial_floats(lx / k, ly / k, lz / k, cin, cout, U->sms));
     }
     if (e == cudaSuccess) e = dalloc(&U->wpart, wp);
     if (e == cudaSuccess) e = dalloc(&U->bpart, bp);
-    if (e == cudaSuccess) e = dalloc(&U->hpart, (int64_t)head_blocks(n1) * 18);
+    if (e == cudaSuccess) e = dalloc(&U->hpart, (int64_t)head_blocks(n1, U->sms) * 18);
   }
   if (e != cudaSuccess) {
     free_grid(U);
@@ -191,6 +191,7 @@ int conv(tsf_unet* U, int layer, int mode, const uint4* in, int in_chunks, int l
   a.mask = mask;
   a.mask_plane0 = mask_plane0;
   a.status = U->status;
+  a.sms = U->sms;
   a.head = U->rounded + kNet.head_w;
   a.f = U->fbuf;
   a.g0 = U->g0;
@@ -240,7 +241,7 @@ int wgrad(tsf_unet* U, int layer, const uint4* x, const uint4* gz, int lx, int l
   const Layer& l = kNet.L[layer];
   tsf::note_launch();
   return launch_wgrad(x, l.cin_pad, l.cin_real, gz, l.cout, lx, ly, lz, U->wpart, U->grad + l.w_off, U->bpart,
-                      U->grad + l.b_off, U->status, U->st) == 0
+                      U->grad + l.b_off, U->status, U->sms, U->st) == 0
              ? TSF_OK
              : TSF_ECUDA;
 }
@@ -262,7 +263,7 @@ int backward(tsf_unet* U, float* keep) {
   };
   int r = TSF_OK;
   launch_head_backward(U->u1, U->rounded + kNet.head_w, n1, U->fbuf, U->gbuf, U->gzA1, U->hpart, U->loss, U->grad,
-                       kNet.head_w, kNet.head_b, st);
+                       kNet.head_w, kNet.head_b, U->sms, st);
   put(U->gzA1, 16, n1);
   if (!r) r = wgrad(U, D1B, U->a1d, U->gzA1, lx, ly, lz);
   if (!r) r = conv(U, D1B, kConvDgrad, U->gzA1, 2, lx, ly, lz, U->gzB1, 0, 0, U->a1d, 0);
@@ -334,6 +335,7 @@ int tsf_unet_create(const float* params, int64_t n, void* cuda_stream, tsf_unet*
   *out = nullptr;
   tsf_unet* U = new tsf_unet();
   cudaGetDevice(&U->device);
+  U->sms = tsf::d1_sms();
   U->st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = dalloc(&U->status, 1);
   if (e == cudaSuccess) e = dalloc(&U->params, n);

@@ -49,10 +49,11 @@ struct ConvArgs {
   const float* f;
   float* g0;
   uint32_t* status;   // device status word (kUnetErrSpin)
+  int sms;            // of the device
   ConvPlan plan;
 };
 
-ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout);
+ConvPlan plan_conv(int lx, int ly, int lz, int chunks, int cout, int sms);
 int launch_conv(const ConvArgs& a, const void* in_planes, int in_chunks, cudaStream_t st);
 
 void launch_pack_input(const float* f, float tau, int64_t nv, void* x, cudaStream_t st);
@@ -61,9 +62,10 @@ void launch_upsample_back(const void* g, int g_plane0, int planes, int lx, int l
                           int act_plane0, void* out, cudaStream_t st);
 void launch_skip_back(const void* gs, int gs_plane0, const void* gp, const void* s, int s_plane0, int planes, int lx,
                       int ly, int lz, void* out, cudaStream_t st);
-int head_blocks(int64_t nv);
+int head_blocks(int64_t nv, int sms);
 void launch_head_backward(const void* u1, const float* hw, int64_t nv, const float* f, const float* g, void* gz,
-                          double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, cudaStream_t st);
+                          double* partial, double* loss, float* grad, int64_t hw_off, int64_t hb_off, int sms,
+                          cudaStream_t st);
 // Weight gradient of one convolution (k_wgrad_tc): tile, operand blocks and
 // grid (blocks x groups).
 struct WgradPlan {
@@ -75,11 +77,12 @@ struct WgradPlan {
 };
 constexpr int kWgTx = 112;                // voxels of a step along x, at most
 constexpr size_t kWgSmem = 208 * 1024;    // stages of a block
-WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout);
-int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout);
-int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout);
+WgradPlan plan_wgrad(int lx, int ly, int lz, int cin, int cout, int sms);
+int64_t wgrad_partial_floats(int lx, int ly, int lz, int cin, int cout, int sms);
+int64_t bias_partial_floats(int lx, int ly, int lz, int cin, int cout, int sms);
 int launch_wgrad(const void* x, int cin, int cin_real, const void* gz, int cout, int lx, int ly, int lz,
-                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, cudaStream_t st);
+                 float* partial, float* gw, float* bpartial, float* gb, uint32_t* status, int sms,
+                 cudaStream_t st);
 void launch_pack_weights(const float* w, int cout_f, int cin_real, int cin_pad, int transpose, void* pack,
                          cudaStream_t st);
 int64_t pack_elems(int cout_f, int cin_pad, int transpose);
